@@ -134,14 +134,7 @@ void count_launches(int n) { g_launches.fetch_add((uint64_t)n, std::memory_order
 WsLayout plan_workspace(const Shape& s) {
   WsLayout L{};
   const size_t U = (size_t)s.U, m = (size_t)s.m, d = (size_t)kD;
-  // portable scoring: chunks of a multiple of 64 keys, enough of them that
-  // U x chunks fills the GPU a few times over (608 CTAs) without splitting a
-  // unit into chunks of fewer than 64 keys
-  {
-    const int per_unit = std::max(1, std::min((608 + std::max(s.U, 1) - 1) / std::max(s.U, 1),
-                                              (s.n + 63) / 64));
-    L.chunk = std::max(64, ((s.n + per_unit - 1) / per_unit + 63) / 64 * 64);
-  }
+  L.chunk = score_simt_chunk(s);
   L.nchunk = (s.n + L.chunk - 1) / L.chunk;
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -169,6 +162,7 @@ WsLayout plan_workspace(const Shape& s) {
     L.flags = take(U * (size_t)s.B);
     L.gram = take(U * m * m * 8);
     L.rz = take(U * m * d * 8);
+    L.state = take(U * sizeof(int));
   }
   L.scores = take(U * (size_t)s.P * 4);
   L.y = take(U * m * d * 4);

@@ -58,6 +58,7 @@ struct WsLayout {
   size_t flags;   // uint8 [U][B]      fixed-token flags
   size_t gram;    // acc   [U][m][m]   X_G X_G^T + lambda I, then its Cholesky factor
   size_t rz;      // acc   [U][m][d]   residual R, then Z
+  size_t state;   // int   [U]         outcome of the unit's solve
   size_t merge_tc;  // tensor-core merge: R/Z, Gram [U][128][128] fp32, normalisers, positions, fixed flags
   // compress intermediates
   size_t scores;  // float [U][P]
@@ -89,6 +90,7 @@ void count_launches(int n);
 cudaError_t launch_score_simt(const Shape& s, const void* q, const void* k, const void* v,
                               float* scores, float* y, float* row_stats, char* ws,
                               const WsLayout& L, cudaStream_t st);
+int score_simt_chunk(const Shape& s);   // keys per CTA of the portable scoring
 cudaError_t launch_select(const Shape& s, const float* scores, int32_t* idx, char* ws,
                           const WsLayout& L, cudaStream_t st);
 // Tensor-core window scoring (bf16, m <= 256 in blocks of 128 rows).  The

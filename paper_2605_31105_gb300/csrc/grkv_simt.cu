@@ -1,198 +1,292 @@
-// Portable CUDA-core kernels of the GRKV compression path.
+// Window scoring on CUDA cores (fp32 inputs, and bf16 under GRKV_FORCE_SIMT),
+// and the selection kernels of every path.
 //
-// These run for fp32 inputs, and for bf16 when GRKV_FORCE_SIMT is set.  They
-// favour plain, checkable arithmetic over speed: every logit is an fp32 FMA
-// chain over the head dimension, probabilities use expf and an IEEE divide,
-// and every reduction runs in a fixed order, so results are deterministic.
-// The value-step solve accumulates in double for fp32 inputs.
-#include <cfloat>
+// Every logit is an fp32 FMA chain over the head dimension, probabilities use
+// expf and an IEEE divide, and every reduction runs in a fixed order, so
+// results are deterministic.
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 
 #include "block_select.cuh"
-#include "grkv_internal.cuh"
+#include "simt_common.cuh"
 
 namespace grkv {
 namespace {
 
-constexpr int QP = kD + 1;  // padded row stride (floats) of q / key tiles in shared memory
+// ------------------------------------------------------------ logits tile --
+// Both passes form S = Q K^T in tiles of MR window rows x 64 keys: 256 threads
+// as 16 x 16, thread (ty, tx) rows ty MR/16 .. and keys tx, tx + 16, ...  The
+// operands stay [row][t] in shared memory with rows of 132 floats, read four t
+// at a time: with MR = 128, 12 16-byte loads feed 128 FMAs and the tile is
+// bound by the FMAs (one load per FMA, one output per thread and 64-key
+// chunks cut into 512 CTAs took 355 + 603 us for 8 units of n = 8192, m = 128).
+constexpr int kKeys = 64;        // keys per tile
+constexpr int kSLD = kD + 4;     // row stride of staged operands
+constexpr int kScT = 256;
 
-// Float count rounded up to a multiple of 4, so the next shared-memory region
-// starts on a 16-byte boundary.
-__host__ __device__ constexpr int pad4(int n) { return (n + 3) & ~3; }
-
-__device__ __forceinline__ float ldv(const float* p, size_t i) { return p[i]; }
-__device__ __forceinline__ float ldv(const __nv_bfloat16* p, size_t i) {
-  return __bfloat162float(p[i]);
+// rows x 128 values into shared memory as fp32, rows of `ld` floats; rows past
+// `valid` become zeros.  fp32 rows go by cp.async (committed by the caller).
+template <typename T>
+__device__ __forceinline__ void stage_rows(float* dst, int ld, const T* src, int rows, int valid) {
+  for (int i = threadIdx.x; i < rows * (kD / 4); i += kScT) {
+    const int r = i / (kD / 4), t = i % (kD / 4) * 4;
+    float* d = dst + r * ld + t;
+    const size_t o = (size_t)r * kD + t;
+    if (r >= valid) {
+      *(float4*)d = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else if constexpr (std::is_same<T, float>::value) {
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                       (uint32_t)__cvta_generic_to_shared(d)),
+                   "l"(src + o));
+    } else {
+      const uint2 w = *(const uint2*)(src + o);
+      *(float4*)d = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u),
+                                __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xFFFF0000u));
+    }
+  }
 }
-__device__ __forceinline__ void stv(float* p, size_t i, double x) { p[i] = (float)x; }
-__device__ __forceinline__ void stv(__nv_bfloat16* p, size_t i, float x) {
-  p[i] = __float2bfloat16_rn(x);
+__device__ __forceinline__ void stage_commit() { asm volatile("cp.async.commit_group;"); }
+template <int kPending>
+__device__ __forceinline__ void stage_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory");
 }
 
-// Window slot a = r mod w sits at position n - w + a and sees keys j <= n - w + a.
-__device__ __forceinline__ bool visible(const Shape& s, int r, int j) {
-  return !s.causal || j <= s.n - s.w + (r % s.w);
+template <int RT>
+__device__ __forceinline__ void logits_tile(const float* qs, const float* ks, float (*acc)[4]) {
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+  for (int i = 0; i < RT; ++i)
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj) acc[i][jj] = 0.f;
+#pragma unroll 2
+  for (int t = 0; t < kD; t += 4) {
+    float4 qv[RT], kv[4];
+#pragma unroll
+    for (int i = 0; i < RT; ++i) qv[i] = *(const float4*)(qs + (ty * RT + i) * kSLD + t);
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj) kv[jj] = *(const float4*)(ks + (tx + 16 * jj) * kSLD + t);
+#pragma unroll
+    for (int i = 0; i < RT; ++i)
+#pragma unroll
+      for (int jj = 0; jj < 4; ++jj) {
+        float c = acc[i][jj];
+        c = fmaf(qv[i].x, kv[jj].x, c);
+        c = fmaf(qv[i].y, kv[jj].y, c);
+        c = fmaf(qv[i].z, kv[jj].z, c);
+        acc[i][jj] = fmaf(qv[i].w, kv[jj].w, c);
+      }
+  }
+}
+
+// Merges two (max, sum of exp(l - max)) row statistics.
+__device__ __forceinline__ float2 stat_merge(float2 x, float2 y) {
+  if (y.x == -INFINITY) return x;
+  if (y.x > x.x) return make_float2(y.x, x.y * expf(x.x - y.x) + y.y);
+  return make_float2(x.x, x.y + y.y * expf(y.x - x.x));
+}
+
+template <int RT>
+constexpr size_t stats_smem() {
+  return (size_t)(16 * RT + 2 * kKeys) * kSLD * 4;
+}
+template <int RT>
+constexpr size_t prob_smem() {
+  // Q, two K tiles (the one in use becomes P), two V tiles, row statistics, column sums
+  return ((size_t)(16 * RT + 2 * kKeys) * kSLD + 2 * kKeys * kD + 2 * 16 * RT + 16 * kKeys) * 4;
 }
 
 // ---------------------------------------------------------------- pass A --
 // Row statistics of one chunk of keys: (max_j l_rj, sum_j exp(l_rj - max)).
-template <typename T>
-__global__ void __launch_bounds__(256) k_stats_chunk(const T* __restrict__ q,
-                                                     const T* __restrict__ k, Shape s, int chunk,
-                                                     int nchunk, float2* __restrict__ pstats) {
+template <typename T, int RT>
+__global__ void __launch_bounds__(kScT, RT == 8 ? 1 : 2)
+    k_stats_chunk(const T* __restrict__ q, const T* __restrict__ k, Shape s, int chunk, int nchunk,
+                  float2* __restrict__ pstats) {
   extern __shared__ __align__(16) float sm[];
-  float* qs = sm;                          // [m][QP], padded to 16 bytes
-  float* ks = qs + pad4(s.m * QP);         // [64][kD]
-  float2* red = (float2*)(ks + 64 * kD);   // [256], 8-byte aligned
-  const int u = blockIdx.y, c = blockIdx.x, tid = threadIdx.x;
+  constexpr int MR = 16 * RT;
+  float* qs = sm;                   // [MR][kSLD]
+  float* ks = qs + MR * kSLD;       // two tiles of [kKeys][kSLD]
+  const int u = blockIdx.y, c = blockIdx.x;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const int j0 = c * chunk, j1 = min(s.n, j0 + chunk);
-  const T* qu = q + (size_t)u * s.m * kD;
   const T* ku = k + (size_t)u * s.n * kD;
-  for (int i = tid; i < s.m * kD; i += blockDim.x) qs[(i / kD) * QP + i % kD] = ldv(qu, i);
-  const int tpr = max(1, (int)blockDim.x / s.m);
-  const int r = tid / tpr, sub = tid % tpr;
-  const bool active = r < s.m;
-  float M = -INFINITY, L = 0.f;
-  for (int base = j0; base < j1; base += 64) {
-    const int len = min(64, j1 - base);
+  for (int row0 = 0; row0 < s.m; row0 += MR) {
     __syncthreads();
-    for (int i = tid; i < len * kD; i += blockDim.x) ks[i] = ldv(ku, (size_t)base * kD + i);
-    __syncthreads();
-    if (!active) continue;
-    for (int jj = sub; jj < len; jj += tpr) {
-      const int j = base + jj;
-      if (!visible(s, r, j)) continue;
-      float acc = 0.f;
-#pragma unroll 8
-      for (int t = 0; t < kD; ++t) acc = fmaf(qs[r * QP + t], ks[jj * kD + t], acc);
-      const float l = s.scale * acc;
-      if (l > M) {
-        L = L * expf(M - l) + 1.f;
-        M = l;
-      } else {
-        L += expf(l - M);
+    stage_rows(qs, kSLD, q + ((size_t)u * s.m + row0) * kD, MR, s.m - row0);
+    stage_rows(ks, kSLD, ku + (size_t)j0 * kD, kKeys, j1 - j0);
+    stage_commit();
+    float2 st[RT];
+#pragma unroll
+    for (int i = 0; i < RT; ++i) st[i] = make_float2(-INFINITY, 0.f);
+    for (int base = j0, b = 0; base < j1; base += kKeys, b ^= 1) {
+      if (base + kKeys < j1)
+        stage_rows(ks + (b ^ 1) * kKeys * kSLD, kSLD, ku + (size_t)(base + kKeys) * kD, kKeys,
+                   j1 - base - kKeys);
+      stage_commit();
+      stage_wait<1>();
+      __syncthreads();
+      float acc[RT][4];
+      logits_tile<RT>(qs, ks + b * kKeys * kSLD, acc);
+#pragma unroll
+      for (int i = 0; i < RT; ++i) {
+        const int r = row0 + ty * RT + i;
+        float l[4], mx = -INFINITY;
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {
+          const int j = base + tx + 16 * jj;
+          l[jj] = (j < j1 && visible(s, r, j)) ? s.scale * acc[i][jj] : -INFINITY;
+          mx = fmaxf(mx, l[jj]);
+        }
+        if (mx == -INFINITY) continue;
+        if (mx > st[i].x) {
+          st[i].y *= expf(st[i].x - mx);
+          st[i].x = mx;
+        }
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) st[i].y += expf(l[jj] - st[i].x);
       }
+      __syncthreads();   // the other buffer is refilled next
     }
-  }
-  red[tid] = make_float2(M, L);
-  __syncthreads();
-  if (active && sub == 0) {
-    float Mr = -INFINITY, Lr = 0.f;
-    for (int t = 0; t < tpr; ++t) {
-      const float2 pr = red[r * tpr + t];
-      if (pr.x == -INFINITY) continue;
-      if (pr.x > Mr) {
-        Lr = Lr * expf(Mr - pr.x) + pr.y;
-        Mr = pr.x;
-      } else {
-        Lr += pr.y * expf(pr.x - Mr);
+    // a row's 16 threads are half a warp
+#pragma unroll
+    for (int i = 0; i < RT; ++i) {
+#pragma unroll
+      for (int o = 1; o < 16; o <<= 1) {
+        const float2 y = make_float2(__shfl_xor_sync(0xffffffffu, st[i].x, o),
+                                     __shfl_xor_sync(0xffffffffu, st[i].y, o));
+        st[i] = stat_merge(st[i], y);
       }
+      const int r = row0 + ty * RT + i;
+      if (tx == 0 && r < s.m) pstats[((size_t)u * nchunk + c) * s.m + r] = st[i];
     }
-    pstats[((size_t)u * nchunk + c) * s.m + r] = make_float2(Mr, Lr);
-  }
-}
-
-__global__ void k_stats_reduce(const float2* __restrict__ pstats, Shape s, int nchunk,
-                               float* __restrict__ row_stats) {
-  const int u = blockIdx.x;
-  for (int r = threadIdx.x; r < s.m; r += blockDim.x) {
-    float M = -INFINITY, L = 0.f;
-    for (int c = 0; c < nchunk; ++c) {
-      const float2 pr = pstats[((size_t)u * nchunk + c) * s.m + r];
-      if (pr.x == -INFINITY) continue;
-      if (pr.x > M) {
-        L = L * expf(M - pr.x) + pr.y;
-        M = pr.x;
-      } else {
-        L += pr.y * expf(pr.x - M);
-      }
-    }
-    row_stats[((size_t)u * s.m + r) * 2 + 0] = M;
-    row_stats[((size_t)u * s.m + r) * 2 + 1] = L;
   }
 }
 
 // ---------------------------------------------------------------- pass B --
-// Probabilities of one chunk: prefix scores (column sums over the m rows, in
-// row order) and the chunk's share of Y = P V.
-template <typename T, int RPT>
-__global__ void __launch_bounds__(512) k_prob_chunk(const T* __restrict__ q,
-                                                    const T* __restrict__ k,
-                                                    const T* __restrict__ v, Shape s, int chunk,
-                                                    int nchunk, const float* __restrict__ row_stats,
-                                                    float* __restrict__ scores,
-                                                    float* __restrict__ ypart) {
+// Probabilities of one chunk: prefix scores (column sums over the m rows) and
+// the chunk's share of Y = P V.  Each CTA combines the unit's row statistics
+// itself; the first chunk's also writes them out.
+template <typename T, int RT>
+__global__ void __launch_bounds__(kScT, 1)
+    k_prob_chunk(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, Shape s,
+                 int chunk, int nchunk, const float2* __restrict__ pstats,
+                 float* __restrict__ row_stats, float* __restrict__ scores,
+                 float* __restrict__ ypart) {
   extern __shared__ __align__(16) float sm[];
-  float* qs = sm;                 // [m][QP]
-  float* ks = qs + s.m * QP;      // [32][QP]
-  float* vs = ks + 32 * QP;       // [32][kD]
-  float* ps = vs + 32 * kD;       // [m][33]
-  float* st = ps + s.m * 33;      // [m][2]  (M_r, L_r)
+  constexpr int MR = 16 * RT;
+  float* qs = sm;                            // [MR][kSLD]
+  float* ks = qs + MR * kSLD;                // two tiles of [kKeys][kSLD]; then P [key][row]
+  float* vs = ks + 2 * kKeys * kSLD;         // two tiles of [kKeys][kD]
+  float2* st = (float2*)(vs + 2 * kKeys * kD);   // [MR] (M_r, L_r)
+  float* cs = (float*)(st + MR);             // [16][kKeys] column sums of each ty
   const int u = blockIdx.y, c = blockIdx.x, tid = threadIdx.x;
+  const int tx = tid & 15, ty = tid >> 4;
   const int j0 = c * chunk, j1 = min(s.n, j0 + chunk);
-  const T* qu = q + (size_t)u * s.m * kD;
   const T* ku = k + (size_t)u * s.n * kD;
   const T* vu = v + (size_t)u * s.n * kD;
-  for (int i = tid; i < s.m * kD; i += blockDim.x) qs[(i / kD) * QP + i % kD] = ldv(qu, i);
-  for (int i = tid; i < s.m * 2; i += blockDim.x) st[i] = row_stats[(size_t)u * s.m * 2 + i];
-  const int e = tid & (kD - 1), rq = tid >> 7;  // 4 row phases of 128 columns
-  float acc[RPT];
-#pragma unroll
-  for (int i = 0; i < RPT; ++i) acc[i] = 0.f;
-  for (int base = j0; base < j1; base += 32) {
-    const int len = min(32, j1 - base);
+  for (int row0 = 0; row0 < s.m; row0 += MR) {
     __syncthreads();
-    for (int i = tid; i < 32 * kD; i += blockDim.x) {
-      const int jj = i / kD, t = i % kD;
-      const bool in = jj < len;
-      ks[jj * QP + t] = in ? ldv(ku, (size_t)(base + jj) * kD + t) : 0.f;
-      vs[i] = in ? ldv(vu, (size_t)(base + jj) * kD + t) : 0.f;
-    }
-    __syncthreads();
-    for (int pr = tid; pr < s.m * 32; pr += blockDim.x) {
-      const int r = pr >> 5, jj = pr & 31, j = base + jj;
-      float p = 0.f;
-      if (jj < len && visible(s, r, j)) {
-        float a = 0.f;
+    auto stage_tile = [&](int base, int b) {
+      stage_rows(ks + b * kKeys * kSLD, kSLD, ku + (size_t)base * kD, kKeys, j1 - base);
+      stage_rows(vs + b * kKeys * kD, kD, vu + (size_t)base * kD, kKeys, j1 - base);
+    };
+    stage_rows(qs, kSLD, q + ((size_t)u * s.m + row0) * kD, MR, s.m - row0);
+    stage_tile(j0, 0);
+    stage_commit();
+    for (int r = tid; r < MR; r += kScT) {
+      float2 x = make_float2(-INFINITY, 0.f);
+      if (row0 + r < s.m) {
 #pragma unroll 8
-        for (int t = 0; t < kD; ++t) a = fmaf(qs[r * QP + t], ks[jj * QP + t], a);
-        p = expf(s.scale * a - st[2 * r]) / st[2 * r + 1];
+        for (int h = 0; h < nchunk; ++h)
+          x = stat_merge(x, pstats[((size_t)u * nchunk + h) * s.m + row0 + r]);
+        if (c == 0) *(float2*)(row_stats + ((size_t)u * s.m + row0 + r) * 2) = x;
       }
-      ps[r * 33 + jj] = p;
+      st[r] = x;
     }
-    __syncthreads();
-    if (tid < len && base + tid < s.P) {
-      float cs = 0.f;
-      for (int r = 0; r < s.m; ++r) cs += ps[r * 33 + tid];
-      scores[(size_t)u * s.P + base + tid] = cs;
+    float y[RT][8];
+#pragma unroll
+    for (int i = 0; i < RT; ++i)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) y[i][e] = 0.f;
+    for (int base = j0, b = 0; base < j1; base += kKeys, b ^= 1) {
+      if (base + kKeys < j1) stage_tile(base + kKeys, b ^ 1);
+      stage_commit();
+      stage_wait<1>();
+      __syncthreads();
+      float* kt = ks + b * kKeys * kSLD;
+      float acc[RT][4];
+      logits_tile<RT>(qs, kt, acc);
+      __syncthreads();   // K is used up: its buffer takes P
+      float sum[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int i = 0; i < RT; ++i) {
+        const int r = row0 + ty * RT + i;
+        const float2 ml = st[ty * RT + i];
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {
+          const int j = base + tx + 16 * jj;
+          float p = 0.f;
+          if (r < s.m && j < j1 && visible(s, r, j)) p = expf(s.scale * acc[i][jj] - ml.x) / ml.y;
+          kt[(tx + 16 * jj) * kSLD + ty * RT + i] = p;
+          sum[jj] += p;
+        }
+      }
+#pragma unroll
+      for (int jj = 0; jj < 4; ++jj) cs[ty * kKeys + tx + 16 * jj] = sum[jj];
+      __syncthreads();
+      if (tid < kKeys && base + tid < min(j1, s.P)) {
+        float t = 0.f;
+#pragma unroll
+        for (int g = 0; g < 16; ++g) t += cs[g * kKeys + tid];
+        float* o = scores + (size_t)u * s.P + base + tid;
+        *o = row0 ? *o + t : t;   // the same thread wrote the earlier rows' sum
+      }
+      const float* vt = vs + b * kKeys * kD;
+#pragma unroll 4
+      for (int jj = 0; jj < kKeys; ++jj) {
+        const float4 v0 = *(const float4*)(vt + jj * kD + tx * 4);
+        const float4 v1 = *(const float4*)(vt + jj * kD + 64 + tx * 4);
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+          const float p = kt[jj * kSLD + ty * RT + i];
+          y[i][0] = fmaf(p, v0.x, y[i][0]);
+          y[i][1] = fmaf(p, v0.y, y[i][1]);
+          y[i][2] = fmaf(p, v0.z, y[i][2]);
+          y[i][3] = fmaf(p, v0.w, y[i][3]);
+          y[i][4] = fmaf(p, v1.x, y[i][4]);
+          y[i][5] = fmaf(p, v1.y, y[i][5]);
+          y[i][6] = fmaf(p, v1.z, y[i][6]);
+          y[i][7] = fmaf(p, v1.w, y[i][7]);
+        }
+      }
+      __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-      const int r = rq + 4 * i;
-      if (r < s.m) {
-        float a = acc[i];
-        for (int jj = 0; jj < 32; ++jj) a = fmaf(ps[r * 33 + jj], vs[jj * kD + e], a);
-        acc[i] = a;
-      }
+    for (int i = 0; i < RT; ++i) {
+      const int r = row0 + ty * RT + i;
+      if (r >= s.m) break;
+      float* o = ypart + (((size_t)u * nchunk + c) * s.m + r) * kD + tx * 4;
+      *(float4*)o = make_float4(y[i][0], y[i][1], y[i][2], y[i][3]);
+      *(float4*)(o + 64) = make_float4(y[i][4], y[i][5], y[i][6], y[i][7]);
     }
-  }
-#pragma unroll
-  for (int i = 0; i < RPT; ++i) {
-    const int r = rq + 4 * i;
-    if (r < s.m) ypart[(((size_t)u * nchunk + c) * s.m + r) * kD + e] = acc[i];
   }
 }
 
-__global__ void k_y_reduce(const float* __restrict__ ypart, Shape s, int nchunk,
-                           float* __restrict__ y) {
-  const int u = blockIdx.x;
-  const size_t md = (size_t)s.m * kD;
-  for (size_t i = threadIdx.x; i < md; i += blockDim.x) {
-    float a = 0.f;
-    for (int c = 0; c < nchunk; ++c) a += ypart[((size_t)u * nchunk + c) * md + i];
-    y[(size_t)u * md + i] = a;
+// Y = sum of the chunks' shares, in chunk order; one float4 per thread.
+__global__ void __launch_bounds__(256) k_y_reduce(const float4* __restrict__ ypart, Shape s,
+                                                  int nchunk, float4* __restrict__ y) {
+  const int u = blockIdx.y, md = s.m * (kD / 4), i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= md) return;
+  float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+  for (int c = 0; c < nchunk; ++c) {
+    const float4 x = ypart[((size_t)u * nchunk + c) * md + i];
+    a.x += x.x;
+    a.y += x.y;
+    a.z += x.z;
+    a.w += x.w;
   }
+  y[(size_t)u * md + i] = a;
 }
 
 // ------------------------------------------------------------- selection --
@@ -472,309 +566,36 @@ __global__ void __launch_bounds__(kSelThreads, 1) k_select_smem(const float* __r
   for (int a = tid; a < s.w; a += kSelThreads) out[s.kk + a] = P + a;
 }
 
-// ------------------------------------------------------------------ merge --
-// One CTA per unit.  A is the accumulation type of the regression (double for
-// fp32 inputs, float for bf16).  phase 0 runs the whole value step; phase 1
-// stops once R and N are in the workspace and phase 2 starts from Z there
-// (the fp32 solve between them is k_solve_dense).
-template <typename T, typename A>
-__global__ void __launch_bounds__(512) k_merge(
-    const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
-    const float* __restrict__ scores, const float* __restrict__ y, const int32_t* __restrict__ idx,
-    T* __restrict__ k_out, T* __restrict__ v_out, Shape s, float* __restrict__ xbuf,
-    uint8_t* __restrict__ flags, A* __restrict__ gram, A* __restrict__ rz, int* status,
-    int phase) {
-  extern __shared__ __align__(16) float sm[];
-  __shared__ int hist[256];
-  __shared__ int sh[48];
-  const int u = blockIdx.x, tid = threadIdx.x, m = s.m, B = s.B;
-  const int nthr = blockDim.x;
-  float* qs = sm;               // [m][QP]
-  float* tile = qs + m * QP;    // [32][QP]
-  float* xt = tile + 32 * QP;   // [m][33]
-  const int32_t* id = idx + (size_t)u * B;
-  // retained position of slot i; an entry outside [0, n) is reported and read as 0
-  auto pos = [&](int i) {
-    const int j = id[i];
-    return (unsigned)j < (unsigned)s.n ? j : 0;
-  };
-  float* X = xbuf + (size_t)u * m * B;
-  uint8_t* F = flags + (size_t)u * B;
-  A* N = gram + (size_t)u * m * m;
-  A* RZ = rz + (size_t)u * m * kD;
-  const T* ku = k + (size_t)u * s.n * kD;
-  const T* vu = v + (size_t)u * s.n * kD;
-  T* ko = k_out + (size_t)u * B * kD;
-  T* vo = v_out + (size_t)u * B * kD;
-  const float* yu = y + (size_t)u * m * kD;
-  const float* cu = scores + (size_t)u * s.P;
-  if (phase == 2 && s.lambda_inf) return;   // phase 1 wrote V_out = V0
-  if (phase != 2) {
-  for (int i = tid; i < B; i += nthr)
-    if ((unsigned)id[i] >= (unsigned)s.n) set_status(status, GRKV_ERR_INVALID_ARG);
-
-  for (int i = tid; i < m * kD; i += nthr)
-    qs[(i / kD) * QP + i % kD] = ldv(q + (size_t)u * m * kD, i);
-  // K_out = K0 (the key step is not applied)
-  for (int i = tid; i < B * kD; i += nthr) ko[i] = ku[(size_t)pos(i / kD) * kD + i % kD];
-
-  // Fixed set: retained sinks, the window, and the n_fix best-scored
-  // retained prefix non-sink tokens.
-  auto cand = [&](int i) {
-    const int j = pos(i);
-    return j >= s.n_sink && j < s.P;
-  };
-  int nc = 0;
-  for (int i = tid; i < B; i += nthr) {
-    F[i] = cand(i) ? 0 : 1;
-    nc += cand(i) ? 1 : 0;
-  }
-  int ncand;
-  (void)block_exclusive_scan(nc, sh + 8, &ncand);
-  const int nf = min(s.n_fix, ncand);
-  if (nf > 0) {
-    auto get = [&](int i, uint32_t* key) {
-      if (!cand(i)) return false;
-      *key = order_key(cu[pos(i)]);
-      return true;
-    };
-    block_topk_mark(get, [&](int i, int) { F[i] = 1; }, B, nf, hist, sh);
-  }
-  __syncthreads();
-
-  // Retained logits, then row softmax over the retained keys -> X.
-  for (int base = 0; base < B; base += 32) {
-    const int len = min(32, B - base);
-    __syncthreads();
-    for (int i = tid; i < 32 * kD; i += nthr) {
-      const int jj = i / kD, t = i % kD;
-      tile[jj * QP + t] = jj < len ? ldv(ku, (size_t)pos(base + jj) * kD + t) : 0.f;
-    }
-    __syncthreads();
-    for (int pr = tid; pr < m * 32; pr += nthr) {
-      const int r = pr >> 5, jj = pr & 31;
-      if (jj >= len) continue;
-      const int j = pos(base + jj);
-      float l = -INFINITY;
-      if (visible(s, r, j)) {
-        float a = 0.f;
-#pragma unroll 8
-        for (int t = 0; t < kD; ++t) a = fmaf(qs[r * QP + t], tile[jj * QP + t], a);
-        l = s.scale * a;
-      }
-      X[(size_t)r * B + base + jj] = l;
-    }
-  }
-  __syncthreads();
-  {
-    const int lane = tid & 31, wid = tid >> 5, nw = nthr >> 5;
-    for (int r = wid; r < m; r += nw) {
-      float* xr = X + (size_t)r * B;
-      float M = -INFINITY;
-      for (int i = lane; i < B; i += 32) M = fmaxf(M, xr[i]);
-      for (int o = 16; o; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-      float L = 0.f;
-      for (int i = lane; i < B; i += 32) L += expf(xr[i] - M);
-      for (int o = 16; o; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
-      for (int i = lane; i < B; i += 32) xr[i] = expf(xr[i] - M) / L;
-    }
-  }
-  __syncthreads();
-  if (s.lambda_inf) {
-    for (int i = tid; i < B * kD; i += nthr) vo[i] = vu[(size_t)pos(i / kD) * kD + i % kD];
-    return;
-  }
-
-  // R = Y - X V0, 16 rows per thread per pass.
-  const int e = tid & (kD - 1), rq = tid >> 7, nrq = nthr >> 7;
-  constexpr int RPP = 16;
-  for (int r0 = 0; r0 < m; r0 += RPP * nrq) {
-    A acc[RPP];
-#pragma unroll
-    for (int i = 0; i < RPP; ++i) acc[i] = 0;
-    for (int base = 0; base < B; base += 32) {
-      const int len = min(32, B - base);
-      __syncthreads();
-      for (int i = tid; i < 32 * kD; i += nthr) {
-        const int jj = i / kD, t = i % kD;
-        tile[jj * QP + t] = jj < len ? ldv(vu, (size_t)pos(base + jj) * kD + t) : 0.f;
-      }
-      for (int i = tid; i < m * 32; i += nthr) {
-        const int r = i >> 5, jj = i & 31;
-        xt[r * 33 + jj] = jj < len ? X[(size_t)r * B + base + jj] : 0.f;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int i = 0; i < RPP; ++i) {
-        const int r = r0 + rq + nrq * i;
-        if (r < m) {
-          A a = acc[i];
-          for (int jj = 0; jj < len; ++jj) a += (A)xt[r * 33 + jj] * (A)tile[jj * QP + e];
-          acc[i] = a;
-        }
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < RPP; ++i) {
-      const int r = r0 + rq + nrq * i;
-      if (r < m) RZ[(size_t)r * kD + e] = (A)yu[(size_t)r * kD + e] - acc[i];
-    }
-  }
-
-  // Gram of the free columns: N = X_G X_G^T + lambda I, 32 entries per thread per pass.
-  constexpr int GPP = 32;
-  for (int p0 = 0; p0 < m * m; p0 += GPP * nthr) {
-    A g[GPP];
-#pragma unroll
-    for (int i = 0; i < GPP; ++i) g[i] = 0;
-    for (int base = 0; base < B; base += 32) {
-      const int len = min(32, B - base);
-      __syncthreads();
-      for (int i = tid; i < m * 32; i += nthr) {
-        const int r = i >> 5, jj = i & 31;
-        xt[r * 33 + jj] = (jj < len && !F[base + jj]) ? X[(size_t)r * B + base + jj] : 0.f;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int i = 0; i < GPP; ++i) {
-        const int p = p0 + tid + nthr * i;
-        if (p < m * m) {
-          const int r1 = p / m, r2 = p % m;
-          A a = g[i];
-          for (int jj = 0; jj < len; ++jj) a += (A)xt[r1 * 33 + jj] * (A)xt[r2 * 33 + jj];
-          g[i] = a;
-        }
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < GPP; ++i) {
-      const int p = p0 + tid + nthr * i;
-      if (p < m * m) N[p] = g[i] + ((p / m == p % m) ? (A)s.lambda : (A)0);
-    }
-  }
-  __syncthreads();
-  if (phase == 1) return;
-
-  // Cholesky N = L L^T in place (lower triangle), right-looking.
-  for (int c = 0; c < m; ++c) {
-    if (tid == 0) {
-      const A dkk = N[(size_t)c * m + c];
-      sh[0] = (dkk > (A)0) ? 0 : 1;
-      if (dkk > (A)0) N[(size_t)c * m + c] = sqrt(dkk);
-    }
-    __syncthreads();
-    if (sh[0]) {  // singular dual system: report it and leave V0 in place
-      if (tid == 0) set_status(status, GRKV_ERR_NUMERIC);
-      for (int i = tid; i < B * kD; i += nthr) vo[i] = vu[(size_t)pos(i / kD) * kD + i % kD];
-      return;
-    }
-    const A piv = N[(size_t)c * m + c];
-    for (int i = c + 1 + tid; i < m; i += nthr) N[(size_t)i * m + c] /= piv;
-    __syncthreads();
-    const int rest = m - c - 1;
-    for (int p = tid; p < rest * rest; p += nthr) {
-      const int i = c + 1 + p / rest, j = c + 1 + p % rest;
-      if (j <= i) N[(size_t)i * m + j] -= N[(size_t)i * m + c] * N[(size_t)j * m + c];
-    }
-    __syncthreads();
-  }
-  // Z = N^-1 R: forward then backward substitution, one column per thread.
-  if (tid < kD) {
-    for (int i = 0; i < m; ++i) {
-      A z = RZ[(size_t)i * kD + tid];
-      for (int c = 0; c < i; ++c) z -= N[(size_t)i * m + c] * RZ[(size_t)c * kD + tid];
-      RZ[(size_t)i * kD + tid] = z / N[(size_t)i * m + i];
-    }
-    for (int i = m - 1; i >= 0; --i) {
-      A z = RZ[(size_t)i * kD + tid];
-      for (int c = i + 1; c < m; ++c) z -= N[(size_t)c * m + i] * RZ[(size_t)c * kD + tid];
-      RZ[(size_t)i * kD + tid] = z / N[(size_t)i * m + i];
-    }
-  }
-  __syncthreads();
-
-  }   // phase != 2
-
-  // V_out[G] = V0[G] + X_G^T Z, V_out[F] = V0[F].
-  for (int base = 0; base < B; base += 32) {
-    const int len = min(32, B - base);
-    __syncthreads();
-    for (int i = tid; i < m * 32; i += nthr) {
-      const int r = i >> 5, jj = i & 31;
-      xt[r * 33 + jj] = jj < len ? X[(size_t)r * B + base + jj] : 0.f;
-    }
-    __syncthreads();
-    for (int p = tid; p < len * kD; p += nthr) {
-      const int jj = p / kD, c = p % kD, i = base + jj;
-      const size_t src = (size_t)pos(i) * kD + c;
-      if (F[i]) {
-        vo[(size_t)i * kD + c] = vu[src];
-      } else {
-        A a = 0;
-        for (int r = 0; r < m; ++r) a += (A)xt[r * 33 + jj] * RZ[(size_t)r * kD + c];
-        stv(vo, (size_t)i * kD + c, (A)ldv(vu, src) + a);
-      }
-    }
-  }
-}
-
-template <typename T>
+template <typename T, int RT>
 cudaError_t score_impl(const Shape& s, const T* q, const T* k, const T* v, float* scores,
                        float* y, float* row_stats, char* ws, const WsLayout& L,
                        cudaStream_t st) {
   float2* pstats = (float2*)(ws + L.pstats);
   float* ypart = (float*)(ws + L.ypart);
-  const size_t smA = ((size_t)pad4(s.m * QP) + 64 * kD) * 4 + 256 * sizeof(float2);
-  cudaError_t e = cudaFuncSetAttribute(k_stats_chunk<T>,
+  constexpr size_t smA = stats_smem<RT>(), smB = prob_smem<RT>();
+  cudaError_t e = cudaFuncSetAttribute(k_stats_chunk<T, RT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smA);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_prob_chunk<T, RT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smB);
   if (e != cudaSuccess) return e;
-  dim3 grid(L.nchunk, s.U);
-  k_stats_chunk<T><<<grid, 256, smA, st>>>(q, k, s, L.chunk, L.nchunk, pstats);
-  k_stats_reduce<<<s.U, 256, 0, st>>>(pstats, s, L.nchunk, row_stats);
-  const size_t smB = ((size_t)s.m * QP + 32 * QP + 32 * kD + (size_t)s.m * 33 + s.m * 2) * 4;
-  auto launchB = [&](auto kern) {
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)smB);
-    if (err != cudaSuccess) return err;
-    kern<<<grid, 512, smB, st>>>(q, k, v, s, L.chunk, L.nchunk, row_stats, scores, ypart);
-    return cudaGetLastError();
-  };
-  const int rpt = (s.m + 3) / 4;
-  if (rpt <= 8) e = launchB(k_prob_chunk<T, 8>);
-  else if (rpt <= 16) e = launchB(k_prob_chunk<T, 16>);
-  else if (rpt <= 32) e = launchB(k_prob_chunk<T, 32>);
-  else e = launchB(k_prob_chunk<T, 64>);
-  if (e != cudaSuccess) return e;
-  k_y_reduce<<<s.U, 512, 0, st>>>(ypart, s, L.nchunk, y);
-  count_launches(4);
+  const dim3 grid(L.nchunk, s.U);
+  k_stats_chunk<T, RT><<<grid, kScT, smA, st>>>(q, k, s, L.chunk, L.nchunk, pstats);
+  k_prob_chunk<T, RT><<<grid, kScT, smB, st>>>(q, k, v, s, L.chunk, L.nchunk, pstats, row_stats,
+                                               scores, ypart);
+  k_y_reduce<<<dim3((s.m * (kD / 4) + 255) / 256, s.U), 256, 0, st>>>((const float4*)ypart, s,
+                                                                      L.nchunk, (float4*)y);
+  count_launches(3);
   return cudaGetLastError();
 }
 
-template <typename T, typename A>
-cudaError_t merge_impl(const Shape& s, const T* q, const T* k, const T* v, const float* scores,
-                       const float* y, const int32_t* idx, T* k_out, T* v_out, char* ws,
-                       const WsLayout& L, cudaStream_t st) {
-  const size_t sm = ((size_t)s.m * QP + 32 * QP + (size_t)s.m * 33) * 4;
-  cudaError_t e = cudaFuncSetAttribute(k_merge<T, A>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sm);
-  if (e != cudaSuccess) return e;
-  auto run = [&](int phase) {
-    k_merge<T, A><<<s.U, 512, sm, st>>>(q, k, v, scores, y, idx, k_out, v_out, s,
-                                        (float*)(ws + L.xbuf), (uint8_t*)(ws + L.flags),
-                                        (A*)(ws + L.gram), (A*)(ws + L.rz), (int*)(ws + L.status),
-                                        phase);
-    count_launches(1);
-    return cudaGetLastError();
-  };
-  // fp32 inputs keep the double-precision solve inside the kernel; bf16 inputs
-  // take the blocked shared-memory solve between two phases
-  if (!std::is_same<A, float>::value) return run(0);
-  if ((e = run(1)) != cudaSuccess) return e;
-  if (!s.lambda_inf &&
-      (e = launch_solve_dense(s.U, s.m, s.m, 0, 0.f, 0, (const float*)(ws + L.gram),
-                              (float*)(ws + L.rz), (int*)(ws + L.status), st)) != cudaSuccess)
-    return e;
-  return run(2);
+// The row tile follows m: 32 or 64 rows at a time waste less of it.
+template <typename T>
+cudaError_t score_rows(const Shape& s, const T* q, const T* k, const T* v, float* scores, float* y,
+                       float* row_stats, char* ws, const WsLayout& L, cudaStream_t st) {
+  if (s.m <= 32) return score_impl<T, 2>(s, q, k, v, scores, y, row_stats, ws, L, st);
+  if (s.m <= 64) return score_impl<T, 4>(s, q, k, v, scores, y, row_stats, ws, L, st);
+  return score_impl<T, 8>(s, q, k, v, scores, y, row_stats, ws, L, st);
 }
 
 }  // namespace
@@ -783,10 +604,28 @@ cudaError_t launch_score_simt(const Shape& s, const void* q, const void* k, cons
                               float* scores, float* y, float* row_stats, char* ws,
                               const WsLayout& L, cudaStream_t st) {
   if (s.dtype == GRKV_F32)
-    return score_impl<float>(s, (const float*)q, (const float*)k, (const float*)v, scores, y,
+    return score_rows<float>(s, (const float*)q, (const float*)k, (const float*)v, scores, y,
                              row_stats, ws, L, st);
-  return score_impl<__nv_bfloat16>(s, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k,
+  return score_rows<__nv_bfloat16>(s, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k,
                                    (const __nv_bfloat16*)v, scores, y, row_stats, ws, L, st);
+}
+
+// Keys per CTA of the portable scoring passes: whole tiles of 64, so that the
+// U x chunks CTAs (one per SM at a time) finish soonest, a CTA costing its
+// tiles plus about two tiles of set-up.
+int score_simt_chunk(const Shape& s) {
+  const long long tiles = (s.n + kKeys - 1) / kKeys, sms = 152, U = std::max(s.U, 1);
+  long long best = 1, cost = -1;
+  for (long long chunks = 1; chunks <= std::min(tiles, 608ll); ++chunks) {
+    const long long per = (tiles + chunks - 1) / chunks;
+    const long long ctas = U * ((tiles + per - 1) / per);
+    const long long c = (ctas + sms - 1) / sms * (per + 2);
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best = per;
+    }
+  }
+  return (int)best * kKeys;
 }
 
 bool select_uses_pooled_buffer(const Shape& s) { return s.P > kSelMaxP; }
@@ -809,18 +648,6 @@ cudaError_t launch_select_pooled(const Shape& s, const float* scores, int32_t* i
 cudaError_t launch_select(const Shape& s, const float* scores, int32_t* idx, char* ws,
                           const WsLayout& L, cudaStream_t st) {
   return launch_select_pooled(s, scores, idx, (float*)(ws + L.pooled), st);
-}
-
-cudaError_t launch_merge_simt(const Shape& s, const void* q, const void* k, const void* v,
-                              const float* scores, const float* y, const int32_t* idx,
-                              void* k_out, void* v_out, char* ws, const WsLayout& L,
-                              cudaStream_t st) {
-  if (s.dtype == GRKV_F32)
-    return merge_impl<float, double>(s, (const float*)q, (const float*)k, (const float*)v,
-                                     scores, y, idx, (float*)k_out, (float*)v_out, ws, L, st);
-  return merge_impl<__nv_bfloat16, float>(
-      s, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, scores, y,
-      idx, (__nv_bfloat16*)k_out, (__nv_bfloat16*)v_out, ws, L, st);
 }
 
 }  // namespace grkv
