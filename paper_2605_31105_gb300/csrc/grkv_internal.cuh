@@ -113,11 +113,14 @@ cudaError_t launch_score_tc(const Shape& s, const void* q, const void* k, const 
 
 // Tensor-core value merge (bf16, m <= 256 in 128-row blocks, B <= 32768).
 bool merge_tc_supported(const Shape& s);
-// The regression solve for m <= 256 (grkv_merge_tc.cu): gram [U][ld][ld]
+// The fp32 regression solve for m <= 256 (grkv_solve.cu): gram [U][ld][ld]
 // (N with lambda when sym = 0; raw Gram blocks, symmetrised with lambda added,
-// when sym = 1), rz [U][ld][128] (R in, Z out).
-cudaError_t launch_solve_dense(int U, int m, int ld, int sym, float lambda, int lambda_inf,
-                               const float* gram, float* rz, int* status, cudaStream_t st);
+// when sym = 1; the block of rows < 128, columns >= 128 is overwritten), rz
+// [U][ld][128] (R in, Z out).  For m > 128, fac holds 128 columns of fac_ld
+// floats per unit, units fac_unit floats apart, and fail one int per unit.
+cudaError_t launch_solve(int U, int m, int ld, int sym, float lambda, int lambda_inf, float* gram,
+                         float* rz, float* fac, size_t fac_unit, int fac_ld, int* fail,
+                         int* status, cudaStream_t st);
 size_t merge_tc_ws_bytes(const Shape& s);
 // row_stats (nullable): the full-cache row statistics; with them the Gram
 // needs one pass over the retained keys.

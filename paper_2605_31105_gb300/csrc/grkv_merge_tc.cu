@@ -18,8 +18,7 @@
 //                   terms).  Writes R = Y - R~, G and the row normalisers to the
 //                   workspace.  With the full-cache row statistics only pass 2
 //                   runs.
-//   k_merge_solve   fp32 in shared memory: N = sym(G) + lambda I, blocked
-//                   Cholesky, Z = N^-1 R by blocked triangular solves.
+//   launch_solve    N = sym(G) + lambda I, Z = N^-1 R in fp32 (grkv_solve.cu).
 //   k_merge_update  over the slots: S^T = K0 Q^T (one TMEM lane per token),
 //                   X_G^T (zero for fixed slots) as bf16 high / low parts back
 //                   into TMEM, dV = XGh^T Zh + XGh^T Zl + XGl^T Zh with X_G^T
@@ -47,7 +46,6 @@ constexpr int kThreadsU = 736;   // k_merge_update
 constexpr uint32_t kTileBytes = kTile * kD * 2;   // 32 KB
 constexpr int kMaxB = 32768;
 constexpr long long kBudget = 1ll << 32;
-constexpr int kLD = 129;   // fp32 row stride of N and R/Z in k_merge_solve
 
 // Shared memory (offsets from a 1024-byte aligned base).  k_merge_gram: Q, a
 // ring of four gathered tiles, two XGh tiles.  k_merge_update: Q, two K0
@@ -59,8 +57,6 @@ constexpr uint32_t kOffXG = kOffRing + kRingG * kTileBytes;   // gram: 2 tiles
 constexpr uint32_t kOffBar = 7 * kTileBytes;
 static_assert(kOffXG + 2 * kTileBytes == kOffBar, "shared-memory layout");
 constexpr uint32_t kSmemBytes = kOffBar + 256 + 1024;
-// k_merge_solve: packed N (tri(128) + 4 floats), R/Z [128][129] fp32, 1 / L_jj, the failure flag
-constexpr uint32_t kSolveSmem = ((128 * 129) / 2 + 4 + kRows * kLD + kRows + 32) * 4;
 
 // TMEM columns.  gram: S[2] 0..255, R~ 256..383, Gram 384..511.
 // update: S^T[2] (then X_G^T) 0..255, D[2] 256..511.
@@ -700,307 +696,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
-// ======================================================== k_merge_solve
-// N lives in shared memory as a packed lower triangle (row i at tri(i)), so
-// two CTAs fit on an SM.  The register-resident pieces of the blocked
-// Cholesky and of the triangular solves are separate (non-inlined) functions
-// so that their 32-element arrays stay in registers.
-__host__ __device__ constexpr int tri(int i) { return (i * (i + 1)) >> 1; }
-constexpr int kTri = tri(kRows) + 4;   // packed N, padded to 16 bytes
-constexpr int kSolveThreads = 256;
-
-// Factors the 32 x 32 diagonal block at k0 (right-looking; lane l holds row
-// k0 + l) and stores 1 / L_jj.  Returns true on a non-positive pivot.
-__device__ __noinline__ bool chol_diag(float* N, float* dinv, int k0, int lane) {
-  const int rb = tri(k0 + lane) + k0;
-  float x[32];
-#pragma unroll
-  for (int j = 0; j < 32; ++j) x[j] = j <= lane ? N[rb + j] : 0.f;
-  bool bad = false;
-#pragma unroll
-  for (int k = 0; k < 32; ++k) {
-    const float dkk = __shfl_sync(0xffffffffu, x[k], k);
-    bad |= !(dkk > 0.f);
-    const float inv = dkk > 0.f ? rsqrtf(dkk) : 0.f;   // 1 / L_kk
-    const float piv = dkk * inv;                         // L_kk
-    x[k] = lane == k ? piv : (lane > k ? x[k] * inv : x[k]);
-    const float lk = x[k];
-#pragma unroll
-    for (int j = k + 1; j < 32; ++j) {
-      const float ljk = __shfl_sync(0xffffffffu, x[k], j);
-      x[j] = lane >= j ? x[j] - lk * ljk : x[j];
-    }
-    if (lane == 0) dinv[k0 + k] = inv;
-  }
-#pragma unroll
-  for (int j = 0; j < 32; ++j)
-    if (j <= lane) N[rb + j] = x[j];
-  return bad;
-}
-
-// Row i of the panel below the diagonal block at k0: L_i,k0.. = A_i,k0.. L_kk^-T.
-__device__ __noinline__ void chol_panel_row(float* N, const float* dinv, int k0, int i) {
-  const int rb = tri(i) + k0;
-  float x[32];
-#pragma unroll
-  for (int j = 0; j < 32; ++j) x[j] = N[rb + j];
-#pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    const float* lj = N + tri(k0 + j) + k0;
-    float s0 = x[j], s1 = 0.f;
-#pragma unroll
-    for (int p = 0; p < j; ++p) {
-      if (p & 1) s1 += x[p] * lj[p];
-      else s0 -= x[p] * lj[p];
-    }
-    x[j] = (s0 - s1) * dinv[k0 + j];
-  }
-#pragma unroll
-  for (int j = 0; j < 32; ++j) N[rb + j] = x[j];
-}
-
-// Inverts the lower-triangular 32 x 32 diagonal block at k0 in place: lane l
-// computes column l of L_bb^-1 by forward substitution (its entries above the
-// diagonal come out zero) and writes it once every lane has read the block.
-__device__ __noinline__ void tri_inv_diag(float* N, const float* dinv, int k0, int lane) {
-  float x[32];
-#pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    const float* li = N + tri(k0 + i) + k0;
-    float s0 = i == lane ? 1.f : 0.f, s1 = 0.f;
-#pragma unroll
-    for (int k = 0; k < i; ++k) {
-      if (k & 1) s1 += li[k] * x[k];
-      else s0 -= li[k] * x[k];
-    }
-    x[i] = (s0 - s1) * dinv[k0 + i];
-  }
-  __syncwarp();
-#pragma unroll
-  for (int i = 0; i < 32; ++i)
-    if (i >= lane) N[tri(k0 + i) + k0 + lane] = x[i];
-}
-
-// N = (G + G^T) / 2 + lambda I on the window rows (identity on padding rows),
-// Cholesky N = L L^T in 32-row blocks, then Z = L^-T L^-1 R by block
-// substitution with the inverted diagonal blocks; fp32 in shared memory.  A non-positive pivot reports GRKV_ERR_NUMERIC and leaves Z = 0
-// (values stay V0); lambda = +inf also gives Z = 0.
-__global__ void __launch_bounds__(kSolveThreads, 2) k_merge_solve(MArgs a) {
-  extern __shared__ __align__(16) float ssm[];
-  float* N = ssm;                   // packed lower triangle
-  float* R = N + kTri;              // [128][kLD]: G first, then R, then Z
-  float* dinv = R + kRows * kLD;    // [128]
-  int* fail = (int*)(dinv + kRows);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nt = blockDim.x;
-  const int u = blockIdx.x, m = a.m;
-  float* RZ = a.rz + (size_t)u * kRows * kD;
-  if (a.lambda_inf) {
-    for (int p = tid; p < kRows * kD / 4; p += nt) ((float4*)RZ)[p] = make_float4(0.f, 0.f, 0.f, 0.f);
-    return;
-  }
-  if (tid == 0) *fail = 0;
-  // G into the R buffer with every load of a half in flight at once (one
-  // element per lane and step: conflict-free stores into the padded rows)
-  const float* Gs = a.gram + (size_t)u * kRows * kRows;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    float g[32];
-#pragma unroll
-    for (int k = 0; k < 32; ++k) g[k] = __ldg(Gs + tid + kSolveThreads * (32 * h + k));
-#pragma unroll
-    for (int k = 0; k < 32; ++k) {
-      const int p = tid + kSolveThreads * (32 * h + k);
-      R[(p >> 7) * kLD + (p & 127)] = g[k];
-    }
-  }
-  // R's loads are issued before the symmetric part is formed and stored after
-  float rr[64];
-#pragma unroll
-  for (int k = 0; k < 64; ++k) rr[k] = __ldg(RZ + tid + kSolveThreads * k);
-  __syncthreads();
-  for (int i = warp; i < kRows; i += kSolveThreads / 32)
-    for (int j = lane; j <= i; j += 32) {
-      float val;
-      if (i >= m || j >= m) val = (i == j) ? 1.f : 0.f;
-      else if (i == j) val = R[i * kLD + i] + a.lambda;
-      else val = 0.5f * (R[i * kLD + j] + R[j * kLD + i]);
-      N[tri(i) + j] = val;
-    }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < 64; ++k) {
-    const int p = tid + kSolveThreads * k;
-    R[(p >> 7) * kLD + (p & 127)] = rr[k];
-  }
-  for (int kb = 0; kb < kRows / 32; ++kb) {
-    const int k0 = kb * 32;
-    if (warp == 0 && chol_diag(N, dinv, k0, lane) && lane == 0) *fail = 1;
-    __syncthreads();
-    for (int i = k0 + 32 + tid; i < kRows; i += nt) chol_panel_row(N, dinv, k0, i);
-    __syncthreads();
-    // trailing update of the lower triangle in 4x4 register blocks
-    const int k1 = k0 + 32, t4 = (kRows - k1) / 4, nb = t4 * (t4 + 1) / 2;
-    for (int t = tid; t < nb; t += nt) {
-      int bi = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
-      while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
-      while (bi * (bi + 1) / 2 > t) --bi;
-      const int i = k1 + 4 * bi, j = k1 + 4 * (t - bi * (bi + 1) / 2);
-      float acc[4][4] = {};
-      const float* li[4];
-      const float* lj[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        li[r] = N + tri(i + r) + k0;
-        lj[r] = N + tri(j + r) + k0;
-      }
-#pragma unroll 4
-      for (int pp = 0; pp < 32; ++pp) {
-        float vi[4], vj[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          vi[r] = li[r][pp];
-          vj[r] = lj[r][pp];
-        }
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) acc[r][c] += vi[r] * vj[c];
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-          if (j + c <= i + r) N[tri(i + r) + j + c] -= acc[r][c];
-    }
-    __syncthreads();
-  }
-  if (*fail) {
-    if (tid == 0) set_status(a.status, GRKV_ERR_NUMERIC);
-    for (int p = tid; p < kRows * kD / 4; p += nt) ((float4*)RZ)[p] = make_float4(0.f, 0.f, 0.f, 0.f);
-    return;
-  }
-  // the diagonal blocks of L are replaced by their inverses (one warp each)
-  if (warp < kRows / 32) tri_inv_diag(N, dinv, warp * 32, lane);
-  __syncthreads();
-  // forward: L W = R in 32-row blocks, W_b = L_bb^-1 (R_b - L_b,<b W_<b);
-  // thread: rows 4 rg .. 4 rg + 3 of the block, columns e + 32 c
-  const int rg = warp, e = lane;
-  for (int ib = 0; ib < kRows / 32; ++ib) {
-    const int i0 = ib * 32;
-    {
-      float acc[4][4] = {};
-      const float* lr[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) lr[r] = N + tri(i0 + 4 * rg + r) + i0;
-#pragma unroll 4
-      for (int kx = 0; kx < 4 * rg + 4; ++kx) {
-        float l[4], z[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) l[r] = kx <= 4 * rg + r ? lr[r][kx] : 0.f;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) z[c] = R[(i0 + kx) * kLD + e + 32 * c];
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) acc[r][c] += l[r] * z[c];
-      }
-      __syncthreads();
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) R[(i0 + 4 * rg + r) * kLD + e + 32 * c] = acc[r][c];
-    }
-    __syncthreads();
-    // rows below: 4 rows x 4 columns (stride 32) per thread
-    const int i1 = i0 + 32, nb = (kRows - i1) / 4 * 32;
-    for (int t = tid; t < nb; t += nt) {
-      const int i = i1 + 4 * (t >> 5), e = t & 31;
-      float acc[4][4] = {};
-      const float* li[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) li[r] = N + tri(i + r) + i0;
-#pragma unroll 4
-      for (int kx = 0; kx < 32; ++kx) {
-        float l[4], z[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) l[r] = li[r][kx];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) z[c] = R[(i0 + kx) * kLD + e + 32 * c];
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) acc[r][c] += l[r] * z[c];
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) R[(i + r) * kLD + e + 32 * c] -= acc[r][c];
-    }
-    __syncthreads();
-  }
-  // backward: L^T Z = W, Z_b = L_bb^-T (W_b - L_>b,b^T Z_>b)
-  for (int ib = kRows / 32 - 1; ib >= 0; --ib) {
-    const int i0 = ib * 32;
-    {
-      float acc[4][4] = {};
-#pragma unroll 4
-      for (int kx = 4 * rg; kx < 32; ++kx) {
-        const float* lk = N + tri(i0 + kx) + i0 + 4 * rg;
-        float l[4], z[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) l[r] = 4 * rg + r <= kx ? lk[r] : 0.f;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) z[c] = R[(i0 + kx) * kLD + e + 32 * c];
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) acc[r][c] += l[r] * z[c];
-      }
-      __syncthreads();
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) R[(i0 + 4 * rg + r) * kLD + e + 32 * c] = acc[r][c];
-    }
-    __syncthreads();
-    // rows above: 4 rows x 4 columns (stride 32) per thread
-    const int nb = i0 / 4 * 32;
-    for (int t = tid; t < nb; t += nt) {
-      const int i = 4 * (t >> 5), e = t & 31;
-      float acc[4][4] = {};
-#pragma unroll 4
-      for (int kx = 0; kx < 32; ++kx) {
-        const float* lk = N + tri(i0 + kx) + i;
-        float l[4], z[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) l[r] = lk[r];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) z[c] = R[(i0 + kx) * kLD + e + 32 * c];
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) acc[r][c] += l[r] * z[c];
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) R[(i + r) * kLD + e + 32 * c] -= acc[r][c];
-    }
-    __syncthreads();
-  }
-  for (int p = tid; p < kRows * kD / 4; p += nt) {
-    const float* rr = R + (p >> 5) * kLD + (p & 31) * 4;
-    ((float4*)RZ)[p] = make_float4(rr[0], rr[1], rr[2], rr[3]);
-  }
-}
-
 // ======================================================== k_merge_cross
 // The off-diagonal Gram block of a unit with two row blocks (128 < m <= 256):
 // G01 = X_G0 X_G1^T over the non-fixed positions, as the split products
 // Xh0 Xh1^T + Xl0 Xh1^T + Xh0 Xl1^T (the low-low term dropped, as in the
 // diagonal blocks).  X uses the final row normalisers of both blocks (from
 // the diagonal launches), so nothing is rescaled afterwards.  G01 goes to
-// gram[u][r0][128 + r1] and, transposed, to gram[u][128 + r1][r0].  Roles
+// gram[u][r0][128 + r1].  Roles
 // (384 threads): warp 0 the Q loads; warps 0, 2, 3 the K0 gathers; warp 1 MMA
 // issue; warps 4-7 the rows of block 0 (X_0 high / low parts written back
 // over S_0 in TMEM, the A operands); warps 8-11 the rows of block 1 (XGh_1,
@@ -1165,18 +867,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc_fence_after();
       if (ok) {
         float* up = a.gram + ((size_t)u * a.ldr + row) * a.ldr + kRows;   // row r0, columns 128 + r1
-        float* lo = a.gram + ((size_t)u * a.ldr + kRows) * a.ldr + row;    // rows 128 + r1, column r0
 #pragma unroll 1
         for (int c = 0; c < 4; ++c) {
           float g[32];
           tmem_ld32f(lane_addr + kColGC + 32 * c, g);
           tmem_wait32(g);
 #pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            const float x = TG > 0 ? g[e] : 0.f;
-            up[32 * c + e] = x;
-            lo[(size_t)(32 * c + e) * a.ldr] = x;
-          }
+          for (int e = 0; e < 32; e += 4)
+            *(float4*)(up + 32 * c + e) = TG > 0 ? make_float4(g[e], g[e + 1], g[e + 2], g[e + 3])
+                                                 : make_float4(0.f, 0.f, 0.f, 0.f);
         }
       }
     }
@@ -1186,173 +885,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   if (warp == 1) tmem_dealloc(tmem, 512);
-}
-
-// ======================================================== k_solve_dense
-// The regression solve for m <= 256: N and R ([m][128]) from the workspace,
-// Z = N^-1 R written over R.  With sym = 0, gram holds N = X_G X_G^T +
-// lambda I (the portable merge); with sym = 1 it holds the raw Gram blocks of
-// the tensor-core merge and N = (G + G^T) / 2 + lambda I.  Each unit's arrays
-// hold ld rows.  The same blocked fp32 algorithm as k_merge_solve, for up to
-// 256 rows: N as a packed lower triangle in shared memory (rows past m are
-// identity), Cholesky in 32-row blocks, the diagonal blocks inverted in place,
-// then block substitution over R in two passes of 64 columns.  lambda = +inf
-// gives Z = 0.  One 512-thread CTA per unit.
-constexpr int kDenseM = 256, kDenseNT = 512, kDenseC = 64, kDenseLD = kDenseC + 1;
-constexpr int kDenseTri = tri(kDenseM) + 4;
-constexpr uint32_t kDenseSmem = (kDenseTri + kDenseM * kDenseLD + kDenseM + 32) * 4;
-
-__global__ void __launch_bounds__(kDenseNT, 1)
-    k_solve_dense(const float* __restrict__ gram, float* __restrict__ rz, int m, int ld, int sym,
-                  float lambda, int lambda_inf, int* status) {
-  extern __shared__ __align__(16) float dsm[];
-  float* N = dsm;                       // packed lower triangle
-  float* R = N + kDenseTri;             // [256][kDenseLD]: one column pass of R, then of Z
-  float* dinv = R + kDenseM * kDenseLD; // [256]
-  int* fail = (int*)(dinv + kDenseM);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int u = blockIdx.x;
-  const float* Gu = gram + (size_t)u * ld * ld;
-  float* RZ = rz + (size_t)u * ld * kD;
-  if (lambda_inf) {
-    for (int p = tid; p < m * kD; p += kDenseNT) RZ[p] = 0.f;
-    return;
-  }
-  if (tid == 0) *fail = 0;
-  // the lower triangle row by row (with sym: halved off the diagonal, lambda
-  // added on it), then with sym the upper triangle's halves added, also read
-  // row by row: both passes load whole rows
-  for (int i = warp; i < kDenseM; i += kDenseNT / 32)
-    for (int j = lane; j <= i; j += 32) {
-      float val = i == j ? 1.f : 0.f;
-      if (i < m && j < m) {
-        val = __ldg(Gu + (size_t)i * ld + j);
-        if (sym) val = i == j ? val + lambda : 0.5f * val;
-      }
-      N[tri(i) + j] = val;
-    }
-  if (sym) {
-    __syncthreads();
-    for (int r = warp; r < m; r += kDenseNT / 32)
-      for (int c = r + 1 + lane; c < m; c += 32) N[tri(c) + r] += 0.5f * __ldg(Gu + (size_t)r * ld + c);
-  }
-  __syncthreads();
-  for (int kb = 0; kb < kDenseM / 32; ++kb) {
-    const int k0 = kb * 32;
-    if (warp == 0 && chol_diag(N, dinv, k0, lane) && lane == 0) *fail = 1;
-    __syncthreads();
-    for (int i = k0 + 32 + tid; i < kDenseM; i += kDenseNT) chol_panel_row(N, dinv, k0, i);
-    __syncthreads();
-    // trailing update of the lower triangle in 4x4 register blocks
-    const int k1 = k0 + 32, t4 = (kDenseM - k1) / 4, nb = t4 * (t4 + 1) / 2;
-    for (int t = tid; t < nb; t += kDenseNT) {
-      int bi = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
-      while ((bi + 1) * (bi + 2) / 2 <= t) ++bi;
-      while (bi * (bi + 1) / 2 > t) --bi;
-      const int i = k1 + 4 * bi, j = k1 + 4 * (t - bi * (bi + 1) / 2);
-      float acc[4][4] = {};
-#pragma unroll 4
-      for (int pp = 0; pp < 32; ++pp) {
-        float vi[4], vj[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          vi[r] = N[tri(i + r) + k0 + pp];
-          vj[r] = N[tri(j + r) + k0 + pp];
-        }
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) acc[r][c] += vi[r] * vj[c];
-      }
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-          if (j + c <= i + r) N[tri(i + r) + j + c] -= acc[r][c];
-    }
-    __syncthreads();
-  }
-  if (*fail) {
-    if (tid == 0) set_status(status, GRKV_ERR_NUMERIC);
-    for (int p = tid; p < m * kD; p += kDenseNT) RZ[p] = 0.f;
-    return;
-  }
-  if (warp < kDenseM / 32) tri_inv_diag(N, dinv, warp * 32, lane);
-  __syncthreads();
-  // block steps: thread = rows 4 rg .. 4 rg + 3 of a 32-row block, column cc
-  const int rg = warp & 7, cc = (tid >> 8) * 32 + lane;
-  for (int c0 = 0; c0 < kD; c0 += kDenseC) {
-    for (int p = tid; p < kDenseM * kDenseC; p += kDenseNT) {
-      const int r = p / kDenseC, c = p % kDenseC;
-      R[r * kDenseLD + c] = r < m ? RZ[(size_t)r * kD + c0 + c] : 0.f;
-    }
-    __syncthreads();
-    // forward: W_b = L_bb^-1 (R_b - L_b,<b W_<b)
-    for (int ib = 0; ib < kDenseM / 32; ++ib) {
-      const int i0 = ib * 32;
-      float acc[4] = {};
-      for (int kx = 0; kx < 4 * rg + 4; ++kx) {
-        const float z = R[(i0 + kx) * kDenseLD + cc];
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-          acc[r] += (kx <= 4 * rg + r ? N[tri(i0 + 4 * rg + r) + i0 + kx] : 0.f) * z;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int r = 0; r < 4; ++r) R[(i0 + 4 * rg + r) * kDenseLD + cc] = acc[r];
-      __syncthreads();
-      // rows below: 4 rows x 1 column per task
-      const int i1 = i0 + 32, ntask = (kDenseM - i1) / 4 * kDenseC;
-      for (int t = tid; t < ntask; t += kDenseNT) {
-        const int i = i1 + 4 * (t / kDenseC), c = t % kDenseC;
-        float a4[4] = {};
-#pragma unroll 8
-        for (int kx = 0; kx < 32; ++kx) {
-          const float z = R[(i0 + kx) * kDenseLD + c];
-#pragma unroll
-          for (int r = 0; r < 4; ++r) a4[r] += N[tri(i + r) + i0 + kx] * z;
-        }
-#pragma unroll
-        for (int r = 0; r < 4; ++r) R[(i + r) * kDenseLD + c] -= a4[r];
-      }
-      __syncthreads();
-    }
-    // backward: Z_b = L_bb^-T (W_b - L_>b,b^T Z_>b)
-    for (int ib = kDenseM / 32 - 1; ib >= 0; --ib) {
-      const int i0 = ib * 32;
-      float acc[4] = {};
-      for (int kx = 4 * rg; kx < 32; ++kx) {
-        const float z = R[(i0 + kx) * kDenseLD + cc];
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-          acc[r] += (4 * rg + r <= kx ? N[tri(i0 + kx) + i0 + 4 * rg + r] : 0.f) * z;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int r = 0; r < 4; ++r) R[(i0 + 4 * rg + r) * kDenseLD + cc] = acc[r];
-      __syncthreads();
-      // rows above: 4 rows x 1 column per task
-      const int ntask = i0 / 4 * kDenseC;
-      for (int t = tid; t < ntask; t += kDenseNT) {
-        const int i = 4 * (t / kDenseC), c = t % kDenseC;
-        float a4[4] = {};
-#pragma unroll 8
-        for (int kx = 0; kx < 32; ++kx) {
-          const float z = R[(i0 + kx) * kDenseLD + c];
-#pragma unroll
-          for (int r = 0; r < 4; ++r) a4[r] += N[tri(i0 + kx) + i + r] * z;
-        }
-#pragma unroll
-        for (int r = 0; r < 4; ++r) R[(i + r) * kDenseLD + c] -= a4[r];
-      }
-      __syncthreads();
-    }
-    for (int p = tid; p < m * kDenseC; p += kDenseNT) {
-      const int r = p / kDenseC, c = p % kDenseC;
-      RZ[(size_t)r * kD + c0 + c] = R[r * kDenseLD + c];
-    }
-    __syncthreads();
-  }
 }
 
 // ======================================================== k_merge_update
@@ -1702,17 +1234,6 @@ MergeWs merge_ws(const Shape& s) {
 
 size_t merge_tc_ws_bytes(const Shape& s) { return merge_ws(s).total; }
 
-cudaError_t launch_solve_dense(int U, int m, int ld, int sym, float lambda, int lambda_inf,
-                               const float* gram, float* rz, int* status, cudaStream_t st) {
-  if (m > kDenseM || ld < m) return cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(k_solve_dense, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kDenseSmem);
-  if (e != cudaSuccess) return e;
-  k_solve_dense<<<U, kDenseNT, kDenseSmem, st>>>(gram, rz, m, ld, sym, lambda, lambda_inf, status);
-  count_launches(1);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const void* v,
                             const float* scores, const float* y, const float* row_stats,
                             const int32_t* idx, void* k_out, void* v_out, char* ws,
@@ -1763,8 +1284,6 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
                                 kSmemBytes)) != cudaSuccess ||
       (e = cudaFuncSetAttribute(k_merge_update, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 kSmemBytesU)) != cudaSuccess ||
-      (e = cudaFuncSetAttribute(k_merge_solve, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                kSolveSmem)) != cudaSuccess ||
       (e = cudaFuncSetAttribute(k_merge_fixed, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 s.B * 4)) != cudaSuccess)
     return e;
@@ -1789,23 +1308,26 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
       launches += 1;
     }
   }
+  if (W.nrb > 1) {
+    k_merge_cross<<<s.U, kThreads, kSmemBytesC, st>>>(mq, mk, a);
+    launches += 1;
+  }
+  count_launches(launches);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  // with two row blocks the solve keeps its first factor where the transpose of
+  // the cross block would be, and its failure flags in redo, which is spent
+  if ((e = launch_solve(s.U, s.m, W.ldr, 1, s.lambda, s.lambda_inf, a.gram, a.rz,
+                        a.gram + (size_t)kRows * W.ldr, (size_t)W.ldr * W.ldr, W.ldr, a.redo,
+                        a.status, st)) != cudaSuccess)
+    return e;
   if (W.nrb == 1) {
     a.rb = 0;
     a.row0 = 0;
     a.upd_mode = 0;
-    k_merge_solve<<<s.U, kSolveThreads, kSolveSmem, st>>>(a);
     k_merge_update<<<s.U, kThreadsU, kSmemBytesU, st>>>(mq, mk, mv, mko, mvo, a);
-    launches += 2;
+    launches = 1;
   } else {
-    // two row blocks: the cross Gram block, the 256-row solve, and the value
-    // update of each row block (the first leaves V0 + dV_0 in vpart)
-    k_merge_cross<<<s.U, kThreads, kSmemBytesC, st>>>(mq, mk, a);
-    launches += 1;
-    count_launches(launches);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = launch_solve_dense(s.U, s.m, W.ldr, 1, s.lambda, s.lambda_inf, a.gram, a.rz,
-                                a.status, st)) != cudaSuccess)
-      return e;
+    // the value update of each row block (the first leaves V0 + dV_0 in vpart)
     launches = 0;
     for (int rb = 0; rb < 2; ++rb) {
       a.rb = rb;

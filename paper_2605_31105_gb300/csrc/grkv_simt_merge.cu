@@ -21,7 +21,7 @@
 //   k_simt_solve64  units left to fp64
 //   k_simt_update   V_out = V0 + X_G^T Z in 32 x 32 tiles
 // bf16 inputs run the same tiles with plain fp32 sums and the blocked fp32
-// solve (k_solve_dense).
+// solve (grkv_solve.cu).
 #include <cmath>
 #include <type_traits>
 
@@ -666,7 +666,11 @@ cudaError_t merge_impl(const Shape& s, const T* q, const T* k, const T* v, const
       count_launches(1);
       e = cudaGetLastError();
     } else {
-      e = launch_solve_dense(s.U, s.m, s.m, 0, 0.f, 0, (const float*)gram, (float*)rz, a.status, st);
+      // gram's region holds 8 bytes per entry: the second half takes the factor
+      // of the first 128 rows (m^2 >= 128^2 floats a unit where it is used)
+      e = launch_solve(s.U, s.m, s.m, 0, 0.f, 0, (float*)gram, (float*)rz,
+                       (float*)gram + (size_t)s.U * s.m * s.m, (size_t)s.m * s.m, 128, a.state,
+                       a.status, st);
     }
   }
   if (e != cudaSuccess) return e;
