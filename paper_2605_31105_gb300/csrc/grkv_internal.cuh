@@ -125,6 +125,11 @@ size_t merge_tc_ws_bytes(const Shape& s);
 // row_stats (nullable): the full-cache row statistics; with them the Gram
 // needs one pass over the retained keys.
 size_t key_ws_bytes(const Shape& s);
+// The value step's fixed-token flags [U][B] in the workspace, on either path.
+const uint8_t* merge_tc_fixed(const Shape& s, const char* ws, const WsLayout& L);
+inline const uint8_t* value_step_fixed(const Shape& s, const char* ws, const WsLayout& L) {
+  return s.tc_merge ? merge_tc_fixed(s, ws, L) : (const uint8_t*)(ws + L.flags);
+}
 // The key step (GRKV_UPDATE_K) and, for S > 1, the remaining alternating
 // steps; k, v are the full caches (K0 and V0 of steps t >= 1).
 cudaError_t launch_key_step(const Shape& s, const void* q, const void* k, const void* v,

@@ -35,6 +35,7 @@
 
 #include "block_select.cuh"
 #include "grkv_internal.cuh"
+#include "key_args.cuh"
 #include "sm100.cuh"
 
 namespace grkv {
@@ -1259,37 +1260,7 @@ cudaError_t launch_key_step(const Shape& s, const void* q, const void* k, const 
   a.k_out = k_out;
   a.status = (int*)(ws + L.status);
   a.use_tc = s.m <= 128;
-  const uint32_t dyn = a.use_tc ? kTcSmem : 0;
-  cudaError_t e = cudaFuncSetAttribute(k_key_step, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kTcSmem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_alternate_step, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kTcSmem);
-  if (e != cudaSuccess) return e;
-  // the split the workspace was sized for, halved while the device cannot
-  // hold a cluster of that many CTAs
-  int C = key_cluster(s);
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  cfg.blockDim = dim3(kKT);
-  cfg.dynamicSmemBytes = dyn;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  for (; C > 1; C /= 2) {
-    cfg.gridDim = dim3((unsigned)(U * C));
-    attr[0].val.clusterDim.x = C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, k_key_step, &cfg) == cudaSuccess &&
-        nclusters > 0)
-      break;
-    (void)cudaGetLastError();
-  }
-  const KeyLayout kl = key_layout(s, C);
-  a.cluster = C;
+  const KeyLayout kl = key_layout(s, key_cluster(s));
   a.vec = (float*)(base + kl.vec);
   a.app = (float*)(base + kl.app);
   a.rho2p = (float*)(base + kl.rho2p);
@@ -1300,6 +1271,7 @@ cudaError_t launch_key_step(const Shape& s, const void* q, const void* k, const 
   a.T2 = (float*)(base + kl.T2);
   a.GQ = (float*)(base + kl.GQ);
   a.fixed = (uint8_t*)(base + kl.fixed);
+  cudaError_t e;
   if (s.steps > 1) {
     char* alt = base + kl.alt;
     a.Kt = (float*)alt;
@@ -1307,19 +1279,55 @@ cudaError_t launch_key_step(const Shape& s, const void* q, const void* k, const 
     a.G = a.Vt + U * B * d;
     a.RZ = a.G + U * m * m;
     a.done = (int*)(a.RZ + U * m * d);
-    e = cudaMemsetAsync(a.done, 0, U * sizeof(int), st);
-    if (e != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(a.done, 0, U * sizeof(int), st)) != cudaSuccess) return e;
   }
-  count_launches(1);
-  if (C > 1) {
-    e = cudaMemsetAsync(a.cnt, 0, U * sizeof(int), st);
-    if (e != cudaSuccess) return e;
-    cfg.gridDim = dim3((unsigned)(U * C));
-    attr[0].val.clusterDim.x = C;
-    e = cudaLaunchKernelEx(&cfg, k_key_step, a);
-  } else {
-    k_key_step<<<s.U, kKT, dyn, st>>>(a);
-    e = cudaGetLastError();
+  const KeyClusterArgs ca{s.n, s.w, s.m, s.B, s.causal, s.cg_iters, s.scale, s.lambda_k, s.cg_tol,
+                          q, y, idx, value_step_fixed(s, ws, L), v_out, k_out, a.Kt, a.status};
+  bool on_chip = false;
+  e = launch_key_cluster(s, ca, st, &on_chip);
+  if (e != cudaSuccess || (on_chip && s.steps == 1)) return e;
+  const uint32_t dyn = a.use_tc ? kTcSmem : 0;
+  e = cudaFuncSetAttribute(k_key_step, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_alternate_step, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kTcSmem);
+  if (e != cudaSuccess) return e;
+  a.cluster = 1;
+  if (!on_chip) {
+    // the split the workspace was sized for, halved while the device cannot
+    // hold a cluster of that many CTAs
+    int C = key_cluster(s);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cfg.blockDim = dim3(kKT);
+    cfg.dynamicSmemBytes = dyn;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    for (; C > 1; C /= 2) {
+      cfg.gridDim = dim3((unsigned)(U * C));
+      attr[0].val.clusterDim.x = C;
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      int nclusters = 0;
+      if (cudaOccupancyMaxActiveClusters(&nclusters, k_key_step, &cfg) == cudaSuccess &&
+          nclusters > 0)
+        break;
+      (void)cudaGetLastError();
+    }
+    a.cluster = C;
+    count_launches(1);
+    if (C > 1) {
+      e = cudaMemsetAsync(a.cnt, 0, U * sizeof(int), st);
+      if (e != cudaSuccess) return e;
+      cfg.gridDim = dim3((unsigned)(U * C));
+      attr[0].val.clusterDim.x = C;
+      e = cudaLaunchKernelEx(&cfg, k_key_step, a);
+    } else {
+      k_key_step<<<s.U, kKT, dyn, st>>>(a);
+      e = cudaGetLastError();
+    }
   }
   for (int t = 1; t < s.steps && e == cudaSuccess; ++t) {
     a.vt_valid = t > 1;   // V^(1) exists only as written to v_out (rounded)

@@ -1234,6 +1234,10 @@ MergeWs merge_ws(const Shape& s) {
 
 size_t merge_tc_ws_bytes(const Shape& s) { return merge_ws(s).total; }
 
+const uint8_t* merge_tc_fixed(const Shape& s, const char* ws, const WsLayout& L) {
+  return (const uint8_t*)(ws + L.merge_tc + merge_ws(s).fixed);
+}
+
 cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const void* v,
                             const float* scores, const float* y, const float* row_stats,
                             const int32_t* idx, void* k_out, void* v_out, char* ws,
