@@ -42,8 +42,9 @@ constexpr uint32_t kVPart = kNc * 128 * 2;     // one part of the CTA's K0 or V*
 constexpr uint32_t kSPart = 128 * kNc * 2;     // one part of dS
 constexpr uint32_t kDBytes = 128 * 128 * 4;    // dS parts, or the exchanged m x d values
 
-// TMEM columns: parts of p (or alpha), parts of dS2 (or X), T / T2, the product.
-constexpr uint32_t kColP = 0, kColX = 192, kColT = 288, kColO = 352;
+// TMEM columns: parts of p (or alpha; Q Q^T at first), parts of dS2 (or X), then
+// T, the three orders of T2, or the product with V*.
+constexpr uint32_t kColP = 0, kColX = 192, kColT = 288, kColO = kColT;
 
 template <int kC>
 struct alignas(16) Misc {
@@ -325,7 +326,7 @@ __global__ void __launch_bounds__(kThr, 1) k_key_cluster(KeyClusterArgs a) {
     products(kParts, kParts, [&](int pa, int pb, uint32_t acc) {
 #pragma unroll
       for (int kk = 0; kk < 8; ++kk)
-        mma_bf16(tm + kColO, sw128_desc(gqa + pa * kQPart + (kk >> 2) * (kQPart / 2) + (kk & 3) * 32, 16, 1024),
+        mma_bf16(tm + kColP, sw128_desc(gqa + pa * kQPart + (kk >> 2) * (kQPart / 2) + (kk & 3) * 32, 16, 1024),
                  sw128_desc(gqa + pb * kQPart + (kk >> 2) * (kQPart / 2) + (kk & 3) * 32, 16, 1024),
                  idesc_bf16(128, 128, 0, 0), acc | (kk > 0));
     });
@@ -371,7 +372,7 @@ __global__ void __launch_bounds__(kThr, 1) k_key_cluster(KeyClusterArgs a) {
 #pragma unroll 1
   for (int h = 0; h < 2; ++h) {
     float v[32];
-    tmem_ld32f(lane_tm + kColO + 64 * half + 32 * h, v);
+    tmem_ld32f(lane_tm + kColP + 64 * half + 32 * h, v);
     tmem_wait32(v);
     const float s2 = a.scale * a.scale;
 #pragma unroll
@@ -500,21 +501,31 @@ __global__ void __launch_bounds__(kThr, 1) k_key_cluster(KeyClusterArgs a) {
     stage_ds();
     if (!ready(ok)) break;
     if (tid == 0)
-      products(3, 3, [&](int pa, int pb, uint32_t acc) {   // T2 = (s^2 Q Q^T) dS
+      products(3, 1, [&](int pa, int, uint32_t acc) {
+        // T2 = (s^2 Q Q^T) dS: part pa meets parts 0 .. 2 - pa of dS side by side (64
+        // columns each), so that order o = pa + pb gathers at columns 64 o; one part pair at
+        // a time, each MMA would read A again for half the columns (3.7 K cycles against 1.9 K)
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk)
-          mma_bf16(tm + kColT, sw128_desc(gqa + pa * kQPart + (kk >> 2) * (kQPart / 2) + (kk & 3) * 32, 16, 1024),
-                   sw128_desc(dta + pb * kSPart + kk * 2048, kSPart, 1024),
-                   idesc_bf16(128, nn, 0, 1), acc | (kk > 0));
+          mma_bf16(tm + kColT + 64 * pa,
+                   sw128_desc(gqa + pa * kQPart + (kk >> 2) * (kQPart / 2) + (kk & 3) * 32, 16, 1024),
+                   sw128_desc(dta + kk * 2048, kSPart, 1024),
+                   idesc_bf16(128, 64 * (3 - pa), 0, 1), acc | (kk > 0));
       });
     ok = mma_done();
-    float t[32];
+    float t[32], t1[32];
+    tmem_ld32f(lane_tm + kColT + 64 + 32 * half, t1);
+    tmem_wait32(t1);
+    tmem_ld32f(lane_tm + kColT + 128 + 32 * half, t);
+    tmem_wait32(t);
+#pragma unroll
+    for (int e = 0; e < 32; ++e) t1[e] += t[e];
     tmem_ld32f(lane_tm + kColT + 32 * half, t);
     tmem_wait32(t);
     float rho2 = 0.f;
 #pragma unroll
     for (int e = 0; e < 32; ++e) {
-      if ((fixed >> e & 1) || 32 * half + e >= nc) t[e] = 0.f;
+      t[e] = (fixed >> e & 1) || 32 * half + e >= nc ? 0.f : t[e] + t1[e];
       rho2 = fmaf(X[e], t[e], rho2);
     }
     send_row(rho2, &x.rho2[0][0], &x.ex_rho2, sum2);
