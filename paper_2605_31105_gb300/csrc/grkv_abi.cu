@@ -124,6 +124,8 @@ int make_shape(const grkv_params* p, Shape* s) {
   s->steps = p->steps;
   s->step_tol = p->step_tol;
   s->lambda_k = p->lambda_k;
+  s->units = nullptr;
+  s->rows = 0;
   return GRKV_OK;
 }
 

@@ -17,6 +17,13 @@ constexpr int kMaxScoreCtas = 256;  // persistent score grid bound used to size 
 constexpr int kMaxCgIters = 4096;   // bound on the key step's conjugate-gradient iterations
 constexpr int kMaxSteps = 64;       // bound on the alternating steps S
 
+// A unit's budget when units have their own (grkv_compress_ragged): retained
+// tokens, score-ranked fixed tokens, and its first row of the packed outputs.
+struct UnitRow {
+  int32_t B, n_fix;
+  int64_t off;
+};
+
 // Validated problem sizes, derived once on the host.
 struct Shape {
   int U, g, n, d, w, B, m;
@@ -37,7 +44,13 @@ struct Shape {
   float lambda_k; // ridge weight of the key step
   int steps;      // S alternating value / key steps (Algorithm 1)
   float step_tol; // stop once max |K^(t+1) - K^(t)|, max |V^(t+1) - V^(t)| <= step_tol
+  const UnitRow* units;  // device table [U], or null: every unit has B, n_fix and row u B
+  size_t rows;           // with a table: rows of the packed outputs
 };
+
+__device__ inline UnitRow unit_row(const UnitRow* units, int u, int B, int n_fix) {
+  return units ? units[u] : UnitRow{B, n_fix, (int64_t)u * B};
+}
 
 // Byte offsets of the workspace regions (each 256-B aligned).
 struct WsLayout {

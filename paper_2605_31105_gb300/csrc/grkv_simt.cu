@@ -1,5 +1,4 @@
-// Window scoring on CUDA cores (fp32 inputs, and bf16 under GRKV_FORCE_SIMT),
-// and the selection kernels of every path.
+// Window scoring on CUDA cores (fp32 inputs, and bf16 under GRKV_FORCE_SIMT).
 //
 // Every logit is an fp32 FMA chain over the head dimension, probabilities use
 // expf and an IEEE divide, and every reduction runs in a fixed order, so
@@ -8,7 +7,6 @@
 #include <cmath>
 #include <type_traits>
 
-#include "block_select.cuh"
 #include "simt_common.cuh"
 
 namespace grkv {
@@ -289,283 +287,6 @@ __global__ void __launch_bounds__(256) k_y_reduce(const float4* __restrict__ ypa
   y[(size_t)u * md + i] = a;
 }
 
-// ------------------------------------------------------------- selection --
-__global__ void __launch_bounds__(1024) k_select(const float* __restrict__ scores, Shape s,
-                                                 float* __restrict__ pooled,
-                                                 int32_t* __restrict__ idx) {
-  __shared__ int hist[256];
-  __shared__ int sh[48];
-  const int u = blockIdx.x, tid = threadIdx.x, P = s.P, h = s.pool_k / 2;
-  const float* c = scores + (size_t)u * P;
-  float* pl = pooled + (size_t)u * P;
-  int32_t* out = idx + (size_t)u * s.B;
-  // four positions per step, the neighbour offset outermost, so that each
-  // step's loads are independent of one another
-  for (int j0 = tid; j0 < P; j0 += 4 * blockDim.x) {
-    int j[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) j[q] = j0 + q * blockDim.x;
-    if (s.pool_type == GRKV_POOL_MAX) {
-      float mx[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) mx[q] = j[q] < P ? c[j[q]] : 0.f;
-      for (int t = 1; t <= h; ++t) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (j[q] >= P) continue;
-          if (j[q] - t >= 0) mx[q] = fmaxf(mx[q], c[j[q] - t]);
-          if (j[q] + t < P) mx[q] = fmaxf(mx[q], c[j[q] + t]);
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (j[q] < P) pl[j[q]] = mx[q];
-    } else {
-      double a[4] = {0.0, 0.0, 0.0, 0.0};   // left to right, zero padding, divisor k
-      for (int t = -h; t <= h; ++t) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (j[q] < P && j[q] + t >= 0 && j[q] + t < P) a[q] += (double)c[j[q] + t];
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (j[q] < P) pl[j[q]] = (float)(a[q] / (double)s.pool_k);
-    }
-  }
-  __syncthreads();
-  if (s.kk >= P) {
-    for (int j = tid; j < P; j += blockDim.x) out[j] = j;
-  } else if (s.kk > 0) {
-    auto get = [&](int i, uint32_t* key) {
-      *key = order_key(pl[i]);
-      return true;
-    };
-    // positions: count the marks of earlier segments first
-    const int seg = (P + blockDim.x - 1) / blockDim.x;
-    const int lo = min(P, tid * seg), hi = min(P, lo + seg);
-    uint32_t tau;
-    int need_eq;
-    block_kth_largest(get, P, s.kk, hist, sh, &tau, &need_eq);
-    // the segment's keys in chunks of eight loaded together
-    auto seg_keys = [&](int i0, uint32_t* kk) {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) kk[q] = i0 + q < hi ? order_key(pl[i0 + q]) : 0u;
-    };
-    int eq = 0;
-    for (int i0 = lo; i0 < hi; i0 += 8) {
-      uint32_t kk[8];
-      seg_keys(i0, kk);
-#pragma unroll
-      for (int q = 0; q < 8; ++q) eq += (i0 + q < hi && kk[q] == tau);
-    }
-    int tot;
-    const int er0 = block_exclusive_scan(eq, sh + 8, &tot);
-    int sel = 0, er = er0;
-    for (int i0 = lo; i0 < hi; i0 += 8) {
-      uint32_t kk[8];
-      seg_keys(i0, kk);
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        if (i0 + q >= hi) continue;
-        if (kk[q] > tau) {
-          ++sel;
-        } else if (kk[q] == tau) {
-          if (er < need_eq) ++sel;
-          ++er;
-        }
-      }
-    }
-    int pos = block_exclusive_scan(sel, sh + 8, &tot);
-    er = er0;
-    for (int i0 = lo; i0 < hi; i0 += 8) {
-      uint32_t kk[8];
-      seg_keys(i0, kk);
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        if (i0 + q >= hi) continue;
-        if (kk[q] > tau) {
-          out[pos++] = i0 + q;
-        } else if (kk[q] == tau) {
-          if (er < need_eq) out[pos++] = i0 + q;
-          ++er;
-        }
-      }
-    }
-  }
-  for (int a = tid; a < s.w; a += blockDim.x) out[s.kk + a] = P + a;
-}
-
-// Selection with the unit's keys resident in shared memory (n - w <= 32768):
-// one 1024-thread CTA per unit.  The scores are staged once; thread t owns the
-// 32 contiguous positions 32t .. 32t+31 and pools them into order-preserving
-// keys held in its registers (max pooling of width 7 as a sliding window over
-// the 38 scores around the segment); the (B - w)-th largest key is found by
-// four 8-bit radix passes over per-warp histograms, and the positions are
-// compacted in order from the same segments.  Same result as k_select.
-// Shared-memory words are padded by one per 32 (index j + j / 32) so that
-// both the strided staging and the segment reads are free of bank conflicts.
-constexpr int kSelThreads = 1024, kSelPer = 32, kSelMaxP = kSelThreads * kSelPer;
-
-__host__ __device__ __forceinline__ int sel_pad(int j) { return j + (j >> 5); }
-
-size_t select_smem_bytes(int P) {
-  return ((size_t)sel_pad(P) + 4) * 4 + (size_t)32 * 256 * 4;
-}
-
-__global__ void __launch_bounds__(kSelThreads, 1) k_select_smem(const float* __restrict__ scores,
-                                                                Shape s,
-                                                                int32_t* __restrict__ idx) {
-  extern __shared__ uint32_t skey[];   // [sel_pad(P)] scores, then keys
-  __shared__ int hist[256];
-  __shared__ int sh[48];
-  const int u = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int P = s.P, h = s.pool_k / 2;
-  int* whist = (int*)(skey + ((sel_pad(P) + 4) & ~3));   // [32][256]
-  const float* c = scores + (size_t)u * P;
-  int32_t* out = idx + (size_t)u * s.B;
-#pragma unroll 8
-  for (int e = 0; e < kSelPer; ++e) {
-    const int j = tid + e * kSelThreads;
-    if (j < P) skey[sel_pad(j)] = __float_as_uint(__ldg(c + j));
-  }
-  __syncthreads();
-  auto cs = [&](int j) { return __uint_as_float(skey[sel_pad(j)]); };
-  const int lo = tid * kSelPer;   // this thread's segment lo .. lo + 31
-  uint32_t kr[kSelPer];
-  if (s.pool_type == GRKV_POOL_MAX && h == 3) {
-    // w[i] = score at lo - 3 + i (cells outside [0, P) are ignored: -inf);
-    // the window max over w[e .. e + 6] from pairs and quadruples
-    float w[kSelPer + 6];
-#pragma unroll
-    for (int i = 0; i < kSelPer + 6; ++i) {
-      const int j = lo - 3 + i;
-      w[i] = (j >= 0 && j < P) ? cs(j) : -INFINITY;
-    }
-    float m2[kSelPer + 5], m4[kSelPer + 3];
-#pragma unroll
-    for (int i = 0; i < kSelPer + 5; ++i) m2[i] = fmaxf(w[i], w[i + 1]);
-#pragma unroll
-    for (int i = 0; i < kSelPer + 3; ++i) m4[i] = fmaxf(m2[i], m2[i + 2]);
-#pragma unroll
-    for (int e = 0; e < kSelPer; ++e)
-      kr[e] = lo + e < P ? order_key(fmaxf(fmaxf(m4[e], m2[e + 4]), w[e + 6])) : 0u;
-  } else {
-#pragma unroll
-    for (int e = 0; e < kSelPer; ++e) {
-      const int j = lo + e;
-      kr[e] = 0u;
-      if (j < P) {
-        float pv;
-        if (s.pool_type == GRKV_POOL_MAX) {
-          pv = cs(j);
-          for (int t = 1; t <= h; ++t) {
-            if (j - t >= 0) pv = fmaxf(pv, cs(j - t));
-            if (j + t < P) pv = fmaxf(pv, cs(j + t));
-          }
-        } else {
-          double acc = 0.0;   // left to right, zero padding, divisor k
-          for (int t = -h; t <= h; ++t)
-            if (j + t >= 0 && j + t < P) acc += (double)cs(j + t);
-          pv = (float)(acc / (double)s.pool_k);
-        }
-        kr[e] = order_key(pv);
-      }
-    }
-  }
-  if (s.kk >= P) {
-    for (int j = tid; j < P; j += kSelThreads) out[j] = j;
-  } else if (s.kk > 0) {
-    // (kk)-th largest key: four 8-bit digits, most significant first
-    uint32_t prefix = 0, mask = 0;
-    int rem = s.kk;
-    for (int shift = 24; shift >= 0; shift -= 8) {
-      for (int i = tid; i < 32 * 256; i += kSelThreads) whist[i] = 0;
-      __syncthreads();
-#pragma unroll
-      for (int e = 0; e < kSelPer; ++e) {
-        if (lo + e < P && (kr[e] & mask) == prefix)
-          atomicAdd(&whist[warp * 256 + ((kr[e] >> shift) & 255u)], 1);
-      }
-      __syncthreads();
-      if (tid < 256) {
-        int a = 0;
-#pragma unroll 8
-        for (int w = 0; w < 32; ++w) a += whist[w * 256 + tid];
-        hist[tid] = a;
-      }
-      __syncthreads();
-      if (warp == 0) {
-        // digit search from 255 down: lane l owns bins 8l..8l+7
-        int cnt[8], own = 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          cnt[q] = hist[8 * lane + q];
-          own += cnt[q];
-        }
-        int suf = own;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_down_sync(0xffffffffu, suf, o);
-          if (lane + o < 32) suf += y;
-        }
-        int above = suf - own, dg = -1, left = 0;
-#pragma unroll
-        for (int q = 7; q >= 0; --q) {
-          if (dg < 0 && (above + cnt[q] >= rem || (lane == 0 && q == 0))) {
-            dg = 8 * lane + q;
-            left = rem - above;
-          }
-          above += cnt[q];
-        }
-        const unsigned found = __ballot_sync(0xffffffffu, dg >= 0);
-        const int srcl = 31 - __clz(found);
-        const int dsel = __shfl_sync(0xffffffffu, dg, srcl), lsel = __shfl_sync(0xffffffffu, left, srcl);
-        if (lane == 0) {
-          sh[0] = dsel;
-          sh[1] = lsel;
-        }
-      }
-      __syncthreads();
-      prefix |= (uint32_t)sh[0] << shift;
-      mask |= 255u << shift;
-      rem = sh[1];
-      __syncthreads();
-    }
-    const uint32_t tau = prefix;
-    const int need_eq = rem;
-    // compaction in position order over the same segments
-    int eq = 0;
-#pragma unroll
-    for (int e = 0; e < kSelPer; ++e) eq += (lo + e < P && kr[e] == tau);
-    int tot;
-    const int er0 = block_exclusive_scan(eq, sh + 8, &tot);
-    int sel = 0, er = er0;
-#pragma unroll
-    for (int e = 0; e < kSelPer; ++e) {
-      if (lo + e >= P) continue;
-      if (kr[e] > tau) {
-        ++sel;
-      } else if (kr[e] == tau) {
-        if (er < need_eq) ++sel;
-        ++er;
-      }
-    }
-    int pos = block_exclusive_scan(sel, sh + 8, &tot);
-    er = er0;
-#pragma unroll
-    for (int e = 0; e < kSelPer; ++e) {
-      if (lo + e >= P) continue;
-      if (kr[e] > tau) {
-        out[pos++] = lo + e;
-      } else if (kr[e] == tau) {
-        if (er < need_eq) out[pos++] = lo + e;
-        ++er;
-      }
-    }
-  }
-  for (int a = tid; a < s.w; a += kSelThreads) out[s.kk + a] = P + a;
-}
-
 template <typename T, int RT>
 cudaError_t score_impl(const Shape& s, const T* q, const T* k, const T* v, float* scores,
                        float* y, float* row_stats, char* ws, const WsLayout& L,
@@ -626,28 +347,6 @@ int score_simt_chunk(const Shape& s) {
     }
   }
   return (int)best * kKeys;
-}
-
-bool select_uses_pooled_buffer(const Shape& s) { return s.P > kSelMaxP; }
-
-cudaError_t launch_select_pooled(const Shape& s, const float* scores, int32_t* idx,
-                                 float* pooled, cudaStream_t st) {
-  if (!select_uses_pooled_buffer(s)) {
-    const size_t bytes = select_smem_bytes(s.P);
-    cudaError_t e =
-        cudaFuncSetAttribute(k_select_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e != cudaSuccess) return e;
-    k_select_smem<<<s.U, kSelThreads, bytes, st>>>(scores, s, idx);
-  } else {
-    k_select<<<s.U, 1024, 0, st>>>(scores, s, pooled, idx);
-  }
-  count_launches(1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_select(const Shape& s, const float* scores, int32_t* idx, char* ws,
-                          const WsLayout& L, cudaStream_t st) {
-  return launch_select_pooled(s, scores, idx, (float*)(ws + L.pooled), st);
 }
 
 }  // namespace grkv
