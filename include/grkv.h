@@ -196,8 +196,9 @@ int grkv_compress(const grkv_params* p, const void* q, const void* k, const void
  * Outputs are packed: unit u's budgets[u] entries of idx and rows of k_out /
  * v_out start at row off_u = budgets[0] + ... + budgets[u-1] (idx [sum B_u]
  * int32, k_out / v_out [sum B_u][d]); each unit's results are those of
- * grkv_compress with B = budgets[u].  The scoring step runs once over all
- * units; selection and the value (and key) step run once per run of
+ * grkv_compress with B = budgets[u].  The scoring step, and on the
+ * tensor-core value step the selection and the merge, run once over all
+ * units; the portable value step and the key step run once per run of
  * consecutive units with equal budgets.  ws must hold
  * grkv_compress_ragged_workspace_size bytes; device errors of any run go to
  * its status word (grkv_status). */

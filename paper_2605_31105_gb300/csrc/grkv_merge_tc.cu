@@ -27,6 +27,7 @@
 //
 // The kernels rely on the idx contract of grkv.h: ascending, with the window
 // n-w..n-1 in the last w slots.
+#include <algorithm>
 #include <cmath>
 
 #include "block_select.cuh"
@@ -45,6 +46,7 @@ constexpr int kThreads = 384;    // k_merge_gram
 constexpr int kThreadsU = 736;   // k_merge_update
 constexpr uint32_t kTileBytes = kTile * kD * 2;   // 32 KB
 constexpr int kMaxB = 32768;
+constexpr int kSms = 152;        // SMs of a GB300
 constexpr long long kBudget = 1ll << 32;
 
 // Shared memory (offsets from a 1024-byte aligned base).  k_merge_gram: Q, a
@@ -92,6 +94,8 @@ struct MArgs {
   int upd_mode;              // update: 0 V_out = V0 + dV; 1 vpart = V0 + dV; 2 V_out = vpart + dV
   float* vpart;              // [U][B][128] fp32, between the update's two row blocks
   int* status;
+  const UnitRow* units;      // budgets of the units, or null (B each)
+  int split;                 // update: CTAs per unit
 };
 
 struct MBars {
@@ -322,8 +326,10 @@ __global__ void __launch_bounds__(256) k_merge_fixed(MArgs a) {
   extern __shared__ uint32_t fkey[];   // [B] candidate keys, 0 = not a candidate
   __shared__ int hist[256], sh[64];
   const int tid = threadIdx.x, nt = blockDim.x;
-  const int u = blockIdx.x, B = a.B;
-  const int32_t* idx_u = a.idx + (size_t)u * B;
+  const int u = blockIdx.x;
+  const UnitRow ur = unit_row(a.units, u, a.B, a.n_fix);
+  const int B = ur.B;
+  const int32_t* idx_u = a.idx + ur.off;
   const float* sc_u = a.scores + (size_t)u * a.P;
   // Candidates for the score-ranked part: retained prefix tokens past the sinks.
   // Their scores are non-negative, so every key is above 0.
@@ -343,7 +349,7 @@ __global__ void __launch_bounds__(256) k_merge_fixed(MArgs a) {
   __syncthreads();
   int ncand;
   (void)block_exclusive_scan(nc, sh + 8, &ncand);
-  const int nf = min(a.n_fix, ncand);
+  const int nf = min(ur.n_fix, ncand);
   uint32_t tau = 0xFFFFFFFFu;
   int need_eq = 0;
   if (nf > 0) {
@@ -366,7 +372,7 @@ __global__ void __launch_bounds__(256) k_merge_fixed(MArgs a) {
     bool fixed = kx == 0u || kx > tau;
     if (kx == tau) fixed = er++ < need_eq;
     fkey[i] = fixed ? 1u : 0u;   // each thread rewrites only its own segment
-    a.fixed[(size_t)u * B + i] = fixed ? 1 : 0;
+    a.fixed[ur.off + i] = fixed ? 1 : 0;
     keep += !fixed;
   }
   int ng;
@@ -375,7 +381,7 @@ __global__ void __launch_bounds__(256) k_merge_fixed(MArgs a) {
   for (int i = lo; i < hi; ++i) {
     const int at = fkey[i] ? ng + (i - g) : g;
     g += !fkey[i];
-    a.src[(size_t)u * B + at] = pos(i);
+    a.src[ur.off + at] = pos(i);
   }
   if (tid == 0) a.ng[u] = ng;
 }
@@ -401,7 +407,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint8_t* sm = (uint8_t*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
   MBars* bars = (MBars*)(sm + kOffBar);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int u = blockIdx.x, B = a.B, T = (B + kTile - 1) / kTile;
+  const int u = blockIdx.x;
+  const UnitRow ur = unit_row(a.units, u, a.B, a.n_fix);
+  const int B = ur.B, T = (B + kTile - 1) / kTile;
   if (a.gram_mode == 2 && __ldg(a.redo + u * a.nrb + a.rb) == 0) return;   // the single pass was valid
   const bool single = a.gram_mode == 1;
   const int k0 = single ? T : 0;   // first job
@@ -422,8 +430,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
     // the gathers: warps 0, 2 and 3 (three SM sub-partitions)
-    const int32_t* idx_u = a.idx + (size_t)u * B;
-    const int32_t* src_u = a.src + (size_t)u * B;
+    const int32_t* idx_u = a.idx + ur.off;
+    const int32_t* src_u = a.src + ur.off;
     const int row0 = u * a.n;   // first row of this unit in the 2-D K / V maps
     const int pw = warp == 0 ? 0 : warp - 1;
     Gatherer<kRingG, 3> gt{sm + kOffRing, bars->ring_full, bars->ring_empty};
@@ -729,7 +737,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint8_t* xgh = sm + kOffXhC;
   uint8_t* xgl = sm + kOffXlC;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int u = blockIdx.x, B = a.B;
+  const int u = blockIdx.x;
+  const UnitRow ur = unit_row(a.units, u, a.B, a.n_fix);
+  const int B = ur.B;
   const int ng = __ldg(a.ng + u), TG = (ng + kTile - 1) / kTile;
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) {
@@ -766,7 +776,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
     __syncwarp();
-    const int32_t* src_u = a.src + (size_t)u * B;
+    const int32_t* src_u = a.src + ur.off;
     const int pw = warp == 0 ? 0 : warp - 1;
     Gatherer<2, 3> gt{sm + kOffRingC, bars->ring_full, bars->ring_empty};
     int jn[4];
@@ -888,7 +898,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // ======================================================== k_merge_update
-// Slot order, one unit per CTA, 736 threads.  Roles: warp 0 the Q load and
+// Slot order, a unit's tiles over `split` CTAs, 736 threads.  Roles: warp 0 the Q load and
 // the K_out tile stores, warp 22 the V_out tile stores; warp 1 MMA issue;
 // warps 2, 3, 16, 17 the K0 gathers and 18-21 the V0 gathers (two-slot rings
 // each, on all four SM sub-partitions); warps 4-7 and 8-11
@@ -915,6 +925,16 @@ constexpr uint32_t kOffLamU = kOffBar + 256;               // [128] row normalis
 static_assert(kOffZU + 2 * kTileBytes == kOffBar, "update shared-memory layout");
 constexpr uint32_t kSmemBytesU = kOffLamU + kRows * 4 + 1024;
 
+// The first `rows` rows of a swizzled tile to consecutive rows of an output, by one warp.
+__device__ __forceinline__ void copy_rows(__nv_bfloat16* dst, const uint8_t* tile, int rows, int lane) {
+#pragma unroll 4
+  for (int i = lane; i < rows * 16; i += 32) {
+    const int r = i >> 4, c = i & 15;
+    *(uint4*)(dst + (size_t)r * kD + c * 8) =
+        *(const uint4*)(tile + (c >> 3) * (kTileBytes / 2) + sw128_offset(r, c & 7));
+  }
+}
+
 __global__ void __launch_bounds__(kThreadsU, 1)
     k_merge_update(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                    const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmKo,
@@ -926,8 +946,18 @@ __global__ void __launch_bounds__(kThreadsU, 1)
   uint8_t* zh = sm + kOffZU;
   uint8_t* zl = zh + kTileBytes;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int u = blockIdx.x, B = a.B, T = (B + kTile - 1) / kTile;
-  const int32_t* idx_u = a.idx + (size_t)u * B;
+  // the CTA's tiles T0 .. T0 + T - 1 of the unit (`split` CTAs per unit)
+  const int u = blockIdx.x / a.split, part = blockIdx.x - u * a.split;
+  const UnitRow ur = unit_row(a.units, u, a.B, a.n_fix);
+  const int B = ur.B, Tu = (B + kTile - 1) / kTile;
+  const int T0 = (int)((long long)part * Tu / a.split);
+  const int T = (int)((long long)(part + 1) * Tu / a.split) - T0, S0 = T0 * kTile;
+  const int32_t* idx_u = a.idx + ur.off;
+  // packed outputs (budgets of their own): tiles are addressed by row, and a unit's last,
+  // partial tile is copied by a warp so that it ends where the next unit's rows begin
+  const bool packed = a.units != nullptr;
+  const int out_y = packed ? (int)ur.off + S0 : S0, out_z = packed ? 0 : u;
+  const int t_part = packed && S0 + T * kTile > B ? T - 1 : -1;   // the partial tile, if any
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bars->k_full[i], 4);    // one expect_tx arrival per gathering warp
@@ -991,10 +1021,10 @@ __global__ void __launch_bounds__(kThreadsU, 1)
         const int sl = t & 1;
         ok = mbar_wait(&bars->k_full[sl], (t >> 1) & 1, abort_flag, kBudget);
         if (!ok) break;
-        if (a.upd_mode != 2) {   // the second row block's K_out is the first's
+        if (a.upd_mode != 2 && t != t_part) {   // the second row block's K_out is the first's
           const uint8_t* kt = sm + kOffKU + sl * kTileBytes;
-          tma_store_3d(&tmKo, kt, 0, t * kTile, u);
-          tma_store_3d(&tmKo, kt + kTileBytes / 2, 64, t * kTile, u);
+          tma_store_3d(&tmKo, kt, 0, out_y + t * kTile, out_z);
+          tma_store_3d(&tmKo, kt + kTileBytes / 2, 64, out_y + t * kTile, out_z);
           bulk_commit();
           bulk_wait_read<0>();
         }
@@ -1003,6 +1033,11 @@ __global__ void __launch_bounds__(kThreadsU, 1)
       bulk_wait_all();
       if (!ok) set_status(a.status, GRKV_ERR_TIMEOUT);
     }
+    __syncwarp();
+    if (t_part >= 0 && a.upd_mode != 2 &&
+        mbar_wait_warp(&bars->k_full[t_part & 1], (t_part >> 1) & 1, abort_flag))
+      copy_rows(a.k_out + (ur.off + S0 + (size_t)t_part * kTile) * kD,
+                sm + kOffKU + (t_part & 1) * kTileBytes, B - S0 - t_part * kTile, lane);
   } else if (warp == 22) {
     if (lane == 0) {
       prefetch_tensormap(&tmVo);
@@ -1012,10 +1047,10 @@ __global__ void __launch_bounds__(kThreadsU, 1)
         const int sl = t & 1;
         ok = mbar_wait(&bars->vo_full[sl], (t >> 1) & 1, abort_flag, kBudget);
         if (!ok) break;
-        if (a.upd_mode != 1) {   // mode 1 leaves its result in vpart
+        if (a.upd_mode != 1 && t != t_part) {   // mode 1 leaves its result in vpart
           const uint8_t* vt = sm + kOffVU + sl * kTileBytes;
-          tma_store_3d(&tmVo, vt, 0, t * kTile, u);
-          tma_store_3d(&tmVo, vt + kTileBytes / 2, 64, t * kTile, u);
+          tma_store_3d(&tmVo, vt, 0, out_y + t * kTile, out_z);
+          tma_store_3d(&tmVo, vt + kTileBytes / 2, 64, out_y + t * kTile, out_z);
           bulk_commit();
           bulk_wait_read<0>();
         }
@@ -1024,6 +1059,11 @@ __global__ void __launch_bounds__(kThreadsU, 1)
       bulk_wait_all();
       if (!ok) set_status(a.status, GRKV_ERR_TIMEOUT);
     }
+    __syncwarp();
+    if (t_part >= 0 && a.upd_mode != 1 &&
+        mbar_wait_warp(&bars->vo_full[t_part & 1], (t_part >> 1) & 1, abort_flag))
+      copy_rows(a.v_out + (ur.off + S0 + (size_t)t_part * kTile) * kD,
+                sm + kOffVU + (t_part & 1) * kTileBytes, B - S0 - t_part * kTile, lane);
   } else if (warp == 2 || warp == 3 || (warp >= 16 && warp < 22)) {
     // K0 gathers: warps 2, 3, 16, 17; V0 gathers: warps 18 - 21 (own rings, so
     // that a K tile never waits for a V slot)
@@ -1035,11 +1075,11 @@ __global__ void __launch_bounds__(kThreadsU, 1)
                      is_v ? bars->v_empty : bars->k_empty};
     const CUtensorMap* map = is_v ? &tmV : &tmK;
     int jn[4];
-    if (TG > 0) g.rows(idx_u, B, a.n, row0, 0, pw, lane, jn);
+    if (TG > 0) g.rows(idx_u, B, a.n, row0, T0, pw, lane, jn);
     bool ok = true;
     for (int t = 0; t < TG && ok; ++t) {
       const int j[4] = {jn[0], jn[1], jn[2], jn[3]};
-      if (t + 1 < TG) g.rows(idx_u, B, a.n, row0, t + 1, pw, lane, jn);
+      if (t + 1 < TG) g.rows(idx_u, B, a.n, row0, T0 + t + 1, pw, lane, jn);
       ok = g.load(map, j, pw, lane, abort_flag);
     }
     g.drain(abort_flag);
@@ -1097,8 +1137,8 @@ __global__ void __launch_bounds__(kThreadsU, 1)
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
     bool ok = true;
     for (int t = cg; t < T && ok; t += 2) {
-      const int sl = t & 1, slot = t * kTile + tok;
-      const bool zero = slot >= B || __ldg(a.fixed + (size_t)u * B + min(slot, B - 1)) != 0;
+      const int sl = t & 1, slot = S0 + t * kTile + tok;
+      const bool zero = slot >= B || __ldg(a.fixed + ur.off + min(slot, B - 1)) != 0;
       ok = mbar_wait_warp(&bars->s_full[sl], (t >> 1) & 1, abort_flag);
       if (!ok) break;
       tc_fence_after();
@@ -1136,9 +1176,9 @@ __global__ void __launch_bounds__(kThreadsU, 1)
     const int mode = a.upd_mode;
     bool ok = true;
     for (int t = 0; t < T && ok; ++t) {
-      const int sl = t & 1, slot = t * kTile + tok;
+      const int sl = t & 1, slot = S0 + t * kTile + tok;
       const bool in = slot < B;
-      const bool live = in && (mode != 0 || __ldg(a.fixed + (size_t)u * B + min(slot, B - 1)) == 0);
+      const bool live = in && (mode != 0 || __ldg(a.fixed + ur.off + min(slot, B - 1)) == 0);
       ok = mbar_wait_warp(&bars->d_full[sl], (t >> 1) & 1, abort_flag);
       if (ok && mode != 2) ok = mbar_wait_warp(&bars->v_full[sl], (t >> 1) & 1, abort_flag);
       if (ok && mode == 2 && t >= 2)
@@ -1147,7 +1187,7 @@ __global__ void __launch_bounds__(kThreadsU, 1)
       tc_fence_after();
       uint8_t* vt = sm + kOffVU + sl * kTileBytes;
       const uint32_t dcol = lane_addr + kColD + sl * kD;
-      float* vp = mode != 0 ? a.vpart + ((size_t)u * B + min(slot, B - 1)) * kD : nullptr;
+      float* vp = mode != 0 ? a.vpart + (ur.off + min(slot, B - 1)) * kD : nullptr;
 #pragma unroll 1
       for (int c = 0; c < 4; ++c) {
         float dv[32];
@@ -1246,8 +1286,8 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
   if (!encode_bf16_3d(&mq, q, kD, s.m, s.U, 64, kRows) ||
       !encode_bf16_2d_rows(&mk, k, kD, (uint64_t)s.U * s.n) ||
       !encode_bf16_2d_rows(&mv, v, kD, (uint64_t)s.U * s.n) ||
-      !encode_bf16_3d(&mko, k_out, kD, s.B, s.U, 64, kTile) ||
-      !encode_bf16_3d(&mvo, v_out, kD, s.B, s.U, 64, kTile))
+      !encode_bf16_3d(&mko, k_out, kD, s.units ? s.rows : s.B, s.units ? 1 : s.U, 64, kTile) ||
+      !encode_bf16_3d(&mvo, v_out, kD, s.units ? s.rows : s.B, s.units ? 1 : s.U, 64, kTile))
     return cudaErrorInvalidValue;
   MArgs a{};
   a.U = s.U;
@@ -1283,6 +1323,9 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
   a.ldr = W.ldr;
   a.nrb = W.nrb;
   a.status = (int*)(ws + L.status);
+  a.units = s.units;
+  // a unit's update tiles are independent: few units spread over the SMs
+  a.split = std::max(1, std::min(kSms / std::max(s.U, 1), (s.B + kTile - 1) / kTile));
   cudaError_t e;
   if ((e = cudaFuncSetAttribute(k_merge_gram, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 kSmemBytes)) != cudaSuccess ||
@@ -1328,7 +1371,7 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
     a.rb = 0;
     a.row0 = 0;
     a.upd_mode = 0;
-    k_merge_update<<<s.U, kThreadsU, kSmemBytesU, st>>>(mq, mk, mv, mko, mvo, a);
+    k_merge_update<<<s.U * a.split, kThreadsU, kSmemBytesU, st>>>(mq, mk, mv, mko, mvo, a);
     launches = 1;
   } else {
     // the value update of each row block (the first leaves V0 + dV_0 in vpart)
@@ -1337,7 +1380,7 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
       a.rb = rb;
       a.row0 = rb * kRows;
       a.upd_mode = rb == 0 ? 1 : 2;
-      k_merge_update<<<s.U, kThreadsU, kSmemBytesU, st>>>(mq, mk, mv, mko, mvo, a);
+      k_merge_update<<<s.U * a.split, kThreadsU, kSmemBytesU, st>>>(mq, mk, mv, mko, mvo, a);
       launches += 1;
     }
   }

@@ -1,13 +1,19 @@
 // Per-unit budgets: grkv_compress with a budget B_u for every unit, as the
 // paper pairs GRKV with layer-wise (PyramidKV) and head-wise (Ada-KV) budget
 // allocations (Sec. 4.2).  The scoring step does not depend on the budget and
-// runs once over all units; selection and the value (and key) step run once
-// per run of consecutive units that share a budget, on that run's slice of
-// the inputs, each with the same kernels as grkv_compress.  Outputs are
-// packed: unit u's B_u rows start at row off_u = B_0 + ... + B_{u-1}.
+// runs once over all units.  Outputs are packed: unit u's B_u rows start at
+// row off_u = B_0 + ... + B_{u-1}.
+//
+// On the tensor-core value step, selection and merge also run once over all
+// units, each unit at its budget from a device table (k_unit_table): one launch
+// each, whatever the budgets, where a launch per run of equal budgets left 8
+// units on 152 SMs (eight runs of 8 units, n = 16384: 1.59 ms).  The portable value
+// step and the key step run once per run of consecutive units that share a
+// budget, on that run's slice of the inputs.
 #include <algorithm>
 #include <vector>
 
+#include "block_select.cuh"
 #include "grkv_internal.cuh"
 
 namespace grkv {
@@ -22,7 +28,27 @@ __global__ void k_status_merge(int* status, const int* run_status) {
   if (s != 0) atomicCAS(status, 0, s);
 }
 
+// The table rows of up to kChunkUnits units.  Budgets travel as a kernel
+// argument: a captured graph then holds no pointer to the caller's host array.
+constexpr int kChunkUnits = 960;
+struct BudgetChunk {
+  int count, first;
+  int64_t off;                 // packed row of the chunk's first unit
+  int32_t budget[kChunkUnits];
+};
+__global__ void __launch_bounds__(1024) k_unit_table(const __grid_constant__ BudgetChunk c,
+                                                     float beta, UnitRow* table) {
+  __shared__ int sh[32];
+  const int i = threadIdx.x, b = i < c.count ? c.budget[i] : 0;
+  int total;
+  const int pre = block_exclusive_scan(b, sh, &total);
+  if (i < c.count)
+    table[c.first + i] = {b, (int)floor((double)beta * (double)b), c.off + pre};
+}
+
 struct RaggedPlan {
+  bool once;                  // selection and merge in one launch each
+  size_t table;               // UnitRow [U] (once)
   Shape all;                  // every unit, the largest budget (scoring only)
   std::vector<int> begin;     // first unit of each run
   std::vector<int> budget;    // its budget
@@ -48,13 +74,22 @@ int plan_ragged(const grkv_params* p, const int32_t* budgets, RaggedPlan* r) {
   r->begin.clear();
   r->budget.clear();
   r->off.assign(1, 0);
-  size_t run_total = 0, idx_max = 0;
+  r->main_total = plan_workspace(r->all).total;
+  // packed rows index the output tensor maps; a chunk's scan is 32-bit
+  size_t run_total = 0, idx_max = 0, rows = 0;
+  for (int u = 0; u < p->units; ++u) rows += (size_t)budgets[u];
+  r->once = r->all.tc_merge && !r->all.update_k && rows < ((size_t)1 << 31);
   for (int u = 0; u < p->units; ++u) {
     r->off.push_back(r->off.back() + (size_t)budgets[u]);
     if (u == 0 || budgets[u] != budgets[u - 1]) {
       r->begin.push_back(u);
       r->budget.push_back(budgets[u]);
     }
+  }
+  if (r->once) {
+    r->table = align256(r->main_total);
+    r->total = align256(r->table + (size_t)p->units * sizeof(UnitRow));
+    return GRKV_OK;
   }
   for (size_t i = 0; i < r->begin.size(); ++i) {
     const int u1 = i + 1 < r->begin.size() ? r->begin[i + 1] : p->units;
@@ -66,7 +101,6 @@ int plan_ragged(const grkv_params* p, const int32_t* budgets, RaggedPlan* r) {
     run_total = std::max(run_total, plan_workspace(s).total);
     idx_max = std::max(idx_max, (size_t)s.U * s.B);
   }
-  r->main_total = plan_workspace(r->all).total;
   r->run_ws = align256(r->main_total);
   r->run_total = run_total;
   r->idx_scratch = align256(r->run_ws + run_total);
@@ -118,6 +152,26 @@ extern "C" int grkv_compress_ragged(const grkv_params* p, const int32_t* budgets
   float* y = (float*)(w + L.y);
   float* rstats = (float*)(w + L.rstats);
   if (launch_score_any(s, q, k, v, scores, y, rstats, w, L, st) != cudaSuccess) return GRKV_ERR_CUDA;
+  if (r.once) {
+    UnitRow* table = (UnitRow*)(w + r.table);
+    for (int u0 = 0; u0 < s.U; u0 += kChunkUnits) {
+      BudgetChunk c;
+      c.count = std::min(kChunkUnits, s.U - u0);
+      c.first = u0;
+      c.off = (int64_t)r.off[u0];
+      std::copy(budgets + u0, budgets + u0 + c.count, c.budget);
+      k_unit_table<<<1, 1024, 0, st>>>(c, p->beta, table);
+      count_launches(1);
+    }
+    Shape rs = s;
+    rs.units = table;
+    rs.rows = rows;
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = launch_select(rs, scores, idx, w, L, st);
+    if (e == cudaSuccess)
+      e = launch_merge_any(rs, q, k, v, scores, y, rstats, idx, k_out, v_out, w, L, st);
+    return e == cudaSuccess ? GRKV_OK : GRKV_ERR_CUDA;
+  }
   const size_t es = s.dtype == GRKV_BF16 ? 2 : 4, row_bytes = (size_t)kD * es;
   char* rw = w + r.run_ws;
   int32_t* idx_run = (int32_t*)(w + r.idx_scratch);

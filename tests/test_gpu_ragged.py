@@ -59,3 +59,28 @@ def test_equal_budgets_are_grkv_compress(grkv_lib):
         np.testing.assert_array_equal(iu, idx[u])
         np.testing.assert_array_equal(ku, ko[u])
         np.testing.assert_array_equal(vu, vo[u])
+
+
+@pytest.mark.parametrize("wl,pattern", [
+    (gi.workload(1).replace(units=6, n=1500, budget=0), [32, 33, 127, 128, 129, 640]),
+    (gi.Workload("m256", 3, 4, 1200, 128, 64, 0, 7, 1e-1, "bf16", "spans", 321), [64, 200, 256]),
+    # more units than one chunk of the budget table holds
+    (gi.Workload("many", 965, 1, 150, 128, 8, 0, 5, 1e-2, "bf16", "lowrank", 55), [9, 60, 8, 130]),
+], ids=["tile_edges", "m256", "two_chunks"])
+def test_mixed_budgets_are_grkv_compress_unit_by_unit(grkv_lib, wl, pattern):
+    """Every unit's rows equal grkv_compress's at that unit's budget, bit for bit, and the
+    packed rows of a unit end where the next unit's begin."""
+    budgets = [pattern[u % len(pattern)] for u in range(wl.units)]
+    c = G.Case(wl.replace(budget=max(pattern)), units=[u % 7 for u in range(wl.units)])
+    p = G.lib_params(c.wl, c.U)
+    p.flags = b.GRKV_DETERMINISTIC
+    out = _ragged(c, p, budgets)
+    for B in pattern:
+        p.budget = B
+        idx, ko, vo = G.run_compress(c, p)
+        for u in range(c.U):
+            if budgets[u] != B:
+                continue
+            np.testing.assert_array_equal(out[u][0], idx[u])
+            np.testing.assert_array_equal(out[u][1], ko[u])
+            np.testing.assert_array_equal(out[u][2], vo[u])
