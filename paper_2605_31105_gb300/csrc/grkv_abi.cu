@@ -64,7 +64,7 @@ cudaError_t launch_score_any(const Shape& s, const void* q, const void* k, const
                              const WsLayout& L, cudaStream_t st) {
   if (s.tc && s.one_read && !s.deterministic)
     return launch_score_pipe(s, q, k, v, scores, y, row_stats, ws, L, st);
-  if (s.tc) return launch_score_tc(s, q, k, v, scores, y, row_stats, ws, L, 0, st);
+  if (s.tc) return launch_score_tc(s, q, k, v, scores, y, row_stats, ws, L, st);
   return launch_score_simt(s, q, k, v, scores, y, row_stats, ws, L, st);
 }
 
@@ -146,9 +146,8 @@ WsLayout plan_workspace(const Shape& s) {
   };
   L.status = take(256);
   if (s.tc) {
-    int maxc, gu, rounds;
-    L.pstats_tc = take(std::max(score_tc_pstats_bytes(s, &maxc, &gu, &rounds, kMaxScoreCtas),
-                                score_pipe_slot_bytes(s)));
+    int maxc;
+    L.pstats_tc = take(std::max(score_tc_pstats_bytes(s, &maxc), score_pipe_slot_bytes(s)));
     L.flags_tc = take(U * sizeof(int));
     L.lam_tc = take(U * 128 * sizeof(float));
     if (s.deterministic) L.ypart_tc = take(U * (size_t)maxc * m * d * sizeof(float));

@@ -60,8 +60,8 @@ struct WsLayout {
   size_t ypart;   // float  [U][nchunk][m][d]   per-chunk target partials
   int chunk, nchunk;
   // score path (tensor cores)
-  size_t pstats_tc;  // float2 [U][maxc][128] pass-A statistics slots
-  size_t flags_tc;   // int [U] pass-A slots written per unit
+  size_t pstats_tc;  // float2 [U][maxc][128 or 256] pass-A statistics slots
+  size_t flags_tc;   // int [U] pass-A slots written per unit (one-read kernel)
   size_t lam_tc;     // float [U][128] combined log2 row normalisers (one-read scoring)
   size_t ypart_tc;   // float [U][maxc][m][128] segment Y partials (deterministic mode)
   // select
@@ -107,8 +107,8 @@ int score_simt_chunk(const Shape& s);   // keys per CTA of the portable scoring
 cudaError_t launch_select(const Shape& s, const float* scores, int32_t* idx, char* ws,
                           const WsLayout& L, cudaStream_t st);
 // Tensor-core window scoring (bf16, m <= 256 in blocks of 128 rows).  The
-// default, launch_score_tc, runs two launches per row block that each read
-// K; launch_score_pipe (GRKV_ONE_READ_SCORE) reads K once.
+// default, launch_score_tc, runs two launches that each read K;
+// launch_score_pipe (GRKV_ONE_READ_SCORE) reads K once per row block.
 bool score_tc_supported(const Shape& s);
 struct PipePlan {
   int ng, gs;   // CTA groups, CTAs per group
@@ -118,11 +118,11 @@ size_t score_pipe_slot_bytes(const Shape& s);
 cudaError_t launch_score_pipe(const Shape& s, const void* q, const void* k, const void* v,
                               float* scores, float* y, float* row_stats, char* ws,
                               const WsLayout& L, cudaStream_t st);
-size_t score_tc_pstats_bytes(const Shape& s, int* maxc, int* gu, int* rounds, int sms);
+size_t score_tc_pstats_bytes(const Shape& s, int* maxc);   // maxc: slots per unit
 int sm_count();
 cudaError_t launch_score_tc(const Shape& s, const void* q, const void* k, const void* v,
                             float* scores, float* y, float* row_stats, char* ws,
-                            const WsLayout& L, int mode, cudaStream_t st);
+                            const WsLayout& L, cudaStream_t st);
 
 // Tensor-core value merge (bf16, m <= 256 in 128-row blocks, B <= 32768).
 bool merge_tc_supported(const Shape& s);

@@ -195,7 +195,7 @@ cudaError_t score_into(const Shape& s, const void* q, const void* k, const void*
   const WsLayout L = plan_workspace(s);
   float* scores = (float*)(ws - T.score_ws + T.scores);
   float* rstats = (float*)(ws - T.score_ws + T.rstats);
-  if (s.tc) return launch_score_tc(s, q, k, v, scores, y, rstats, ws, L, 0, st);
+  if (s.tc) return launch_score_tc(s, q, k, v, scores, y, rstats, ws, L, st);
   return launch_score_simt(s, q, k, v, scores, y, rstats, ws, L, st);
 }
 
