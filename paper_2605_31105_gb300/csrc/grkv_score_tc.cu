@@ -20,23 +20,31 @@
 // every job, 32 tokens each.  A compute thread owns one window row (one TMEM
 // lane) and one 32-logit chunk of a job, which it copies to registers at once, so
 // that the next S MMA runs under this job's exponentials.  Pass A keeps the row's
-// running max / sum in registers; pass B writes exp2(l - Lambda_r) as bf16 to
-// TMEM columns of its own (the A operand of the Y MMA) and sums probabilities
+// running max / sum in registers; pass B writes exp2(l - Lambda_r) as bf16 over the
+// S columns it came from (the A operand of the Y MMA) and sums probabilities
 // over rows with a warp transpose-reduction.
 //   pass A: warp 2 merges the groups' statistics of each segment (the CTA's
 //           tiles of one unit) into the segment's global slot; warp 3 zeroes Y.
 //   pass B: warp 2 adds the row quarters' sums of every tile and writes the
-//           scores; warps 20-23 combine a unit's slots into log2 normalisers one
-//           segment ahead and add each segment's Y partial to the unit's Y.
+//           scores.  One row block: warps 20-23 combine a unit's slots into log2
+//           normalisers one segment ahead and add each segment's Y partial to the
+//           unit's Y.  Two: the compute threads do both at a segment's ends, and
+//           keep the first block's probabilities in registers until the second's
+//           are there, so that one transpose-reduction serves both.
 //
 // Sixteen compute warps of 32 logits, rather than eight of 64: with two warps per
 // scheduler the chain max -> exponential -> sum was exposed.  Logits are scaled
 // and summed in pairs (fma / add.f32x2), half the issue slots of those steps.
 //
-// Measured, 256 units.  m = 128, n = 32768: pass A 0.300 ms, pass B 0.607 ms, each
-// at 7.1 TB/s of HBM traffic, their bound (eight compute warps: 1.116 ms together).
-// m = 256, n = 131072: pass A 1.94 ms, pass B 4.77 ms, bound by the compute groups
-// (a pair of launches per row block: 8.6 ms together).
+// The MMA warp walks its jobs as a whole and an elected lane issues: with one lane
+// alone, its address arithmetic (it shares a scheduler with four busy warps) took
+// 2.7 K cycles a job and bound both passes of m > 128.
+//
+// Measured, 256 units (eight compute warps and a pair of launches per row block before).
+// m = 128, n = 32768: pass A 0.30 ms, pass B 0.61 ms, at 7.1 TB/s of HBM traffic, their
+// bound (1.116 ms together before).  m = 256, n = 131072: pass A 1.72 ms (4.9 TB/s), pass B
+// 3.17 ms (5.4 TB/s), bound by the latency chains of the compute groups (exponential unit
+// 49% and 27% busy, issue slots 57% and 51%; 8.6 ms together before).
 #include <algorithm>
 #include <cmath>
 
@@ -57,22 +65,28 @@ constexpr uint32_t kTileBytes = kTile * kD * 2;   // 32 KB
 constexpr long long kWaitBudget = 1ll << 32;      // cycles (~2 s) before a wait gives up
 constexpr long long kTestWaitBudget = 1ll << 22;  // ~2 ms: the budget of GRKV_TEST_TIMEOUT
 
-constexpr int score_threads(int pass) { return pass == 0 ? 640 : 768; }
-constexpr int ring_slots(int rb) { return rb == 1 ? 5 : 4; }
+// Pass B over two row blocks: the compute threads, which then have registers for both
+// blocks' probabilities, fetch their own normalisers and add their own Y.
+constexpr int score_threads(int pass, int rb) { return pass == 0 || rb == 2 ? 640 : 768; }
+// K / V tiles in flight.  More is not better: with five, pass B over 256 units n = 32768
+// takes 0.62-0.64 ms instead of 0.61 (HBM serves 152 streams that run further ahead less
+// well); three cost 1%.
+constexpr int kRingSlots = 4;
 
 // Shared-memory layout (offsets from a 1024-byte aligned base): Q, the K / V
 // ring, then one region for pass A's statistics or pass B's sums and normalisers.
 template <int RB>
 struct Layout {
-  static constexpr int kRing = ring_slots(RB);
+  static constexpr int kRing = kRingSlots;
   static constexpr uint32_t kOffQ = 0;                                // RB x 32 KB
   static constexpr uint32_t kOffRing = kOffQ + RB * kTileBytes;       // kRing x 32 KB
   static constexpr uint32_t kOffAux = kOffRing + kRing * kTileBytes;
   // pass A: [2 buf][kGroups][RB][128] float2
   static constexpr uint32_t kAstatBytes = 2 * kGroups * RB * kRows * 8;
-  // pass B: [2 buf][RB][4 row quarters][128] float, then [2 buf][RB][128] float
-  static constexpr uint32_t kRedBytes = 2 * RB * 4 * kTile * 4;
-  static constexpr uint32_t kLamBytes = 2 * RB * kRows * 4;
+  // pass B: [2 buf][4 row quarters][128] float, then the normalisers, [2 buf][128]
+  // float (RB = 1), or the groups' shares of the statistics, [kGroups][256] float2
+  static constexpr uint32_t kRedBytes = 2 * 4 * kTile * 4;
+  static constexpr uint32_t kLamBytes = RB == 1 ? 2 * kRows * 4 : kGroups * RB * kRows * 8;
   static constexpr uint32_t kAuxBytes =
       kAstatBytes > kRedBytes + kLamBytes ? kAstatBytes : kRedBytes + kLamBytes;
   static constexpr uint32_t kOffBar = kOffAux + kAuxBytes;
@@ -80,16 +94,18 @@ struct Layout {
 };
 static_assert(Layout<1>::kSmemBytes <= 227 * 1024 && Layout<2>::kSmemBytes <= 227 * 1024, "smem");
 
-// TMEM columns.  Pass A: four S buffers.  Pass B: one S buffer (free again as soon
-// as the groups have copied it), two P buffers of packed bf16, two Y accumulators
-// (alternate segments of one row block, or the two row blocks).
-constexpr uint32_t kColP = 128, kColY = 256;
-constexpr int s_bufs(int pass) { return pass == 0 ? 4 : 1; }
+// TMEM columns.  Pass A: four S buffers.  Pass B: two S buffers and two Y
+// accumulators (alternate segments of one row block, or the two row blocks); a
+// compute thread writes its 32 probabilities as bf16 pairs over the first 16 of the 32
+// S columns that it has copied to registers.
+constexpr uint32_t kColY = 256;
+constexpr int s_bufs(int pass) { return pass == 0 ? 4 : 2; }
 
 struct Args {
   int U, n, w, m, P, causal;
   int tpu;        // tiles per unit
   int maxc;       // statistics slots per unit
+  int keep_keys;  // pass A leaves its keys in L2 for pass B's reverse sweep
   float sl2;      // scale * log2(e)
   float* scores;   // [U][P]
   float* y;        // [U][m][128], zeroed by pass A
@@ -118,28 +134,47 @@ struct Sched {
   __device__ bool empty(int c) const { return tiles() < G && start(c) == start(c + 1); }
 };
 
-// A CTA's tiles in order.  A segment is the CTA's run of tiles of one unit.
+// A CTA's tiles in order, backwards in pass B (kRev; what pass A read last is read
+// first).  A segment is the CTA's run of tiles of one unit.
+template <bool kRev>
 struct TileIter {
   int tpu, u, ti, left;
   bool begin;
   __device__ TileIter(const Sched& sc, int c) {
-    const long long t0 = sc.start(c);
+    const long long t0 = sc.start(c), t1 = sc.start(c + 1), t = kRev ? t1 - 1 : t0;
     tpu = sc.tpu;
-    left = (int)(sc.start(c + 1) - t0);
-    u = (int)(t0 / tpu);
-    ti = (int)(t0 - (long long)u * tpu);
+    left = (int)(t1 - t0);
+    u = (int)(t / tpu);
+    ti = (int)(t - (long long)u * tpu);
     begin = true;
   }
   __device__ bool more() const { return left > 0; }
-  __device__ bool seg_first() const { return begin || ti == 0; }
-  __device__ bool seg_last() const { return left == 1 || ti == tpu - 1; }
+  __device__ bool seg_first() const { return begin || ti == (kRev ? tpu - 1 : 0); }
+  __device__ bool seg_last() const { return left == 1 || ti == (kRev ? 0 : tpu - 1); }
   __device__ int j0() const { return ti * kTile; }
   __device__ void advance() {
     begin = false;
     --left;
-    if (++ti == tpu) {
+    if (kRev) {
+      if (--ti < 0) {
+        ti = tpu - 1;
+        --u;
+      }
+    } else if (++ti == tpu) {
       ti = 0;
       ++u;
+    }
+  }
+};
+
+// Position in a ring: slot and the parity of its current use.
+struct RingPos {
+  uint32_t slot, phase;
+  __device__ void add(uint32_t k, uint32_t ring) {
+    slot += k;
+    if (slot >= ring) {
+      slot -= ring;
+      phase ^= 1;
     }
   }
 };
@@ -189,14 +224,13 @@ __device__ __forceinline__ void stats_chunk(float* v, bool full, int j0, int lim
     for (int e = 0; e < 32; ++e)
       if (j0 + e > lim || j0 + e >= n) v[e] = -INFINITY;
   }
-  const float vmax = max32(v);
-  if (vmax == -INFINITY) return;
-  const float cm = vmax * sl2;
-  if (cm > M) {
-    L *= fast_exp2(M - cm);
-    M = cm;
-  }
-  const uint64_t s2 = pack2(sl2, sl2), m2 = pack2(-M, -M);
+  // no branch on the maximum: a row that has seen nothing visible yet keeps
+  // M = -inf, L = 0 against the reference 0
+  const float top = fmaxf(M, max32(v) * sl2);
+  const float ref = top == -INFINITY ? 0.f : top;
+  L *= fast_exp2(M - ref);
+  M = top;
+  const uint64_t s2 = pack2(sl2, sl2), m2 = pack2(-ref, -ref);
   uint64_t acc[2] = {0, 0};   // two pairs of zeros
 #pragma unroll
   for (int e = 0; e < 16; ++e) {
@@ -225,8 +259,8 @@ template <int kRing>
 struct Bars {
   uint64_t ring_full[kRing], ring_empty[kRing];
   uint64_t q_full, q_empty;
-  uint64_t s_full[4], s_done[4];            // S written / copied to registers
-  uint64_t p_full[2], p_empty[2];           // P written / read by its Y MMA
+  uint64_t s_full[4], s_done[4];            // S written / (pass A) copied to registers
+  uint64_t p_full[2];                       // pass B: P written
   uint64_t y_full[2], y_empty[2];
   uint64_t astat_full[2], astat_empty[2];   // compute groups -> statistics publisher
   uint64_t red_full[2], red_empty[2];       // compute groups -> score writer
@@ -235,7 +269,7 @@ struct Bars {
   uint32_t tmem;
   int abort;
 };
-static_assert(sizeof(Bars<5>) <= 512, "barrier block");
+static_assert(sizeof(Bars<kRingSlots>) <= 512, "barrier block");
 
 // Merges two (max, sum) row statistics in log2 units.
 __device__ __forceinline__ float2 stat_merge(float2 x, float2 y) {
@@ -245,9 +279,39 @@ __device__ __forceinline__ float2 stat_merge(float2 x, float2 y) {
   return make_float2(M, x.y * fast_exp2(x.x - M) + y.y * fast_exp2(y.x - M));
 }
 
+// log2 normaliser of a row from its combined statistics (infinite past row m: p = 0).
+__device__ __forceinline__ float log2_norm(float2 st, bool row_ok) {
+  return row_ok && st.y > 0.f ? st.x + __log2f(st.y) : INFINITY;
+}
+__device__ __forceinline__ void write_stats(float* out, float2 st) {
+  out[0] = st.x * 0.69314718055994531f;
+  out[1] = st.y;
+}
+// Where CTA `cta` adds row r of unit u's Y partial; in deterministic mode the
+// partial goes to a slot of its own, summed in slot order later.
+__device__ __forceinline__ float* y_row(const Args& a, const Sched& sc, int u, int cta, int r) {
+  return a.ypart ? a.ypart + (((size_t)u * a.maxc + (cta - sc.first_cta(u))) * a.m + r) * kD
+                 : a.y + ((size_t)u * a.m + r) * kD;
+}
+// 32 columns of this thread's Y row from TMEM, stored or added (all lanes of the warp).
+__device__ __forceinline__ void add_y32(uint32_t taddr, float* dst, bool row_ok, bool store) {
+  float v[32];
+  tmem_ld32f(taddr, v);
+  tmem_wait32(v);
+  if (!row_ok) return;
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const float4 x = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+    if (store)
+      ((float4*)dst)[e] = x;
+    else
+      atomicAdd((float4*)dst + e, x);
+  }
+}
+
 // kPass 0: pass A, 1: pass B.  RB: row blocks.
 template <int kPass, int RB>
-__global__ void __launch_bounds__(score_threads(kPass), 1)
+__global__ void __launch_bounds__(score_threads(kPass, RB), 1)
     k_score_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                const __grid_constant__ CUtensorMap tmV, Args a) {
   using Lay = Layout<RB>;
@@ -255,13 +319,16 @@ __global__ void __launch_bounds__(score_threads(kPass), 1)
   // One row block: each V is loaded one tile after its K, as it stays in the
   // ring through the tile's compute.  Two: its first use is half a tile after its K's.
   constexpr bool kLateV = RB == 1;
+  constexpr bool kOwn = kPass == 1 && RB == 2;   // see score_threads
   extern __shared__ __align__(1024) uint8_t smraw[];
   uint8_t* sm = (uint8_t*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
   Bars<kRing>* bars = (Bars<kRing>*)(sm + Lay::kOffBar);
   float2* astat = (float2*)(sm + Lay::kOffAux);                  // pass A
   float* red = (float*)(sm + Lay::kOffAux);                      // pass B
-  float* lam_s = (float*)(sm + Lay::kOffAux + Lay::kRedBytes);   // pass B
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, cta = blockIdx.x;
+  float* lam_s = (float*)(sm + Lay::kOffAux + Lay::kRedBytes);   // pass B, RB = 1
+  float2* stat_s = (float2*)lam_s;                               // pass B, RB = 2
+  const int tid = threadIdx.x, lane = tid & 31, cta = blockIdx.x;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform for the compiler
   const Sched sc{a.U, a.tpu, (int)gridDim.x};
 
   if (tid == 0) {
@@ -277,14 +344,13 @@ __global__ void __launch_bounds__(score_threads(kPass), 1)
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bars->p_full[i], kCompWarps);
-      mbar_init(&bars->p_empty[i], 1);
       mbar_init(&bars->y_full[i], 1);
-      mbar_init(&bars->y_empty[i], 4);
+      mbar_init(&bars->y_empty[i], kOwn ? kCompWarps : 4);
       mbar_init(&bars->astat_full[i], kCompWarps);
       mbar_init(&bars->astat_empty[i], 1);
       mbar_init(&bars->red_full[i], kCompWarps);
       mbar_init(&bars->red_empty[i], 1);
-      mbar_init(&bars->lam_full[i], 4);
+      mbar_init(&bars->lam_full[i], kOwn ? kCompWarps : 4);
       mbar_init(&bars->lam_empty[i], kCompWarps);
     }
     mbar_init(&bars->drain, 1);
@@ -306,7 +372,8 @@ __global__ void __launch_bounds__(score_threads(kPass), 1)
       prefetch_tensormap(&tmQ);
       prefetch_tensormap(&tmK);
       if (kPass == 1) prefetch_tensormap(&tmV);
-      const uint64_t keep = l2_evict_last(), stream = l2_evict_first();
+      const uint64_t keep = l2_evict_last();
+      const uint64_t stream = kPass == 0 && a.keep_keys ? l2_evict_normal() : l2_evict_first();
       uint32_t idx = 0;   // loads issued through the ring
       int seg = 0;
       bool ok = true, late = false;
@@ -323,7 +390,7 @@ __global__ void __launch_bounds__(score_threads(kPass), 1)
         ++idx;
         return true;
       };
-      for (TileIter it(sc, cta); ok && it.more(); it.advance()) {
+      for (TileIter<kPass == 1> it(sc, cta); ok && it.more(); it.advance()) {
         if (it.seg_first()) {
           if (seg >= 1) ok = mbar_wait(&bars->q_empty, (seg - 1) & 1, abort_flag, a.wait_budget);
           if (!ok) break;
@@ -357,89 +424,97 @@ __global__ void __launch_bounds__(score_threads(kPass), 1)
     }
   } else if (warp == 1) {
     // ----------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      const uint32_t id_s = idesc_bf16(kRows, kTile, 0, 0);   // S = Q K^T, both K-major
-      const uint32_t id_y = idesc_bf16(kRows, kD, 0, 1);      // Y += P V, V MN-major
-      TileIter it(sc, cta);
-      const uint32_t T = (uint32_t)it.left;
-      // position of tile t's K and V among the loads
-      auto k_idx = [&](uint32_t t) { return kPass == 0 ? t : !kLateV ? 2 * t : t ? 2 * t - 1 : 0u; };
-      auto v_idx = [&](uint32_t t) { return !kLateV ? 2 * t + 1 : min(2 * t + 2, 2 * T - 1); };
-      struct {
-        uint32_t i, t;
-        int rb, seg;
-        bool seg_first, seg_last;
-      } pj{};   // the job whose Y MMA is issued after the next S MMA
-      auto issue_y = [&]() -> bool {
-        const uint32_t pb = pj.i & 1, vi = v_idx(pj.t), vs = vi % kRing;
-        const uint32_t yb = RB == 1 ? pj.seg & 1 : pj.rb, yuse = RB == 1 ? pj.seg >> 1 : pj.seg;
-        if (pj.seg_first && yuse >= 1 &&
-            !mbar_wait(&bars->y_empty[yb], (yuse - 1) & 1, abort_flag, a.wait_budget))
-          return false;
-        if (!mbar_wait(&bars->p_full[pb], (pj.i >> 1) & 1, abort_flag, a.wait_budget)) return false;
-        if (pj.rb == 0 &&
-            !mbar_wait(&bars->ring_full[vs], (vi / kRing) & 1, abort_flag, a.wait_budget))
-          return false;
+    // The whole warp walks the jobs (uniform control flow and descriptors; one
+    // elected lane issues): the issuer shares its scheduler with four compute warps,
+    // and one lane's address arithmetic was what bound pass B (2.7 K cycles a job).
+    constexpr uint32_t id_s = idesc_bf16(kRows, kTile, 0, 0);   // S = Q K^T, both K-major
+    constexpr uint32_t id_y = idesc_bf16(kRows, kD, 0, 1);      // Y += P V, V MN-major
+    const uint64_t q_desc = sw128_desc(smem_u32(sm + Lay::kOffQ), 16, 1024);
+    const uint64_t k_desc = sw128_desc(smem_u32(sm + Lay::kOffRing), 16, 1024);
+    const uint64_t v_desc = sw128_desc(smem_u32(sm + Lay::kOffRing), kTileBytes / 2, 1024);
+    constexpr uint32_t kTileDesc = kTileBytes >> 4;   // a tile's bytes in descriptor units
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      return mbar_wait_warp(bar, parity, abort_flag, a.wait_budget);
+    };
+    TileIter<kPass == 1> it(sc, cta);
+    // ring slot and phase of the next K and V: with kLateV the loads are K0, K1, V0,
+    // K2, V1, ..., V(last - 1), V(last), else K0, V0, K1, V1, ...
+    RingPos kp{0, 0}, vp{0, 0};
+    vp.add(kLateV && it.left > 1 ? 2 : 1, kRing);
+    uint32_t i = 0, t = 0;
+    int seg = 0, y_seg = 0;
+    bool ok = true;
+    // The Y MMA of the job before: issued after this job's S MMA.
+    bool y_first = false, y_last = false;
+    int y_left = it.left;   // tiles whose Y MMAs are still to come
+    auto issue_y = [&](uint32_t yi, int rb) -> bool {
+      const uint32_t pb = yi & 1;
+      const uint32_t yb = RB == 1 ? y_seg & 1 : rb, yuse = RB == 1 ? y_seg >> 1 : y_seg;
+      if (y_first && yuse >= 1 && !wait(&bars->y_empty[yb], (yuse - 1) & 1)) return false;
+      if (!wait(&bars->p_full[pb], (yi >> 1) & 1)) return false;
+      if (rb == 0 && !wait(&bars->ring_full[vp.slot], vp.phase)) return false;
+      tc_fence_after();
+      mma8_ts<id_y, kTileBytes / 16 / 16>(tmem + kColY + yb * kD, tmem + pb * kTile,
+                                          v_desc + vp.slot * kTileDesc, !y_first);
+      if (rb == RB - 1) {
+        mma_commit_elect(&bars->ring_empty[vp.slot]);
+        // the last V follows its predecessor directly
+        --y_left;
+        vp.add(kLateV && y_left == 1 ? 1 : 2, kRing);
+      }
+      if (y_last) {
+        mma_commit_elect(&bars->y_full[yb]);
+        if (rb == RB - 1) ++y_seg;
+      }
+      return true;
+    };
+    for (; ok && it.more(); it.advance(), ++t) {
+      const bool first = it.seg_first(), last = it.seg_last();
+      if (first) ok = wait(&bars->q_full, seg & 1);
+      if (ok) ok = wait(&bars->ring_full[kp.slot], kp.phase);
+#pragma unroll
+      for (int rb = 0; rb < RB; ++rb, ++i) {
+        // Pass A: the buffer's last logits are in registers.  Pass B: the Y MMA that
+        // reads the buffer's last probabilities was issued before this S MMA; a
+        // tile's S also says that its score sums (tile t - 2's) have been read.
+        const uint32_t sb = i % kS, use = i / kS;
+        if (kPass == 0 && ok && use >= 1) ok = wait(&bars->s_done[sb], (use - 1) & 1);
+        if (kPass == 1 && rb == 0 && ok && t >= 2)
+          ok = wait(&bars->red_empty[t & 1], ((t >> 1) - 1) & 1);
+        if (!ok) break;
         tc_fence_after();
-        const uint32_t va = smem_u32(sm + Lay::kOffRing + vs * kTileBytes);
-#pragma unroll
-        for (int kk = 0; kk < kTile / 16; ++kk)
-          mma_bf16_ts(tmem + kColY + yb * kD, tmem + kColP + pb * 64 + kk * 8,
-                      sw128_desc(va + kk * 2048, kTileBytes / 2, 1024), id_y,
-                      (pj.seg_first && kk == 0) ? 0u : 1u);
-        mma_commit(&bars->p_empty[pb]);
-        if (pj.rb == RB - 1) mma_commit(&bars->ring_empty[vs]);
-        if (pj.seg_last) mma_commit(&bars->y_full[yb]);
-        return true;
-      };
-      uint32_t i = 0, t = 0;
-      int seg = 0;
-      bool ok = true;
-      for (; ok && it.more(); it.advance(), ++t) {
-        const bool first = it.seg_first(), last = it.seg_last();
-        if (first) ok = mbar_wait(&bars->q_full, seg & 1, abort_flag, a.wait_budget);
-        const uint32_t ki = k_idx(t), ks = ki % kRing;
-        if (ok) ok = mbar_wait(&bars->ring_full[ks], (ki / kRing) & 1, abort_flag, a.wait_budget);
-        const uint32_t ka = smem_u32(sm + Lay::kOffRing + ks * kTileBytes);
-        for (int rb = 0; ok && rb < RB; ++rb, ++i) {
-          const uint32_t sb = i % kS, use = i / kS;
-          if (use >= 1)
-            ok = mbar_wait(&bars->s_done[sb], (use - 1) & 1, abort_flag, a.wait_budget);
+        mma8_ss<id_s>(tmem + sb * kTile, q_desc + rb * kTileDesc, k_desc + kp.slot * kTileDesc);
+        mma_commit_elect(&bars->s_full[sb]);
+        if (rb == RB - 1) {
+          mma_commit_elect(&bars->ring_empty[kp.slot]);
+          if (last) mma_commit_elect(&bars->q_empty);
+        }
+        if (kPass == 1) {
+          if (i > 0) ok = issue_y(i - 1, RB == 1 ? 0 : 1 - rb);
           if (!ok) break;
-          tc_fence_after();
-          const uint32_t qa = smem_u32(sm + Lay::kOffQ + rb * kTileBytes);
-#pragma unroll
-          for (int kk = 0; kk < kD / 16; ++kk) {
-            const uint32_t off = (kk >> 2) * (kTileBytes / 2) + (kk & 3) * 32;
-            mma_bf16(tmem + sb * kTile, sw128_desc(qa + off, 16, 1024),
-                     sw128_desc(ka + off, 16, 1024), id_s, kk > 0);
-          }
-          mma_commit(&bars->s_full[sb]);
-          if (rb == RB - 1) {
-            mma_commit(&bars->ring_empty[ks]);
-            if (last) mma_commit(&bars->q_empty);
-          }
-          if (kPass == 1) {
-            if (i > 0) ok = issue_y();
-            pj = {i, t, rb, seg, first, last};
+          if (rb == 0) {
+            y_first = first;
+            y_last = last;
           }
         }
-        if (last) ++seg;
       }
-      if (kPass == 1 && ok && i > 0) issue_y();
-      // every MMA issued so far completes before TMEM can be released (this
-      // wait ignores the abort flag, and is bounded)
-      mma_commit(&bars->drain);
-      volatile int no_abort = 0;
-      mbar_wait(&bars->drain, 0, &no_abort, a.wait_budget);
+      kp.add(kPass == 0 || (kLateV && t == 0) ? 1 : 2, kRing);
+      if (last) ++seg;
     }
+    if (kPass == 1 && ok && i > 0) issue_y(i - 1, RB - 1);
+    // every MMA issued so far completes before TMEM can be released (this
+    // wait ignores the abort flag, and is bounded)
+    mma_commit_elect(&bars->drain);
+    volatile int no_abort = 0;
+    mbar_wait(&bars->drain, 0, &no_abort, a.wait_budget);
+    __syncwarp();
   } else if (kPass == 0 && warp == 2) {
     // ----------------------------------------------- statistics publisher
     // Merges the compute groups' row statistics of each segment into the
     // segment's global slot.
     int aseg = 0;
     bool ok = true;
-    for (TileIter it(sc, cta); ok && it.more(); it.advance()) {
+    for (TileIter<kPass == 1> it(sc, cta); ok && it.more(); it.advance()) {
       if (!it.seg_last()) continue;
       const int ab = aseg & 1;
       ok = mbar_wait_warp(&bars->astat_full[ab], (aseg >> 1) & 1, abort_flag, a.wait_budget);
@@ -468,31 +543,24 @@ __global__ void __launch_bounds__(score_threads(kPass), 1)
     }
   } else if (kPass == 1 && warp == 2) {
     // ------------------------------------------------------- score writer
-    // Adds the four row quarters' sums of every tile (both row blocks') and
-    // writes the prefix scores.
+    // Adds the four row quarters' sums of every tile and writes the prefix scores.
     uint32_t t = 0;
     bool ok = true;
-    for (TileIter it(sc, cta); ok && it.more(); it.advance(), ++t) {
+    for (TileIter<kPass == 1> it(sc, cta); ok && it.more(); it.advance(), ++t) {
       const uint32_t tb = t & 1;
       ok = mbar_wait_warp(&bars->red_full[tb], (t >> 1) & 1, abort_flag, a.wait_budget);
       if (!ok) break;
-      const float* rt = red + tb * RB * 4 * kTile;
+      const float* rt = red + tb * 4 * kTile;
       float* out = a.scores + (size_t)it.u * a.P;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const int j = c * 32 + lane;
-        float cs = 0.f;
-#pragma unroll
-        for (int rb = 0; rb < RB; ++rb) {
-          const float* r = rt + rb * 4 * kTile + j;
-          const float x = ((r[0] + r[kTile]) + r[2 * kTile]) + r[3 * kTile];
-          cs = rb ? cs + x : x;
-        }
+        const float cs = ((rt[j] + rt[kTile + j]) + rt[2 * kTile + j]) + rt[3 * kTile + j];
         if (it.j0() + j < a.P) out[it.j0() + j] = cs;
       }
       mbar_arrive_warp(&bars->red_empty[tb], lane);
     }
-  } else if (kPass == 1 && warp >= 4 + kCompWarps) {
+  } else if (kPass == 1 && RB == 1 && warp >= 4 + kCompWarps) {
     // ------------------------------------- statistics fetcher, Y flusher
     // Segment s + 1's normalisers are combined before segment s's Y partial is
     // added.  One thread owns one row (TMEM lane); the CTA that holds the unit's first
@@ -500,39 +568,32 @@ __global__ void __launch_bounds__(score_threads(kPass), 1)
     const int q = warp & 3, row = q * 32 + lane;
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
     const long long t0 = sc.start(cta), t1 = sc.start(cta + 1);
-    const int u0 = (int)(t0 / a.tpu), nseg = t1 > t0 ? (int)((t1 - 1) / a.tpu) - u0 + 1 : 0;
+    // segments from the CTA's last unit down, as its tiles
+    const int u0 = (int)((t1 - 1) / a.tpu), nseg = t1 > t0 ? u0 - (int)(t0 / a.tpu) + 1 : 0;
     bool ok = true;
     for (int s = 0; ok && s <= nseg && nseg > 0; ++s) {
       if (s < nseg) {
-        const int u = u0 + s, lb = s & 1;
+        const int u = u0 - s, lb = s & 1;
         if (s >= 2)
           ok = mbar_wait_warp(&bars->lam_empty[lb], ((s >> 1) - 1) & 1, abort_flag, a.wait_budget);
         if (!ok) break;
         const int ns = sc.nslots(u), c0 = sc.first_cta(u);
         const bool dense = sc.tiles() >= sc.G;   // every CTA holds tiles
+        float2 st = make_float2(-INFINITY, 0.f);
+        // sixteen slots per round trip
+        for (int k0 = 0; k0 < ns; k0 += 16) {
+          float2 pr[16];
 #pragma unroll
-        for (int rb = 0; rb < RB; ++rb) {
-          const int r = rb * kRows + row;
-          float2 st = make_float2(-INFINITY, 0.f);
-          // sixteen slots per round trip
-          for (int k0 = 0; k0 < ns; k0 += 16) {
-            float2 pr[16];
-#pragma unroll
-            for (int kk = 0; kk < 16; ++kk) {
-              const bool use = k0 + kk < ns && (dense || !sc.empty(c0 + k0 + kk));
-              pr[kk] = use ? __ldg(a.pstats + ((size_t)u * a.maxc + k0 + kk) * (RB * kRows) + r)
-                           : make_float2(-INFINITY, 0.f);
-            }
-#pragma unroll
-            for (int kk = 0; kk < 16; ++kk) st = stat_merge(st, pr[kk]);
+          for (int kk = 0; kk < 16; ++kk) {
+            const bool use = k0 + kk < ns && (dense || !sc.empty(c0 + k0 + kk));
+            pr[kk] = use ? __ldg(a.pstats + ((size_t)u * a.maxc + k0 + kk) * kRows + row)
+                         : make_float2(-INFINITY, 0.f);
           }
-          lam_s[(lb * RB + rb) * kRows + row] =
-              (r < a.m && st.y > 0.f) ? st.x + __log2f(st.y) : INFINITY;
-          if (cta == c0 && r < a.m) {
-            a.row_stats[((size_t)u * a.m + r) * 2 + 0] = st.x * 0.69314718055994531f;
-            a.row_stats[((size_t)u * a.m + r) * 2 + 1] = st.y;
-          }
+#pragma unroll
+          for (int kk = 0; kk < 16; ++kk) st = stat_merge(st, pr[kk]);
         }
+        lam_s[lb * kRows + row] = log2_norm(st, row < a.m);
+        if (cta == c0 && row < a.m) write_stats(a.row_stats + ((size_t)u * a.m + row) * 2, st);
         // GRKV_TEST_TIMEOUT: CTA 0 never announces its first normalisers, so
         // its compute groups' bounded wait expires
         __syncwarp();
@@ -540,37 +601,16 @@ __global__ void __launch_bounds__(score_threads(kPass), 1)
           mbar_arrive(&bars->lam_full[lb]);
       }
       if (s == 0) continue;
-      const int fs = s - 1, u = u0 + fs;
-      for (int rb = 0; ok && rb < RB; ++rb) {
-        const int yb = RB == 1 ? fs & 1 : rb, yuse = RB == 1 ? fs >> 1 : fs, r = rb * kRows + row;
-        ok = mbar_wait_warp(&bars->y_full[yb], yuse & 1, abort_flag, a.wait_budget);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t ybase = lane_addr + kColY + yb * kD;
-        // deterministic: the partial goes to its own slot, summed in slot order later
-        const int k = cta - sc.first_cta(u);
-        float* base = a.ypart ? a.ypart + (((size_t)u * a.maxc + k) * a.m + r) * kD
-                              : a.y + ((size_t)u * a.m + r) * kD;
+      const int fs = s - 1, u = u0 - fs, yb = fs & 1;
+      ok = mbar_wait_warp(&bars->y_full[yb], (fs >> 1) & 1, abort_flag, a.wait_budget);
+      if (!ok) break;
+      tc_fence_after();
+      float* dst = y_row(a, sc, u, cta, row);
 #pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
-          float v[32];
-          tmem_ld32f(ybase + c * 32, v);
-          tmem_wait32(v);
-          if (r < a.m) {
-            float4* dst = (float4*)(base + c * 32);
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const float4 x = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
-              if (a.ypart)
-                dst[e] = x;
-              else
-                atomicAdd(dst + e, x);
-            }
-          }
-        }
-        tc_fence_before();
-        mbar_arrive_warp(&bars->y_empty[yb], lane);
-      }
+      for (int c = 0; c < 4; ++c)
+        add_y32(lane_addr + kColY + yb * kD + c * 32, dst + c * 32, row < a.m, a.ypart != nullptr);
+      tc_fence_before();
+      mbar_arrive_warp(&bars->y_empty[yb], lane);
     }
     if (!ok && row == 0) set_status(a.status, GRKV_ERR_TIMEOUT);
   } else if (warp >= 4 && warp < 4 + kCompWarps) {
@@ -587,23 +627,65 @@ __global__ void __launch_bounds__(score_threads(kPass), 1)
     uint32_t i = 0, t = 0;
     int seg = 0;
     bool ok = true;
-    for (TileIter it(sc, cta); ok && it.more(); it.advance(), ++t) {
+    for (TileIter<kPass == 1> it(sc, cta); ok && it.more(); it.advance(), ++t) {
       const int t0 = it.j0() + 32 * g;   // this group's first token
       const bool in = t0 + 32 <= a.n;
       if (it.seg_first()) {
-        const int lb = seg & 1;
-        if (kPass == 1) {
+        if (kPass == 0) {
+#pragma unroll
+          for (int rb = 0; rb < RB; ++rb) {
+            M[rb] = -INFINITY;
+            L[rb] = 0.f;
+          }
+        } else if (!kOwn) {
+          const int lb = seg & 1;
           ok = mbar_wait_warp(&bars->lam_full[lb], (seg >> 1) & 1, abort_flag, a.wait_budget);
           if (!ok) break;
-        }
+          lam[0] = lam_s[lb * kRows + row];
+          mbar_arrive_warp(&bars->lam_empty[lb], lane);
+        } else {
+          // Each group combines a quarter of the unit's slots.  A segment's jobs pass
+          // through s_done of every warp, so no warp still reads the last shares.
+          const int ns = sc.nslots(it.u), c0 = sc.first_cta(it.u);
+          const bool dense = sc.tiles() >= sc.G;   // every CTA holds tiles
+          float2 st[RB];
 #pragma unroll
-        for (int rb = 0; rb < RB; ++rb) {
-          M[rb] = -INFINITY;
-          L[rb] = 0.f;
-          if (kPass == 1) lam[rb] = lam_s[(lb * RB + rb) * kRows + row];
+          for (int rb = 0; rb < RB; ++rb) {
+            st[rb] = make_float2(-INFINITY, 0.f);
+            for (int k0 = g; k0 < ns; k0 += 8 * kGroups) {   // eight slots per round trip
+              float2 pr[8];
+#pragma unroll
+              for (int kk = 0; kk < 8; ++kk) {
+                const int k = k0 + kk * kGroups;
+                const bool use = k < ns && (dense || !sc.empty(c0 + k));
+                pr[kk] = use ? __ldg(a.pstats + ((size_t)it.u * a.maxc + k) * (RB * kRows) +
+                                     rb * kRows + row)
+                             : make_float2(-INFINITY, 0.f);
+              }
+#pragma unroll
+              for (int kk = 0; kk < 8; ++kk) st[rb] = stat_merge(st[rb], pr[kk]);
+            }
+            stat_s[(g * RB + rb) * kRows + row] = st[rb];
+          }
+          __syncwarp();
+          // GRKV_TEST_TIMEOUT: CTA 0 never completes its first normalisers
+          if (lane == 0 && !(a.test_withhold && cta == 0 && seg == 0 && warp == 4))
+            mbar_arrive(&bars->lam_full[0]);
+          ok = mbar_wait_warp(&bars->lam_full[0], seg & 1, abort_flag, a.wait_budget);
+          if (!ok) break;
+#pragma unroll
+          for (int rb = 0; rb < RB; ++rb) {
+            const int r = rb * kRows + row;
+            float2 x = stat_s[r];
+#pragma unroll
+            for (int h = 1; h < kGroups; ++h) x = stat_merge(x, stat_s[h * RB * kRows + r]);
+            lam[rb] = log2_norm(x, r < a.m);
+            if (g == 0 && cta == c0 && r < a.m)
+              write_stats(a.row_stats + ((size_t)it.u * a.m + r) * 2, x);
+          }
         }
-        if (kPass == 1) mbar_arrive_warp(&bars->lam_empty[lb], lane);
       }
+      float both[RB == 2 ? 32 : 1];   // pass B: the first row block's probabilities
 #pragma unroll
       for (int rb = 0; rb < RB; ++rb, ++i) {
         const uint32_t sb = i % kS;
@@ -614,8 +696,10 @@ __global__ void __launch_bounds__(score_threads(kPass), 1)
         float v[32];
         tmem_ld32f(lane_addr + sb * kTile + 32 * g, v);
         tmem_wait32(v);
-        tc_fence_before();
-        mbar_arrive_warp(&bars->s_done[sb], lane);
+        if (kPass == 0) {
+          tc_fence_before();
+          mbar_arrive_warp(&bars->s_done[sb], lane);
+        }
         // chunks away from the window and the end of the unit need no mask
         const bool full = in && t0 + 31 <= lim[rb];
         if (kPass == 0) {
@@ -623,7 +707,6 @@ __global__ void __launch_bounds__(score_threads(kPass), 1)
           continue;
         }
         const uint64_t s2 = pack2(a.sl2, a.sl2), m2 = pack2(-lam[rb], -lam[rb]);
-        uint32_t pk[16];
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
           float x, y;
@@ -637,16 +720,28 @@ __global__ void __launch_bounds__(score_threads(kPass), 1)
             if (t0 + e > lim[rb] || t0 + e >= a.n) v[e] = 0.f;
         }
 #pragma unroll
-        for (int e = 0; e < 16; ++e) pk[e] = pack_bf16(v[2 * e], v[2 * e + 1]);
-        const uint32_t pb = i & 1;
-        if (i >= 2)
-          ok = mbar_wait_warp(&bars->p_empty[pb], ((i >> 1) - 1) & 1, abort_flag, a.wait_budget);
-        if (!ok) break;
-        tc_fence_after();
-        tmem_st16(lane_addr + kColP + pb * 64 + 16 * g, pk);
+        for (int h = 0; h < 2; ++h) {
+          uint32_t pk[8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) pk[e] = pack_bf16(v[16 * h + 2 * e], v[16 * h + 2 * e + 1]);
+          tmem_st8(lane_addr + sb * kTile + 32 * g + 8 * h, pk);
+        }
         tmem_st_wait();
         tc_fence_before();
-        mbar_arrive_warp(&bars->p_full[pb], lane);
+        mbar_arrive_warp(&bars->p_full[sb], lane);
+        if (RB == 2 && rb == 0) {
+#pragma unroll
+          for (int e = 0; e < 32; ++e) both[e % (RB == 2 ? 32 : 1)] = v[e];
+          continue;
+        }
+        if (RB == 2) {
+          // one reduction for both row blocks
+#pragma unroll
+          for (int e = 0; e < 16; ++e)
+            unpack2(add2(pack2(both[(2 * e) % (RB == 2 ? 32 : 1)], both[(2 * e + 1) % (RB == 2 ? 32 : 1)]),
+                         pack2(v[2 * e], v[2 * e + 1])),
+                    v[2 * e], v[2 * e + 1]);
+        }
         // transpose-reduce: lane t ends with the warp's sum for token t
 #pragma unroll
         for (int hh = 16; hh >= 1; hh >>= 1) {
@@ -659,11 +754,8 @@ __global__ void __launch_bounds__(score_threads(kPass), 1)
           }
         }
         const uint32_t tb = t & 1;
-        if (rb == 0 && t >= 2)
-          ok = mbar_wait_warp(&bars->red_empty[tb], ((t >> 1) - 1) & 1, abort_flag, a.wait_budget);
-        if (!ok) break;
-        red[((tb * RB + rb) * 4 + q) * kTile + 32 * g + lane] = v[0];
-        if (rb == RB - 1) mbar_arrive_warp(&bars->red_full[tb], lane);
+        red[(tb * 4 + q) * kTile + 32 * g + lane] = v[0];
+        mbar_arrive_warp(&bars->red_full[tb], lane);
       }
       if (!ok) break;
       if (it.seg_last()) {
@@ -677,6 +769,19 @@ __global__ void __launch_bounds__(score_threads(kPass), 1)
           for (int rb = 0; rb < RB; ++rb)
             astat[((ab * kGroups + g) * RB + rb) * kRows + row] = make_float2(M[rb], L[rb]);
           mbar_arrive_warp(&bars->astat_full[ab], lane);
+        } else if (kOwn) {
+#pragma unroll
+          for (int rb = 0; rb < RB; ++rb) {
+            const int r = rb * kRows + row;
+            ok = ok && mbar_wait_warp(&bars->y_full[rb], seg & 1, abort_flag, a.wait_budget);
+            if (!ok) break;
+            tc_fence_after();
+            add_y32(lane_addr + kColY + rb * kD + 32 * g, y_row(a, sc, it.u, cta, r) + 32 * g,
+                    r < a.m, a.ypart != nullptr);
+            tc_fence_before();
+            mbar_arrive_warp(&bars->y_empty[rb], lane);
+          }
+          if (!ok) break;
         }
         ++seg;
       }
@@ -721,7 +826,7 @@ cudaError_t launch_pass(int G, const CUtensorMap& mq, const CUtensorMap& mk, con
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   count_launches(1);
-  kern<<<G, score_threads(kPass), smem, st>>>(mq, mk, mv, a);
+  kern<<<G, score_threads(kPass, RB), smem, st>>>(mq, mk, mv, a);
   return cudaGetLastError();
 }
 
@@ -767,6 +872,12 @@ cudaError_t launch_score_tc(const Shape& s, const void* q, const void* k, const 
   a.causal = s.causal;
   a.tpu = (s.n + kTile - 1) / kTile;
   a.maxc = score_tc_slots(s.U, G);
+  // Pass B walks each CTA's tiles backwards, so the keys that pass A read last may
+  // still be in L2.  They are kept there (evict-normal loads) when the cache is many
+  // times L2: 2.1 GB of keys, 256 units n = 32768, 1325 -> 1298 us a compress call.  With
+  // 134 MB of keys (32 units n = 16384) that costs 184 -> 193 us, as the merge then finds
+  // fewer of its rows in L2; 268 MB of keys lose 1%.
+  a.keep_keys = (size_t)s.U * s.n * kD * 2 > ((size_t)512 << 20);
   a.sl2 = (float)((double)s.scale * 1.4426950408889634);
   a.scores = scores;
   a.y = s.deterministic ? nullptr : y;

@@ -184,6 +184,71 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
       : "memory");
 }
 
+// The eight K = 16 steps of a 128 x 128 x 128 product, issued by one elected lane of
+// a converged warp.  The descriptors advance inside: with warp-uniform operands
+// the arithmetic stays on the uniform datapath.
+// D = A B^T, both K-major tiles of two 64-column halves (128-byte swizzle).
+template <uint32_t kIdesc>
+__device__ __forceinline__ void mma8_ss(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc) {
+  asm volatile(
+      "{\n .reg .pred q, f, t;\n .reg .b64 a, b;\n"
+      " elect.sync _|q, 0xffffffff;\n"
+      " setp.ne.b32 f, 0, 0;\n setp.eq.b32 t, 0, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, f;\n"
+      " add.u64 a, %1, 2;\n add.u64 b, %2, 2;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n"
+      " add.u64 a, %1, 4;\n add.u64 b, %2, 4;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n"
+      " add.u64 a, %1, 6;\n add.u64 b, %2, 6;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n"
+      " add.u64 a, %1, 1024;\n add.u64 b, %2, 1024;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n"
+      " add.u64 a, %1, 1026;\n add.u64 b, %2, 1026;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n"
+      " add.u64 a, %1, 1028;\n add.u64 b, %2, 1028;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n"
+      " add.u64 a, %1, 1030;\n add.u64 b, %2, 1030;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, t;\n}\n" ::"r"(d_tmem),
+      "l"(adesc), "l"(bdesc), "n"(kIdesc)
+      : "memory");
+}
+// D (+)= A B^T with A in TMEM, 8 packed columns per step, two steps to every 32
+// columns, and B advancing kStep descriptor units per step.
+template <uint32_t kIdesc, int kStep>
+__device__ __forceinline__ void mma8_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc,
+                                        bool accumulate) {
+  asm volatile(
+      "{\n .reg .pred q, f, t;\n .reg .b64 b;\n .reg .b32 a;\n"
+      " elect.sync _|q, 0xffffffff;\n"
+      " setp.ne.b32 f, %4, 0;\n setp.eq.b32 t, 0, 0;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, f;\n"
+      " add.u32 a, %1, 8;\n add.u64 b, %2, %5;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
+      " add.u32 a, %1, 32;\n add.u64 b, %2, %6;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
+      " add.u32 a, %1, 40;\n add.u64 b, %2, %7;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
+      " add.u32 a, %1, 64;\n add.u64 b, %2, %8;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
+      " add.u32 a, %1, 72;\n add.u64 b, %2, %9;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
+      " add.u32 a, %1, 96;\n add.u64 b, %2, %10;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
+      " add.u32 a, %1, 104;\n add.u64 b, %2, %11;\n"
+      " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "n"(kIdesc), "r"((uint32_t)accumulate), "n"(kStep), "n"(2 * kStep),
+      "n"(3 * kStep), "n"(4 * kStep), "n"(5 * kStep), "n"(6 * kStep), "n"(7 * kStep)
+      : "memory");
+}
+// mma_commit by the elected lane of a converged warp (the lane that issued).
+__device__ __forceinline__ void mma_commit_elect(uint64_t* bar) {
+  asm volatile(
+      "{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n"
+      " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(
+          smem_u32(bar))
+      : "memory");
+}
+
 // 32 consecutive fp32 columns of this thread's TMEM lane.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
   uint32_t r[32];
@@ -252,6 +317,13 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* r) {
       "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
       "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]),
       "r"(r[15])
+      : "memory");
+}
+// 8 packed 32-bit columns into this thread's TMEM lane.
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
+      "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
       : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() {
