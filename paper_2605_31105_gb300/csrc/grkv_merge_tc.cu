@@ -42,11 +42,13 @@ using namespace sm100;
 
 constexpr int kTile = 128;
 constexpr int kRows = 128;
-constexpr int kThreads = 384;    // k_merge_gram
+constexpr int kThreads = 384;    // k_merge_cross
+constexpr int kThreadsG = 640;   // k_merge_gram
 constexpr int kThreadsU = 736;   // k_merge_update
 constexpr uint32_t kTileBytes = kTile * kD * 2;   // 32 KB
 constexpr int kMaxB = 32768;
 constexpr int kSms = 152;        // SMs of a GB300
+constexpr int kClusterSms = 128; // SMs that clusters of up to 8 CTAs (one per SM) can be counted on to fill
 constexpr long long kBudget = 1ll << 32;
 
 // Shared memory (offsets from a 1024-byte aligned base).  k_merge_gram: Q, a
@@ -84,12 +86,11 @@ struct MArgs {
   float* lam;                // [U][128]       log2 normaliser of each window row
   int32_t* src;              // [U][B]         K / V row of each position
   int32_t* ng;               // [U]            number of non-fixed slots
-  int32_t* redo;             // [U]            single-pass result unusable: run two passes
   uint8_t* fixed;            // [U][B]         1 for a fixed slot
-  int gram_mode;             // 0 two passes; 1 one pass against rstats; 2 two passes for redo units
-  // Row blocks (m > 128): a launch takes the 128 window rows row0 .. row0+127
+  int ranks;                 // k_merge_gram: CTAs per unit and row block
+  // Row blocks (m > 128): an update launch takes the 128 window rows row0 .. row0+127
   // of block rb (of nrb); the per-unit arrays hold ldr rows (128 or 256):
-  // rz [U][ldr][128], gram [U][ldr][ldr], lam [U][ldr], redo [U][nrb].
+  // rz [U][ldr][128], gram [U][ldr][ldr], lam [U][ldr].
   int row0, rb, nrb, ldr;
   int upd_mode;              // update: 0 V_out = V0 + dV; 1 vpart = V0 + dV; 2 V_out = vpart + dV
   float* vpart;              // [U][B][128] fp32, between the update's two row blocks
@@ -97,20 +98,6 @@ struct MArgs {
   const UnitRow* units;      // budgets of the units, or null (B each)
   int split;                 // update: CTAs per unit
 };
-
-struct MBars {
-  uint64_t ring_full[4], ring_empty[4];
-  uint64_t q_full;
-  uint64_t s_full[2], s_done[2];
-  uint64_t xg_full[2], xg_empty[2];
-  uint64_t acc_done;
-  uint64_t d_full[2], d_empty[2];
-  uint64_t drain;
-  uint32_t tmem;
-  int abort;
-  int bad;
-};
-static_assert(sizeof(MBars) <= 256, "barrier block");
 
 __device__ __forceinline__ float lo_half(uint32_t h) { return __uint_as_float(h << 16); }
 __device__ __forceinline__ float hi_half(uint32_t h) { return __uint_as_float(h & 0xFFFF0000u); }
@@ -197,36 +184,6 @@ struct Gatherer {
   }
 };
 
-// ring_empty_count: arrivals that release a ring slot; group_count: threads
-// of the compute warps that arrive on s_done, xg_full and d_empty.
-__device__ __forceinline__ void init_common(MBars* bars, int warp, uint32_t ring_empty_count,
-                                            uint32_t group_count, uint32_t epi_count) {
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < 4; ++i) {
-      mbar_init(&bars->ring_full[i], 3);   // one expect_tx arrival per gathering warp
-      mbar_init(&bars->ring_empty[i], ring_empty_count);
-    }
-    mbar_init(&bars->q_full, 1);
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&bars->s_full[i], 1);
-      mbar_init(&bars->s_done[i], group_count);
-      mbar_init(&bars->xg_full[i], group_count);
-      mbar_init(&bars->xg_empty[i], 1);
-      mbar_init(&bars->d_full[i], 1);
-      mbar_init(&bars->d_empty[i], epi_count);
-    }
-    mbar_init(&bars->acc_done, 1);
-    mbar_init(&bars->drain, 1);
-    bars->abort = 0;
-    bars->bad = 0;
-    fence_mbar_init();
-  }
-  if (warp == 1) {
-    tmem_alloc(&bars->tmem, 512);
-    tmem_relinquish();
-  }
-}
-
 // S = Q K0^T for one gathered tile into TMEM columns s_col (issued by one thread).
 __device__ __forceinline__ void issue_s(uint32_t s_tmem, uint32_t qa, uint32_t ka) {
   const uint32_t id_s = idesc_bf16(kRows, kTile, 0, 0);
@@ -246,50 +203,37 @@ __device__ __forceinline__ void store_row_chunk(uint8_t* tile, int row, int C, c
         make_uint4(w[4 * qq], w[4 * qq + 1], w[4 * qq + 2], w[4 * qq + 3]);
 }
 
-// One 32-position chunk of a gram tile whose positions are all non-fixed (and
-// so visible): Xh to TMEM (the A operand of R~ and of the Gram's first term),
-// XGh = Xh to shared memory (the Gram's B operand) and 2 (X - Xh) returned (it
-// goes to TMEM once the S columns it overwrites are read).
-template <int C>
-__device__ __forceinline__ void gram_chunk_fast(const float* v, float sl2, float lam,
-                                                uint32_t sbase, uint8_t* xg, int row,
-                                                uint32_t* lo, float& vmax, float& xsum) {
-  uint32_t hi[16];
+// One 32-position chunk of a row of a gram tile: Xh (packed bf16, the A operand of
+// R~ and of the Gram's first term) and 2 (X - Xh), X = exp2(l - lam); X = 0 past
+// position vl of the chunk when kMasked.  Pairs of floats as in the scoring kernel.
+template <bool kMasked>
+__device__ __forceinline__ void gram_chunk(float* v, int vl, float sl2, float lam, uint32_t* hi,
+                                           uint32_t* lo, float& vmax, float& xsum) {
+  if (kMasked) {
 #pragma unroll
-  for (int e = 0; e < 32; e += 2) {
-    const float x0 = fast_exp2(fmaf(v[e], sl2, -lam)), x1 = fast_exp2(fmaf(v[e + 1], sl2, -lam));
-    vmax = fmaxf(vmax, fmaxf(v[e], v[e + 1]));
-    xsum += x0 + x1;
-    const uint32_t h = pack_bf16(x0, x1);
-    hi[e / 2] = h;
-    lo[e / 2] = pack_bf16(2.f * (x0 - lo_half(h)), 2.f * (x1 - hi_half(h)));
+    for (int e = 0; e < 32; ++e)
+      if (e > vl) v[e] = -INFINITY;
   }
-  tmem_st16(sbase + C * 16, hi);
-  store_row_chunk(xg, row, C, hi);
-}
-// The same for a tile with fixed or invisible positions: X = 0 past vlim,
-// XGh = 0 from position ng on; XGh is written only when the tile has
-// non-fixed positions (want_g).
-template <int C>
-__device__ __forceinline__ void gram_chunk_masked(const float* v, int p0, int vlim, int ng,
-                                                  float sl2, float lam, uint32_t sbase,
-                                                  uint8_t* xg, int row, uint32_t* lo,
-                                                  bool want_g, float& vmax, float& xsum) {
-  uint32_t hi[16], ghi[16];
 #pragma unroll
-  for (int e = 0; e < 32; e += 2) {
-    const int p = p0 + C * 32 + e;
-    const float x0 = p <= vlim ? fast_exp2(fmaf(v[e], sl2, -lam)) : 0.f;
-    const float x1 = p + 1 <= vlim ? fast_exp2(fmaf(v[e + 1], sl2, -lam)) : 0.f;
-    vmax = fmaxf(vmax, fmaxf(p <= vlim ? v[e] : -INFINITY, p + 1 <= vlim ? v[e + 1] : -INFINITY));
-    xsum += x0 + x1;
+  for (int e = 0; e < 32; e += 2) vmax = fmaxf(vmax, fmaxf(v[e], v[e + 1]));
+  const uint64_t s2 = pack2(sl2, sl2), l2 = pack2(-lam, -lam), minus2 = pack2(-2.f, -2.f);
+  uint64_t sum = 0;   // a pair of zeros
+#pragma unroll
+  for (int e = 0; e < 16; ++e) {
+    float x0, x1;
+    unpack2(fma2(pack2(v[2 * e], v[2 * e + 1]), s2, l2), x0, x1);
+    x0 = fast_exp2(x0);
+    x1 = fast_exp2(x1);
+    const uint64_t x = pack2(x0, x1);
+    sum = add2(sum, x);
     const uint32_t h = pack_bf16(x0, x1);
-    hi[e / 2] = h;
-    lo[e / 2] = pack_bf16(2.f * (x0 - lo_half(h)), 2.f * (x1 - hi_half(h)));
-    ghi[e / 2] = (p < ng ? (h & 0xFFFFu) : 0u) | (p + 1 < ng ? (h & 0xFFFF0000u) : 0u);
+    hi[e] = h;
+    unpack2(fma2(pack2(lo_half(h), hi_half(h)), minus2, add2(x, x)), x0, x1);   // exact
+    lo[e] = pack_bf16(x0, x1);
   }
-  tmem_st16(sbase + C * 16, hi);
-  if (want_g) store_row_chunk(xg, row, C, ghi);
+  float s0, s1;
+  unpack2(sum, s0, s1);
+  xsum += s0 + s1;
 }
 
 // Online max / sum of exp2 over one 32-column chunk (log2 units); positions
@@ -387,317 +331,352 @@ __global__ void __launch_bounds__(256) k_merge_fixed(MArgs a) {
 }
 
 // ======================================================== k_merge_gram
-// Roles (384 threads): warp 0 the Q load; warp 1 MMA issue; warps 0, 2, 3 the gathers;
-// warps 4-7 and 8-11 two compute groups (one thread per window row / TMEM
-// lane) taking alternate jobs.  Job k < T: statistics of slot tile k;
-// T <= k < 2T: R~ and Gram of position tile k - T.  Ring loads: K of each
-// pass-1 job, then K and V of each pass-2 job.
+// A cluster of a.ranks CTAs per unit and row block, each on a contiguous share of
+// the unit's tiles; the shares of R~ and of the Gram meet in distributed shared
+// memory, where rank r adds rows [128 r / ranks, 128 (r + 1) / ranks) of all shares
+// in rank order and writes them.
 //
-// gram_mode 1 (the full-cache row statistics are known) runs only the second
-// pass, with X accumulated against the full row maximum M_r instead of the
-// retained one: X' = exp2(l - M_r) = X L'_r with L'_r = sum of X' over the
+// With the full-cache row statistics (always in grkv_compress) one phase: X against
+// the full row maximum M_r, X' = exp2(l - M_r) = X L'_r with L'_r = sum of X' over the
 // visible retained keys, so R = Y - R~'/L'_r and G_ij = G'_ij/(L'_i L'_j).  The
-// retained maximum is at most M_r; if it is more than 64 (log2 units) below
-// it for some row, or L' underflows, the unit is flagged and gram_mode 2
-// recomputes it with both passes.
-__global__ void __launch_bounds__(kThreads, 1)
+// retained maximum is at most M_r; if it is more than 64 (log2 units) below it for
+// some row, or L' underflows, the cluster starts over with two phases, which is
+// also the path without statistics: row statistics over the slots, then R~ and
+// the Gram over the positions with X itself.
+//
+// Roles (640 threads): warp 0 the Q load; warps 0, 2, 3 the gathers; warp 1 MMA
+// issue; warps 4-19 four compute groups of 128 threads, 32 positions of every
+// tile each, one thread per window row (TMEM lane).  A thread copies its 32 logits
+// to registers and writes Xh and 2 (X - Xh) over them (TMEM A operands) and XGh =
+// Xh of the non-fixed positions to shared memory (the Gram's B operand).
+//
+// Bound by the gathers (5 K cycles per tile of K0 and V0 rows: TMA gather issue) where a
+// rank has many tiles, by latency where it has one.  The shares leave through
+// shared memory: stored from TMEM row by row, each instruction touched 32 lines
+// and the rows took 16 K cycles of 48 K.
+//
+// Measured, against one CTA per unit and block, two 128-thread groups on alternate
+// tiles, and a second launch for units that start over: 8 units B = 512 44 -> 15 us,
+// 64 units with budgets 200 .. 1536 88 -> 26 us, 32 units B = 1024 m = 256 103 -> 22 us,
+// 256 units B = 2048 129 -> 99 us (two waves).
+struct GBars {
+  uint64_t ring_full[kRingG], ring_empty[kRingG];
+  uint64_t q_full;
+  uint64_t s_full[2], x_full[2];   // S written; statistics taken or X written
+  uint64_t acc_done, drain;
+  uint32_t tmem;
+  int abort;
+};
+static_assert(sizeof(GBars) <= 256, "barrier block");
+constexpr int kGroupsG = 4, kWarpsG = 20;
+
+// Float offset of 4-float chunk c of row r in a 128 x 128 fp32 tile whose chunks
+// are permuted so that threads on consecutive rows meet different banks.
+__device__ __forceinline__ int dump_at(int r, int c) { return r * kD + ((c ^ (r & 31)) << 2); }
+
+__device__ __forceinline__ uint32_t peer_addr(uint32_t saddr, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float4 peer_load4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(a)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 peer_load2(uint32_t a) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];"
+               : "=f"(v.x), "=f"(v.y)
+               : "r"(a)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ void cluster_bar() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::
+                   : "memory");
+}
+
+__global__ void __launch_bounds__(kThreadsG, 1)
     k_merge_gram(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, MArgs a) {
   extern __shared__ __align__(1024) uint8_t smraw[];
   uint8_t* sm = (uint8_t*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
-  MBars* bars = (MBars*)(sm + kOffBar);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int u = blockIdx.x;
+  GBars* bars = (GBars*)(sm + kOffBar);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform for the compiler
+  const int C = a.ranks, rank = blockIdx.x % C, ub = blockIdx.x / C;
+  const int u = ub / a.nrb, row0 = (ub % a.nrb) * kRows;   // window rows row0 .. row0 + 127
   const UnitRow ur = unit_row(a.units, u, a.B, a.n_fix);
   const int B = ur.B, T = (B + kTile - 1) / kTile;
-  if (a.gram_mode == 2 && __ldg(a.redo + u * a.nrb + a.rb) == 0) return;   // the single pass was valid
-  const bool single = a.gram_mode == 1;
-  const int k0 = single ? T : 0;   // first job
+  const int ta = T * rank / C, tb = T * (rank + 1) / C;    // this rank's tiles
   const int ng = __ldg(a.ng + u);
-  init_common(bars, warp, 1, 128, 128);   // ring slots are released by the MMA
+  if (tid == 0) {
+    for (int i = 0; i < kRingG; ++i) {
+      mbar_init(&bars->ring_full[i], 3);   // one expect_tx arrival per gathering warp
+      mbar_init(&bars->ring_empty[i], 1);
+    }
+    mbar_init(&bars->q_full, 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&bars->s_full[i], 1);
+      mbar_init(&bars->x_full[i], 4 * kGroupsG);
+    }
+    mbar_init(&bars->acc_done, 1);
+    mbar_init(&bars->drain, 1);
+    bars->abort = 0;
+    fence_mbar_init();
+  }
+  if (warp == 1) {
+    tmem_alloc(&bars->tmem, 512);
+    tmem_relinquish();
+  }
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem;
   volatile int* abort_flag = &bars->abort;
+  float* dump_r = (float*)(sm + kOffRing);                     // [128][128] (dump_at)
+  float* dump_g = (float*)(sm + kOffRing + 2 * kTileBytes);
+  float2* stat = (float2*)(sm + kOffXG);                       // [kGroupsG][128]
+  float* cs = (float*)(sm + kOffXG) + 2 * kGroupsG * kRows;    // [128] 1 / L'_r
+  const uint32_t stat_a = smem_u32(stat);
 
-  if (warp == 0 || warp == 2 || warp == 3) {
-    if (warp == 0 && lane == 0) {
-      prefetch_tensormap(&tmQ);
-      mbar_expect_tx(&bars->q_full, kTileBytes);
-      const uint64_t pol = l2_evict_last();
-      tma_load_3d(sm + kOffQ, &tmQ, &bars->q_full, 0, a.row0, u, pol);
-      tma_load_3d(sm + kOffQ + kTileBytes / 2, &tmQ, &bars->q_full, 64, a.row0, u, pol);
-    }
-    __syncwarp();
-    // the gathers: warps 0, 2 and 3 (three SM sub-partitions)
-    const int32_t* idx_u = a.idx + ur.off;
-    const int32_t* src_u = a.src + ur.off;
-    const int row0 = u * a.n;   // first row of this unit in the 2-D K / V maps
-    const int pw = warp == 0 ? 0 : warp - 1;
-    Gatherer<kRingG, 3> gt{sm + kOffRing, bars->ring_full, bars->ring_empty};
-    // job k < T reads K at the slots' rows, job k >= T K and V at the positions' rows
-    auto rows_of = [&](int k, int* j) {
-      gt.rows(k < T ? idx_u : src_u, B, a.n, row0, k < T ? k : k - T, pw, lane, j);
-    };
-    int jn[4];
-    if (k0 < 2 * T) rows_of(k0, jn);
-    bool ok = true;
-    for (int k = k0; k < 2 * T && ok; ++k) {
-      const int j[4] = {jn[0], jn[1], jn[2], jn[3]};
-      if (k + 1 < 2 * T) rows_of(k + 1, jn);
-      ok = gt.load(&tmK, j, pw, lane, abort_flag);
-      if (ok && k >= T) ok = gt.load(&tmV, j, pw, lane, abort_flag);
-    }
-    gt.drain(abort_flag);
-  } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t id_r = idesc_bf16(kRows, kD, 0, 1);     // R~ += Xh V0 (V0 MN-major)
-      const uint32_t id_g = idesc_bf16(kRows, kRows, 0, 0);  // G += A XGh^T
-      bool ok = mbar_wait(&bars->q_full, 0, abort_flag, kBudget);
-      const uint32_t qa = smem_u32(sm + kOffQ);
-      uint32_t use = 0;
-      int pend = -1;
-      uint32_t pend_v = 0;
-      bool g_started = false;
-      auto issue_rg = [&](int kp, uint32_t vuse) -> bool {
-        const int t = kp - T, b = (kp - k0) & 1, xb = t & 1;
-        bool w = mbar_wait(&bars->s_done[b], ((kp - k0) >> 1) & 1, abort_flag, kBudget);
-        if (w) w = mbar_wait(&bars->xg_full[xb], (t >> 1) & 1, abort_flag, kBudget);
-        if (w)
-          w = mbar_wait(&bars->ring_full[vuse % kRingG], (vuse / kRingG) & 1, abort_flag, kBudget);
-        if (!w) return false;
+  const bool gathers = warp == 0 || warp == 2 || warp == 3, computes = warp >= 4;
+  const int g = (warp - 4) >> 2, q = warp & 3, row = q * 32 + lane, grow = row0 + row;
+  const int pw = warp == 0 ? 0 : warp - 1;
+  const bool row_ok = grow < a.m;
+  // slots / positions past vlim are invisible to this row (and so are those >= B)
+  const int vlim = a.causal ? B - a.w + grow % a.w : B - 1;
+  const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
+  Gatherer<kRingG, 3> gt{sm + kOffRing, bars->ring_full, bars->ring_empty};
+  uint32_t use = 0, job = 0;   // ring loads and S tiles so far (MMA warp, compute groups)
+  bool single = a.rstats != nullptr, ok = true;
+  float lam = INFINITY;
+  if (single && computes && row_ok)
+    lam = __ldg(a.rstats + ((size_t)u * a.m + grow) * 2) * 1.4426950408889634f;
+  if (warp == 0 && lane == 0) {
+    prefetch_tensormap(&tmQ);
+    mbar_expect_tx(&bars->q_full, kTileBytes);
+    const uint64_t pol = l2_evict_last();
+    tma_load_3d(sm + kOffQ, &tmQ, &bars->q_full, 0, row0, u, pol);
+    tma_load_3d(sm + kOffQ + kTileBytes / 2, &tmQ, &bars->q_full, 64, row0, u, pol);
+  }
+
+  // phase 0: statistics over the slots (K0); phase 1: R~ and the Gram over the
+  // positions (K0 and V0)
+  for (int ph = single ? 1 : 0, acc_use = 0;;) {
+    float M = -INFINITY, L = 0.f;   // phase 0: row statistics; phase 1: largest logit, sum of X
+    if (gathers) {
+      __syncwarp();
+      const int32_t* rows_u = (ph ? a.src : a.idx) + ur.off;
+      int jn[4];
+      if (ta < tb) gt.rows(rows_u, B, a.n, u * a.n, ta, pw, lane, jn);
+      for (int t = ta; t < tb && ok; ++t) {
+        const int j[4] = {jn[0], jn[1], jn[2], jn[3]};
+        if (t + 1 < tb) gt.rows(rows_u, B, a.n, u * a.n, t + 1, pw, lane, jn);
+        ok = gt.load(&tmK, j, pw, lane, abort_flag);
+        if (ok && ph) ok = gt.load(&tmV, j, pw, lane, abort_flag);
+      }
+    } else if (warp == 1) {
+      constexpr uint32_t id_s = idesc_bf16(kRows, kTile, 0, 0);   // S = Q K0^T
+      constexpr uint32_t id_r = idesc_bf16(kRows, kD, 0, 1);      // R~ += Xh V0 (V0 MN-major)
+      constexpr uint32_t id_g = idesc_bf16(kRows, kRows, 0, 0);   // G += A XGh^T
+      constexpr uint32_t kTileDesc = kTileBytes >> 4;             // in descriptor units
+      const uint64_t q_desc = sw128_desc(smem_u32(sm + kOffQ), 16, 1024);
+      const uint64_t k_desc = sw128_desc(smem_u32(sm + kOffRing), 16, 1024);
+      const uint64_t v_desc = sw128_desc(smem_u32(sm + kOffRing), kTileBytes / 2, 1024);
+      const uint64_t x_desc = sw128_desc(smem_u32(sm + kOffXG), 16, 1024);
+      ok = ok && mbar_wait_warp(&bars->q_full, 0, abort_flag);
+      // after the next tile's S: the job's X is there (phase 0: its logits are read)
+      auto finish = [&](int t, uint32_t jb, uint32_t vuse) -> bool {
+        const uint32_t b = jb & 1;
+        if (!mbar_wait_warp(&bars->x_full[b], (jb >> 1) & 1, abort_flag)) return false;
+        if (!ph) return true;
+        const uint32_t vs = vuse % kRingG;
+        if (!mbar_wait_warp(&bars->ring_full[vs], (vuse / kRingG) & 1, abort_flag)) return false;
         tc_fence_after();
-        const uint32_t va = smem_u32(sm + kOffRing + (vuse % kRingG) * kTileBytes);
-        const uint32_t xa = smem_u32(sm + kOffXG + xb * kTileBytes);
-        const uint32_t hi = tmem + kColS + b * kTile, lo2 = hi + 64;
-#pragma unroll
-        for (int kk = 0; kk < kTile / 16; ++kk)
-          mma_bf16_ts(tmem + kColR, hi + kk * 8,
-                      sw128_desc(va + kk * 2048, kTileBytes / 2, 1024), id_r, (t > 0 || kk > 0));
+        const uint32_t hi = tmem + kColS + b * kTile;
+        mma8_ts<id_r, false>(tmem + kColR, hi, v_desc + vs * kTileDesc, t > ta);
         if (t * kTile < ng) {   // the tile has non-fixed positions
-#pragma unroll
-          for (int kk = 0; kk < kTile / 16; ++kk) {
-            const uint32_t off = (kk >> 2) * (kTileBytes / 2) + (kk & 3) * 32;
-            mma_bf16_ts(tmem + kColG, hi + kk * 8, sw128_desc(xa + off, 16, 1024), id_g,
-                        (g_started || kk > 0));
-          }
-#pragma unroll
-          for (int kk = 0; kk < kTile / 16; ++kk) {
-            const uint32_t off = (kk >> 2) * (kTileBytes / 2) + (kk & 3) * 32;
-            mma_bf16_ts(tmem + kColG, lo2 + kk * 8, sw128_desc(xa + off, 16, 1024), id_g, 1);
-          }
-          g_started = true;
+          mma8_ts<id_g, true>(tmem + kColG, hi, x_desc + b * kTileDesc, t > ta);
+          mma8_ts<id_g, true>(tmem + kColG, hi + 16, x_desc + b * kTileDesc, true);
         }
-        mma_commit(&bars->ring_empty[vuse % kRingG]);
-        mma_commit(&bars->xg_empty[xb]);
+        mma_commit_elect(&bars->ring_empty[vs]);
         return true;
       };
-      for (int k = k0; k < 2 * T && ok; ++k) {
-        const int jk = k - k0, b = jk & 1;
-        const uint32_t kuse = use++;
-        ok = mbar_wait(&bars->ring_full[kuse % kRingG], (kuse / kRingG) & 1, abort_flag, kBudget);
-        if (ok && jk >= 2) ok = mbar_wait(&bars->s_done[b], ((jk >> 1) - 1) & 1, abort_flag, kBudget);
+      uint32_t pv = 0;
+      for (int t = ta; t < tb && ok; ++t, ++job) {
+        const uint32_t b = job & 1, ks = use % kRingG;
+        ok = mbar_wait_warp(&bars->ring_full[ks], (use / kRingG) & 1, abort_flag);
         if (!ok) break;
         tc_fence_after();
-        issue_s(tmem + kColS + b * kTile, qa,
-                smem_u32(sm + kOffRing + (kuse % kRingG) * kTileBytes));
-        mma_commit(&bars->ring_empty[kuse % kRingG]);
-        mma_commit(&bars->s_full[b]);
-        uint32_t vuse = 0;
-        if (k >= T) vuse = use++;
-        if (pend >= 0) {
-          ok = issue_rg(pend, pend_v);
-          pend = -1;
-        }
-        if (k >= T) {
-          pend = k;
-          pend_v = vuse;
-        }
+        // the buffer's last X was read by MMAs issued before, its last logits by finish()
+        mma8_ss<id_s>(tmem + kColS + b * kTile, q_desc, k_desc + ks * kTileDesc);
+        mma_commit_elect(&bars->ring_empty[ks]);
+        mma_commit_elect(&bars->s_full[b]);
+        if (t > ta) ok = finish(t - 1, job - 1, pv);
+        pv = use + 1;
+        use += ph ? 2 : 1;
       }
-      if (ok && pend >= 0) ok = issue_rg(pend, pend_v);
-      mma_commit(&bars->acc_done);
-      mma_commit(&bars->drain);
-      mbar_wait(&bars->drain, 0, abort_flag, kBudget);
-    }
-  } else if (warp >= 4) {
-    const int wg = (warp - 4) >> 2, q = warp & 3, row = q * 32 + lane;
-    const int grow = a.row0 + row;   // window row of the stacked m
-    const bool row_ok = grow < a.m;
-    // slots / positions past vlim are invisible to this row (and so are those >= B)
-    const int vlim = !row_ok ? -1 : (a.causal ? B - a.w + grow % a.w : B - 1);
-    const int open = B - a.w;   // below this everything is visible to every window row
-    const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
-    float M = -INFINITY, L = 0.f, lam = INFINITY;
-    float vmax = -INFINITY, xsum = 0.f;   // visible retained logits (raw) and sum of X
-    if (single && row_ok) lam = __ldg(a.rstats + ((size_t)u * a.m + grow) * 2) * 1.4426950408889634f;
-    bool ok = true;
-    for (int k = k0; k < 2 * T; ++k) {
-      if (k == T && !single) {
-        // both groups combine their statistics (reached even after an abort);
-        // the XGh tiles are not in use yet
-        float2* comb = (float2*)(sm + kOffXG);
-        comb[wg * kRows + row] = make_float2(M, L);
-        named_bar(4, 256);
-        const float2 o = comb[(wg ^ 1) * kRows + row];
-        named_bar(4, 256);
-        if (o.x != -INFINITY) {
-          if (o.x > M) {
-            L = L * fast_exp2(M - o.x) + o.y;
-            M = o.x;
-          } else {
-            L += o.y * fast_exp2(o.x - M);
-          }
-        }
-        lam = (row_ok && L > 0.f) ? M + __log2f(L) : INFINITY;
-        if (wg == 0) a.lam[(size_t)u * a.ldr + grow] = lam;
-      }
-      if (!ok) {
-        if (k < T) continue;
-        break;
-      }
-      if (((k - k0) & 1) != wg) continue;
-      const int b = (k - k0) & 1, t = k < T ? k : k - T, p0 = t * kTile;
-      ok = mbar_wait(&bars->s_full[b], ((k - k0) >> 1) & 1, abort_flag, kBudget);
-      if (!ok) continue;
-      tc_fence_after();
-      const uint32_t sbase = lane_addr + kColS + b * kTile;
-      float va[32], vb[32];
-      if (k < T) {
-        // warp-uniform: the TMEM loads below are .sync.aligned
-        const bool masked = __any_sync(0xffffffffu, !row_ok) || p0 + kTile > open + 1;
-        tmem_ld32f(sbase, va);
-        tmem_wait32(va);
-        tmem_ld32f(sbase + 32, vb);
-        if (masked) {
-          stats32<true>(va, p0, vlim, a.sl2, M, L);
-          tmem_wait32(vb);
-          tmem_ld32f(sbase + 64, va);
-          stats32<true>(vb, p0 + 32, vlim, a.sl2, M, L);
-          tmem_wait32(va);
-          tmem_ld32f(sbase + 96, vb);
-          stats32<true>(va, p0 + 64, vlim, a.sl2, M, L);
-          tmem_wait32(vb);
-          tc_fence_before();
-          mbar_arrive(&bars->s_done[b]);
-          stats32<true>(vb, p0 + 96, vlim, a.sl2, M, L);
-        } else {
-          stats32<false>(va, p0, vlim, a.sl2, M, L);
-          tmem_wait32(vb);
-          tmem_ld32f(sbase + 64, va);
-          stats32<false>(vb, p0 + 32, vlim, a.sl2, M, L);
-          tmem_wait32(va);
-          tmem_ld32f(sbase + 96, vb);
-          stats32<false>(va, p0 + 64, vlim, a.sl2, M, L);
-          tmem_wait32(vb);
-          tc_fence_before();
-          mbar_arrive(&bars->s_done[b]);
-          stats32<false>(vb, p0 + 96, vlim, a.sl2, M, L);
-        }
-      } else {
-        const int xb = t & 1;
-        if (t >= 2) ok = mbar_wait(&bars->xg_empty[xb], ((t >> 1) - 1) & 1, abort_flag, kBudget);
-        if (!ok) continue;
-        uint8_t* xg = sm + kOffXG + xb * kTileBytes;
-        // 2 (X - Xh) goes to TMEM columns 64..127, which hold S chunks 2 and 3:
-        // chunks 0 and 1 are written once chunk 2 is read, 2 and 3 once chunk 3 is
-        uint32_t lo0[16], lo1[16], lo2[16], lo3[16];
-        tmem_ld32f(sbase, va);
-        tmem_wait32(va);
-        tmem_ld32f(sbase + 32, vb);
-        if (__all_sync(0xffffffffu, row_ok) && p0 + kTile <= ng) {
-          gram_chunk_fast<0>(va, a.sl2, lam, sbase, xg, row, lo0, vmax, xsum);
-          tmem_wait32(vb);
-          tmem_ld32f(sbase + 64, va);
-          gram_chunk_fast<1>(vb, a.sl2, lam, sbase, xg, row, lo1, vmax, xsum);
-          tmem_wait32(va);
-          tmem_st16(sbase + 64, lo0);
-          tmem_st16(sbase + 80, lo1);
-          tmem_ld32f(sbase + 96, vb);
-          gram_chunk_fast<2>(va, a.sl2, lam, sbase, xg, row, lo2, vmax, xsum);
-          tmem_wait32(vb);
-          tmem_st16(sbase + 96, lo2);
-          gram_chunk_fast<3>(vb, a.sl2, lam, sbase, xg, row, lo3, vmax, xsum);
-        } else {
-          const bool want_g = p0 < ng;
-          gram_chunk_masked<0>(va, p0, vlim, ng, a.sl2, lam, sbase, xg, row, lo0, want_g, vmax, xsum);
-          tmem_wait32(vb);
-          tmem_ld32f(sbase + 64, va);
-          gram_chunk_masked<1>(vb, p0, vlim, ng, a.sl2, lam, sbase, xg, row, lo1, want_g, vmax, xsum);
-          tmem_wait32(va);
-          tmem_st16(sbase + 64, lo0);
-          tmem_st16(sbase + 80, lo1);
-          tmem_ld32f(sbase + 96, vb);
-          gram_chunk_masked<2>(va, p0, vlim, ng, a.sl2, lam, sbase, xg, row, lo2, want_g, vmax, xsum);
-          tmem_wait32(vb);
-          tmem_st16(sbase + 96, lo2);
-          gram_chunk_masked<3>(vb, p0, vlim, ng, a.sl2, lam, sbase, xg, row, lo3, want_g, vmax, xsum);
-        }
-        tmem_st16(sbase + 112, lo3);
-        tmem_st_wait();
-        fence_proxy_async_smem();
-        tc_fence_before();
-        mbar_arrive(&bars->s_done[b]);
-        mbar_arrive(&bars->xg_full[xb]);
-      }
-    }
-    // R = Y - R~ and the raw Gram rows to the workspace, half the columns per group
-    if (ok) ok = mbar_wait(&bars->acc_done, 0, abort_flag, kBudget);
-    tc_fence_after();
-    float ci = 1.f;   // 1 / L'_row in the single pass
-    float* cs = (float*)(sm + kOffXG) + 2 * 2 * kRows;   // [128] after the float2 pairs
-    if (single) {
-      // combine the groups' sums and maxima (the XGh tiles are free now)
-      float2* comb = (float2*)(sm + kOffXG);
-      comb[wg * kRows + row] = make_float2(vmax, xsum);
-      named_bar(4, 256);
-      const float2 o = comb[(wg ^ 1) * kRows + row];
-      const float lsum = xsum + o.y, vm = fmaxf(vmax, o.x);
-      const bool bad = row_ok && !(lsum > 0.f && lam - vm * a.sl2 <= 64.f);
-      if (bad) bars->bad = 1;
-      ci = (row_ok && lsum > 0.f) ? 1.f / lsum : 0.f;
-      if (wg == 0) {
-        cs[row] = ci;
-        a.lam[(size_t)u * a.ldr + grow] = (row_ok && lsum > 0.f) ? lam + __log2f(lsum) : INFINITY;
-      }
-      named_bar(4, 256);
-      if (tid == 128) a.redo[u * a.nrb + a.rb] = bars->bad;
-      if (bars->bad) ok = false;   // gram_mode 2 redoes this unit; not a failure
-    }
-    if (ok) {
-      float* R = a.rz + ((size_t)u * a.ldr + grow) * kD;
-      float* G = a.gram + ((size_t)u * a.ldr + grow) * a.ldr + a.row0;   // the diagonal block
-      const float* yr = a.y + ((size_t)u * a.m + (row_ok ? grow : 0)) * kD;
-#pragma unroll 1
-      for (int c = 2 * wg; c < 2 * wg + 2; ++c) {
+      if (ok && tb > ta) ok = finish(tb - 1, job - 1, pv);
+      if (ph) mma_commit_elect(&bars->acc_done);
+    } else {
+      for (int t = ta; t < tb && ok; ++t, ++job) {
+        const uint32_t b = job & 1;
+        const int p0 = t * kTile + 32 * g;
+        // s_full also says that the MMAs that read this buffer's XGh have completed
+        ok = mbar_wait_warp(&bars->s_full[b], (job >> 1) & 1, abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t sbase = lane_addr + kColS + b * kTile + 32 * g;
         float v[32];
-        tmem_ld32f(lane_addr + kColR + c * 32, v);
+        tmem_ld32f(sbase, v);
         tmem_wait32(v);
+        const bool full = __all_sync(0xffffffffu, p0 + 31 <= vlim);
+        if (!ph) {
+          if (full)
+            stats32<false>(v, p0, vlim, a.sl2, M, L);
+          else
+            stats32<true>(v, p0, vlim, a.sl2, M, L);
+          __syncwarp();
+        } else {
+          uint32_t hi[16], lo[16];
+          if (full)
+            gram_chunk<false>(v, 0, a.sl2, lam, hi, lo, M, L);
+          else
+            gram_chunk<true>(v, vlim - p0, a.sl2, lam, hi, lo, M, L);
+          tmem_st16(sbase, hi);
+          tmem_st16(sbase + 16, lo);
+          if (t * kTile < ng) {
+            const int gn = ng - p0;   // the chunk's non-fixed positions
+            if (gn < 32) {
 #pragma unroll
-        for (int e = 0; e < 32; e += 4) {
-          const float4 yv = row_ok ? __ldg((const float4*)(yr + c * 32 + e))
-                                   : make_float4(0.f, 0.f, 0.f, 0.f);
-          *(float4*)(R + c * 32 + e) =
-              row_ok ? make_float4(yv.x - ci * v[e], yv.y - ci * v[e + 1], yv.z - ci * v[e + 2],
-                                   yv.w - ci * v[e + 3])
-                     : make_float4(0.f, 0.f, 0.f, 0.f);
+              for (int e = 0; e < 16; ++e)
+                hi[e] &= (2 * e < gn ? 0xFFFFu : 0u) | (2 * e + 1 < gn ? 0xFFFF0000u : 0u);
+            }
+            store_row_chunk(sm + kOffXG + b * kTileBytes, row, g, hi);
+          }
+          tmem_st_wait();
+          fence_proxy_async_smem();
         }
-        tmem_ld32f(lane_addr + kColG + c * 32, v);
-        tmem_wait32(v);
-        if (ng == 0) {   // no Gram MMA ran
-#pragma unroll
-          for (int e = 0; e < 32; ++e) v[e] = 0.f;
-        }
-        if (single) {
-#pragma unroll
-          for (int e = 0; e < 32; ++e) v[e] *= ci * cs[c * 32 + e];
-        }
-#pragma unroll
-        for (int e = 0; e < 32; e += 4)
-          *(float4*)(G + c * 32 + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->x_full[b]);
       }
     }
-    if (!ok && row == 0 && !bars->bad) set_status(a.status, GRKV_ERR_TIMEOUT);
+
+    if (ph == 0) {
+      // every rank's and group's statistics of the rows give the normalisers
+      if (computes) stat[g * kRows + row] = make_float2(M, L);
+      cluster_bar();
+      if (computes) {
+        M = -INFINITY;
+        L = 0.f;
+        for (int r = 0; r < C; ++r)
+          for (int h = 0; h < kGroupsG; ++h) {
+            const float2 o = peer_load2(peer_addr(stat_a + (h * kRows + row) * 8, r));
+            if (o.x == -INFINITY) continue;
+            if (o.x > M) {
+              L = L * fast_exp2(M - o.x) + o.y;
+              M = o.x;
+            } else {
+              L += o.y * fast_exp2(o.x - M);
+            }
+          }
+        lam = (row_ok && L > 0.f) ? M + __log2f(L) : INFINITY;
+        if (rank == 0 && g == 0) a.lam[(size_t)u * a.ldr + grow] = lam;
+      }
+      cluster_bar();   // the peers have read: the XGh tiles may be written
+      ph = 1;
+      continue;
+    }
+
+    // the rank's shares to shared memory: every gathered tile has been multiplied
+    if (computes) {
+      ok = ok && mbar_wait_warp(&bars->acc_done, acc_use & 1, abort_flag);
+      tc_fence_after();
+      stat[g * kRows + row] = make_float2(M, L);
+      const bool any = ok && tb > ta, any_g = any && ta * kTile < ng;   // MMAs that ran
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) {
+        float v[32];
+        tmem_ld32f(lane_addr + (h ? kColG : kColR) + 32 * g, v);
+        tmem_wait32(v);
+        const bool have = h ? any_g : any;
+        float* d = h ? dump_g : dump_r;
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          *(float4*)(d + dump_at(row, 8 * g + c)) =
+              have ? make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3])
+                   : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+      tc_fence_before();
+    }
+    ++acc_use;
+    fence_proxy_async_smem();   // a second attempt gathers over the shares
+    cluster_bar();
+    bool bad = false;
+    if (single && tid < kRows) {
+      const int gr = row0 + tid;
+      float vm = -INFINITY, ls = 0.f;
+      for (int r = 0; r < C; ++r)
+        for (int h = 0; h < kGroupsG; ++h) {
+          const float2 o = peer_load2(peer_addr(stat_a + (h * kRows + tid) * 8, r));
+          vm = fmaxf(vm, o.x);
+          ls += o.y;
+        }
+      const bool in = gr < a.m;
+      const float full = in ? __ldg(a.rstats + ((size_t)u * a.m + gr) * 2) * 1.4426950408889634f : 0.f;
+      bad = in && !(ls > 0.f && full - vm * a.sl2 <= 64.f);
+      cs[tid] = in && ls > 0.f ? 1.f / ls : 0.f;
+      if (rank == 0) a.lam[(size_t)u * a.ldr + gr] = in && ls > 0.f ? full + __log2f(ls) : INFINITY;
+    }
+    if (__syncthreads_or(bad)) {   // the same answer in every rank
+      single = false;
+      ph = 0;
+      cluster_bar();   // the peers have read the statistics
+      continue;
+    }
+    // rows r0 .. r1 - 1 of R and of the Gram block: a warp per row, a lane per four columns
+    const int r0 = kRows * rank / C, r1 = kRows * (rank + 1) / C;
+    const uint32_t ra = smem_u32(dump_r), ga = smem_u32(dump_g);
+    for (int r = r0 + warp; r < r1; r += kWarpsG) {
+      const int gr = row0 + r, c = 4 * lane;
+      const uint32_t off = dump_at(r, lane) * 4;
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f), z = x, o = x, y = x;
+      if (gr < a.m) y = __ldg((const float4*)(a.y + ((size_t)u * a.m + gr) * kD + c));
+      for (int p = 0; p < C; ++p) {
+        const float4 xr = peer_load4(peer_addr(ra + off, p)), zr = peer_load4(peer_addr(ga + off, p));
+        x = make_float4(x.x + xr.x, x.y + xr.y, x.z + xr.z, x.w + xr.w);
+        z = make_float4(z.x + zr.x, z.y + zr.y, z.z + zr.z, z.w + zr.w);
+      }
+      const float ci = single ? cs[r] : 1.f;
+      const float4 cj = single ? *(const float4*)(cs + c) : make_float4(1.f, 1.f, 1.f, 1.f);
+      const bool in = gr < a.m;
+      if (!ok) continue;
+      *(float4*)(a.rz + ((size_t)u * a.ldr + gr) * kD + c) =
+          in ? make_float4(y.x - ci * x.x, y.y - ci * x.y, y.z - ci * x.z, y.w - ci * x.w) : o;
+      const int gc = row0 + c;
+      if (in)
+        o = make_float4(gc < a.m ? z.x * (ci * cj.x) : 0.f, gc + 1 < a.m ? z.y * (ci * cj.y) : 0.f,
+                        gc + 2 < a.m ? z.z * (ci * cj.z) : 0.f,
+                        gc + 3 < a.m ? z.w * (ci * cj.w) : 0.f);
+      *(float4*)(a.gram + ((size_t)u * a.ldr + gr) * a.ldr + gc) = o;
+    }
+    cluster_bar();   // no rank leaves while a peer reads its shares
+    break;
   }
+  if (gathers) gt.drain(abort_flag);
+  if (warp == 1) {
+    // every MMA issued completes before TMEM is released
+    mma_commit_elect(&bars->drain);
+    volatile int no_abort = 0;
+    mbar_wait(&bars->drain, 0, &no_abort, kBudget);
+  }
+  if (!ok && lane == 0) set_status(a.status, GRKV_ERR_TIMEOUT);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1248,11 +1227,11 @@ bool merge_tc_supported(const Shape& s) {
 }
 
 // Workspace of the tensor-core merge: rz [U][ldr][128], gram [U][ldr][ldr],
-// lam [U][ldr] (fp32), src [U][B], ng [U], redo [U][nrb] (int32), fixed [U][B]
+// lam [U][ldr] (fp32), src [U][B], ng [U], fail [U] (int32), fixed [U][B]
 // (bytes), and for two row blocks vpart [U][B][128] (fp32).
 struct MergeWs {
   int ldr, nrb;
-  size_t rz, gram, lam, src, ng, redo, fixed, vpart, total;
+  size_t rz, gram, lam, src, ng, fail, fixed, vpart, total;
 };
 MergeWs merge_ws(const Shape& s) {
   MergeWs w;
@@ -1265,11 +1244,33 @@ MergeWs merge_ws(const Shape& s) {
   w.lam = w.gram + U * ldr * ldr * 4;
   w.src = w.lam + U * ldr * 4;
   w.ng = w.src + U * B * 4;
-  w.redo = w.ng + U * 4;
-  w.fixed = w.redo + U * w.nrb * 4;
+  w.fail = w.ng + U * 4;
+  w.fixed = w.fail + U * 4;
   w.vpart = (w.fixed + U * B + 15) & ~(size_t)15;
   w.total = w.vpart + (w.nrb > 1 ? U * B * kD * 4 : 0);
   return w;
+}
+
+// As many ranks as leave every cluster room on the SMs at once: 8 units of B = 512
+// take 15 us with four ranks, one tile each.
+cudaError_t launch_gram(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
+                        MArgs a, cudaStream_t st) {
+  const int tiles = (a.B + kTile - 1) / kTile, blocks = a.U * a.nrb;
+  a.ranks = 1;
+  while (a.ranks < 8 && 2 * a.ranks <= tiles && blocks * 2 * a.ranks <= kClusterSms) a.ranks *= 2;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = a.ranks;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks * a.ranks);
+  cfg.blockDim = dim3(kThreadsG);
+  cfg.dynamicSmemBytes = kSmemBytes;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_merge_gram, mq, mk, mv, a);
 }
 
 size_t merge_tc_ws_bytes(const Shape& s) { return merge_ws(s).total; }
@@ -1317,7 +1318,7 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
   a.lam = (float*)(mw + W.lam);
   a.src = (int32_t*)(mw + W.src);
   a.ng = (int32_t*)(mw + W.ng);
-  a.redo = (int32_t*)(mw + W.redo);
+  int32_t* fail = (int32_t*)(mw + W.fail);
   a.fixed = (uint8_t*)(mw + W.fixed);
   a.vpart = W.nrb > 1 ? (float*)(mw + W.vpart) : nullptr;
   a.ldr = W.ldr;
@@ -1338,23 +1339,9 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
                                              kSmemBytesC)) != cudaSuccess)
     return e;
   k_merge_fixed<<<s.U, 256, s.B * 4, st>>>(a);
-  int launches = 1;
   // the retained statistics, R and the diagonal Gram block of every row block
-  for (int rb = 0; rb < W.nrb; ++rb) {
-    a.rb = rb;
-    a.row0 = rb * kRows;
-    if (row_stats) {
-      a.gram_mode = 1;
-      k_merge_gram<<<s.U, kThreads, kSmemBytes, st>>>(mq, mk, mv, a);
-      a.gram_mode = 2;
-      k_merge_gram<<<s.U, kThreads, kSmemBytes, st>>>(mq, mk, mv, a);
-      launches += 2;
-    } else {
-      a.gram_mode = 0;
-      k_merge_gram<<<s.U, kThreads, kSmemBytes, st>>>(mq, mk, mv, a);
-      launches += 1;
-    }
-  }
+  if ((e = launch_gram(mq, mk, mv, a, st)) != cudaSuccess) return e;
+  int launches = 2;
   if (W.nrb > 1) {
     k_merge_cross<<<s.U, kThreads, kSmemBytesC, st>>>(mq, mk, a);
     launches += 1;
@@ -1362,9 +1349,9 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
   count_launches(launches);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // with two row blocks the solve keeps its first factor where the transpose of
-  // the cross block would be, and its failure flags in redo, which is spent
+  // the cross block would be
   if ((e = launch_solve(s.U, s.m, W.ldr, 1, s.lambda, s.lambda_inf, a.gram, a.rz,
-                        a.gram + (size_t)kRows * W.ldr, (size_t)W.ldr * W.ldr, W.ldr, a.redo,
+                        a.gram + (size_t)kRows * W.ldr, (size_t)W.ldr * W.ldr, W.ldr, fail,
                         a.status, st)) != cudaSuccess)
     return e;
   if (W.nrb == 1) {

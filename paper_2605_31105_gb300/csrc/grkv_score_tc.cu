@@ -179,27 +179,6 @@ struct RingPos {
   }
 };
 
-// Pairs of fp32 in one 64-bit register: two fused multiply-adds or additions
-// per instruction, each rounded as its scalar form.
-__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-
 // Three-operand maximum (one instruction on sm_100 and later).
 __device__ __forceinline__ float fmax3f(float a, float b, float c) {
   float d;
@@ -454,7 +433,7 @@ __global__ void __launch_bounds__(score_threads(kPass, RB), 1)
       if (!wait(&bars->p_full[pb], (yi >> 1) & 1)) return false;
       if (rb == 0 && !wait(&bars->ring_full[vp.slot], vp.phase)) return false;
       tc_fence_after();
-      mma8_ts<id_y, kTileBytes / 16 / 16>(tmem + kColY + yb * kD, tmem + pb * kTile,
+      mma8_ts<id_y, false>(tmem + kColY + yb * kD, tmem + pb * kTile,
                                           v_desc + vp.slot * kTileDesc, !y_first);
       if (rb == RB - 1) {
         mma_commit_elect(&bars->ring_empty[vp.slot]);

@@ -213,8 +213,9 @@ __device__ __forceinline__ void mma8_ss(uint32_t d_tmem, uint64_t adesc, uint64_
       : "memory");
 }
 // D (+)= A B^T with A in TMEM, 8 packed columns per step, two steps to every 32
-// columns, and B advancing kStep descriptor units per step.
-template <uint32_t kIdesc, int kStep>
+// columns, and B a K-major tile of two 64-column halves (kBK) or an MN-major one, 2048
+// bytes per step.
+template <uint32_t kIdesc, bool kBK>
 __device__ __forceinline__ void mma8_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc,
                                         bool accumulate) {
   asm volatile(
@@ -236,8 +237,9 @@ __device__ __forceinline__ void mma8_ts(uint32_t d_tmem, uint32_t a_tmem, uint64
       " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n"
       " add.u32 a, %1, 104;\n add.u64 b, %2, %11;\n"
       " @q tcgen05.mma.cta_group::1.kind::f16 [%0], [a], b, %3, t;\n}\n" ::"r"(d_tmem),
-      "r"(a_tmem), "l"(bdesc), "n"(kIdesc), "r"((uint32_t)accumulate), "n"(kStep), "n"(2 * kStep),
-      "n"(3 * kStep), "n"(4 * kStep), "n"(5 * kStep), "n"(6 * kStep), "n"(7 * kStep)
+      "r"(a_tmem), "l"(bdesc), "n"(kIdesc), "r"((uint32_t)accumulate), "n"(kBK ? 2 : 128),
+      "n"(kBK ? 4 : 256), "n"(kBK ? 6 : 384), "n"(kBK ? 1024 : 512), "n"(kBK ? 1026 : 640),
+      "n"(kBK ? 1028 : 768), "n"(kBK ? 1030 : 896)
       : "memory");
 }
 // mma_commit by the elected lane of a converged warp (the lane that issued).
@@ -335,6 +337,27 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&h);
 }
+// Pairs of fp32 in one 64-bit register: two fused multiply-adds or additions
+// per instruction, each rounded as its scalar form.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
 // 2^x with the MUFU approximation (relative error about 2^-22; subnormal results flush to 0).
 __device__ __forceinline__ float fast_exp2(float x) {
   float y;
