@@ -4,7 +4,8 @@
 // k_select_reg holds a unit's pooled scores as order-preserving keys in
 // registers, kPer consecutive positions per thread, over one CTA of 1024 threads
 // (n - w <= 32768) or a cluster of 8 (up to 262144).  The cut is the kk-th
-// largest key: its sign and exponent by nine counting steps (a ballot of the
+// largest key, found among the few keys above a sampled bound where that pays, else
+// over all keys: its sign and exponent by nine counting steps (a ballot of the
 // whole block each, no histogram: almost every key shares a few exponents,
 // which serialises shared atomics), its mantissa by three histogram passes
 // over the keys that share them; one scan of (above, equal) counts places the
@@ -164,6 +165,8 @@ __device__ __forceinline__ void cluster_bar() {
                    : "memory");
 }
 
+constexpr int kSamples = 256;   // keys that place the candidates' bound
+
 struct SelSmem {
   int hist[kReps][256];
   int sum[3][256];        // a pass's histogram (read by the peers of a cluster)
@@ -172,6 +175,9 @@ struct SelSmem {
   int scan[kWarps];
   int scan_tot[2][kCluster];   // keys above the cut and equal to it, per CTA
   int digit, left;
+  uint32_t samp[kSamples];
+  uint32_t bound;
+  int cand_tot[kCluster];   // candidates per CTA
 };
 
 template <int kPer, int kCs>
@@ -213,10 +219,15 @@ __global__ void __launch_bounds__(kThr, 1) k_select_reg(const float* __restrict_
   if (s.pool_type == GRKV_POOL_MAX && h == 3) {
     // window max over w[e .. e + 6] from pairs and quadruples (cells outside [0, P) ignored)
     float w[kPer + 6];
+    if (lo >= 3 && lo + kPer + 3 <= P) {
 #pragma unroll
-    for (int i = 0; i < kPer + 6; ++i) {
-      const int j = lo - 3 + i;
-      w[i] = (j >= 0 && j < P) ? at(j) : -INFINITY;
+      for (int i = 0; i < kPer + 6; ++i) w[i] = at(lo - 3 + i);
+    } else {
+#pragma unroll
+      for (int i = 0; i < kPer + 6; ++i) {
+        const int j = lo - 3 + i;
+        w[i] = (j >= 0 && j < P) ? at(j) : -INFINITY;
+      }
     }
     float m2[kPer + 5], m4[kPer + 3];
 #pragma unroll
@@ -250,6 +261,115 @@ __global__ void __launch_bounds__(kThr, 1) k_select_reg(const float* __restrict_
     }
   }
   const int valid = max(0, min(kPer, P - lo));   // positions of this thread inside the prefix
+  // Candidates: the keys at or above a bound that kSamples evenly spaced keys place a little
+  // below the cut (three standard deviations of the sample's count, so the cut is nearly
+  // always among them).  They are a few times kk keys, written in order of position to
+  // shared memory (of the cluster's first CTA), and the exact cut is found among them.
+  // Too few or too many (an unlucky sample, ties) leave it to the steps below, over all keys.
+  // Only where a thread has 32 keys or every step spans a cluster: 256 units n - w = 32736
+  // 51 -> 36 us, 32 of 131,008 95 -> 51 us; with 16 or fewer keys a thread in one CTA the
+  // steps over all keys are as fast or faster (n - w = 16352 18.2 us either way, 8160 13 against 15).
+  constexpr bool kCandidates = kPer * kCs >= 32;
+  constexpr int kCap = kThr * kPer / 2;   // key and position per candidate, over the scores
+  if (kCandidates && kk < kCap) {
+    constexpr int kOwn = kSamples / kCs, kStride = kThr / kOwn;   // one sample every kStride threads
+    if (tid % kStride == 0) {
+      const uint32_t x = valid > 0 ? kr[0] : 0u;
+      const int at_s = rank * kOwn + tid / kStride;
+      if (kCs > 1) {
+#pragma unroll
+        for (int q = 0; q < kCs; ++q) peer_store(peer_addr(&sh.samp[at_s], q), (int)x);
+      } else {
+        sh.samp[at_s] = x;
+      }
+    }
+    if (kCs > 1)
+      cluster_bar();
+    else
+      __syncthreads();
+    if (warp == 0) {
+      const int nv = min(kSamples, (P + kStride * kPer - 1) / (kStride * kPer));   // inside the prefix
+      const float q = (float)kk * (float)nv / (float)P;   // samples above the cut, on average
+      const int r = (int)(q + 3.f * sqrtf(q) + 5.f);
+      uint32_t x[kSamples / 32], bound = 0;
+#pragma unroll
+      for (int i = 0; i < kSamples / 32; ++i) x[i] = sh.samp[i * 32 + lane];
+      if (r < nv) {
+        // the r-th largest sample to its 18 leading bits
+        for (int bit = 31; bit >= 14; --bit) {
+          const uint32_t cand = bound | 1u << bit;
+          int n = 0;
+#pragma unroll
+          for (int i = 0; i < kSamples / 32; ++i) n += x[i] >= cand;
+          if (__reduce_add_sync(0xffffffffu, n) >= r) bound = cand;
+        }
+      }
+      if (lane == 0) sh.bound = bound;
+    }
+    __syncthreads();
+    const uint32_t bound = sh.bound;
+    int mine = 0;
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) mine += e < valid && kr[e] >= bound;
+    int total;
+    int at_c = block_exclusive_scan(mine, sh.scan, &total);
+    if (kCs > 1) {
+      if (tid < kCs) peer_store(peer_addr(&sh.cand_tot[rank], tid), total);
+      cluster_bar();
+      total = 0;
+#pragma unroll
+      for (int q = 0; q < kCs; ++q) {
+        if (q < rank) at_c += sh.cand_tot[q];
+        total += sh.cand_tot[q];
+      }
+    }
+    if (total >= kk && total <= kCap) {   // the same answer in every CTA of the cluster
+      uint32_t* ck = (uint32_t*)sc;       // keys, then positions: the scores are spent
+      uint32_t* cp = ck + kCap;
+      const uint32_t k_at = peer_addr(ck, 0), p_at = peer_addr(cp, 0);
+#pragma unroll
+      for (int e = 0; e < kPer; ++e) {
+        if (e < valid && kr[e] >= bound) {
+          if (kCs > 1) {
+            peer_store(k_at + 4 * at_c, (int)kr[e]);
+            peer_store(p_at + 4 * at_c, lo + e);
+          } else {
+            ck[at_c] = kr[e];
+            cp[at_c] = (uint32_t)(lo + e);
+          }
+          ++at_c;
+        }
+      }
+      if (kCs > 1) {
+        cluster_bar();
+        if (rank != 0) return;
+      } else {
+        __syncthreads();
+      }
+      uint32_t tau;
+      int need_eq;
+      block_kth_largest(
+          [&](int i, uint32_t* key) {
+            *key = ck[i];
+            return true;
+          },
+          total, kk, sh.hist[0], sh.scan, &tau, &need_eq);
+      const int seg = (total + kThr - 1) / kThr;
+      const int i0 = min(total, tid * seg), i1 = min(total, i0 + seg);
+      int cnt = 0;   // above the cut (low half), equal to it
+      for (int i = i0; i < i1; ++i) cnt += ck[i] > tau ? 1 : ck[i] == tau ? 1 << 16 : 0;
+      int all;
+      const int pre = block_exclusive_scan(cnt, sh.scan, &all);
+      int gt = pre & 0xFFFF, eq = pre >> 16;
+      for (int i = i0; i < i1; ++i) {
+        const uint32_t x = ck[i];
+        if (x > tau || (x == tau && eq < need_eq)) out[gt + min(eq, need_eq)] = (int)cp[i];
+        gt += x > tau;
+        eq += x == tau;
+      }
+      return;
+    }
+  }
   // sign and exponent: the largest prefix with at least kk keys at or above it
   uint32_t prefix = 0;
   int above = 0;   // keys at or past the upper end of the prefix's range

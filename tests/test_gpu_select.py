@@ -59,3 +59,20 @@ def test_pooling_widths(grkv_lib, P, pool, kind):
 def test_budget_edges(grkv_lib, P, kk):
     s = _scores(np.random.default_rng(P), P, "ties")
     _check(P, 16, 0 if kk == "none" else P, 7, "max", s)
+
+
+@pytest.mark.parametrize("P,stride", [(32768, 128), (30000, 128), (65536, 256), (131072, 512)])
+@pytest.mark.parametrize("sampled", ["high", "low", "half"])
+def test_misleading_sample(grkv_lib, P, stride, sampled):
+    """The keys that place the candidates' bound (every `stride`-th position) lie above all
+    others (too few candidates), below them (too many), or the cut falls among them."""
+    rng = np.random.default_rng(P + len(sampled))
+    s = (1 + rng.random((2, P))).astype(np.float32)
+    if sampled == "high":
+        s[:, ::stride] += 100
+    elif sampled == "low":
+        s[:, ::stride] *= 1e-6
+    else:
+        s[:, ::stride] += 0.95
+    for kk in (1, P // stride, P // 20, P // 20 + 1):
+        _check(P, 8, kk, 1, "max", s)
