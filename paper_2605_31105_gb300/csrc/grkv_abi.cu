@@ -124,6 +124,7 @@ int make_shape(const grkv_params* p, Shape* s) {
   s->steps = p->steps;
   s->step_tol = p->step_tol;
   s->lambda_k = p->lambda_k;
+  s->chained = false;
   s->units = nullptr;
   s->rows = 0;
   return GRKV_OK;
@@ -288,6 +289,7 @@ int grkv_compress(const grkv_params* p, const void* q, const void* k, const void
   float* rstats = (float*)(w + L.rstats);
   if (s.checks) GRKV_TRY(cuda_rc(launch_check_inputs(s, q, k, v, (int*)(w + L.status), st)));
   GRKV_TRY(cuda_rc(launch_score_any(s, q, k, v, scores, y, rstats, w, L, st)));
+  s.chained = true;
   GRKV_TRY(cuda_rc(launch_select(s, scores, idx, w, L, st)));
   GRKV_TRY(cuda_rc(launch_merge_any(s, q, k, v, scores, y, rstats, idx, k_out, v_out, w, L, st)));
   if (!s.update_k) return GRKV_OK;

@@ -267,6 +267,7 @@ __device__ __forceinline__ void stats32(float* v, int p0, int vlim, float sl2, f
 // ======================================================== k_merge_fixed
 // One CTA (256 threads) per unit; shared memory holds one key per slot.
 __global__ void __launch_bounds__(256) k_merge_fixed(MArgs a) {
+  chain_wait();
   extern __shared__ uint32_t fkey[];   // [B] candidate keys, 0 = not a candidate
   __shared__ int hist[256], sh[64];
   const int tid = threadIdx.x, nt = blockDim.x;
@@ -404,6 +405,7 @@ __device__ __forceinline__ void cluster_bar() {
 __global__ void __launch_bounds__(kThreadsG, 1)
     k_merge_gram(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                  const __grid_constant__ CUtensorMap tmV, MArgs a) {
+  chain_wait();
   extern __shared__ __align__(1024) uint8_t smraw[];
   uint8_t* sm = (uint8_t*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
   GBars* bars = (GBars*)(sm + kOffBar);
@@ -710,6 +712,7 @@ constexpr uint32_t kSmemBytesC = kOffBarC + 256 + 1024;
 __global__ void __launch_bounds__(kThreads, 1)
     k_merge_cross(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                   MArgs a) {
+  chain_wait();
   extern __shared__ __align__(1024) uint8_t smraw[];
   uint8_t* sm = (uint8_t*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
   CBars* bars = (CBars*)(sm + kOffBarC);
@@ -918,6 +921,7 @@ __global__ void __launch_bounds__(kThreadsU, 1)
     k_merge_update(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                    const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmKo,
                    const __grid_constant__ CUtensorMap tmVo, MArgs a) {
+  chain_wait();
   extern __shared__ __align__(1024) uint8_t smraw[];
   uint8_t* sm = (uint8_t*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
   UBars* bars = (UBars*)(sm + kOffBar);
@@ -1258,19 +1262,8 @@ cudaError_t launch_gram(const CUtensorMap& mq, const CUtensorMap& mk, const CUte
   const int tiles = (a.B + kTile - 1) / kTile, blocks = a.U * a.nrb;
   a.ranks = 1;
   while (a.ranks < 8 && 2 * a.ranks <= tiles && blocks * 2 * a.ranks <= kClusterSms) a.ranks *= 2;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = a.ranks;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(blocks * a.ranks);
-  cfg.blockDim = dim3(kThreadsG);
-  cfg.dynamicSmemBytes = kSmemBytes;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_merge_gram, mq, mk, mv, a);
+  return launch_kernel(true, a.ranks, k_merge_gram, dim3(blocks * a.ranks), kThreadsG, kSmemBytes, st,
+                       mq, mk, mv, a);
 }
 
 size_t merge_tc_ws_bytes(const Shape& s) { return merge_ws(s).total; }
@@ -1338,12 +1331,15 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
   if (W.nrb > 1 && (e = cudaFuncSetAttribute(k_merge_cross, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              kSmemBytesC)) != cudaSuccess)
     return e;
-  k_merge_fixed<<<s.U, 256, s.B * 4, st>>>(a);
+  if ((e = launch_kernel(s.chained, 1, k_merge_fixed, dim3(s.U), 256, s.B * 4, st, a)) != cudaSuccess)
+    return e;
   // the retained statistics, R and the diagonal Gram block of every row block
   if ((e = launch_gram(mq, mk, mv, a, st)) != cudaSuccess) return e;
   int launches = 2;
   if (W.nrb > 1) {
-    k_merge_cross<<<s.U, kThreads, kSmemBytesC, st>>>(mq, mk, a);
+    if ((e = launch_kernel(true, 1, k_merge_cross, dim3(s.U), kThreads, kSmemBytesC, st, mq, mk, a)) !=
+        cudaSuccess)
+      return e;
     launches += 1;
   }
   count_launches(launches);
@@ -1358,7 +1354,9 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
     a.rb = 0;
     a.row0 = 0;
     a.upd_mode = 0;
-    k_merge_update<<<s.U * a.split, kThreadsU, kSmemBytesU, st>>>(mq, mk, mv, mko, mvo, a);
+    if ((e = launch_kernel(true, 1, k_merge_update, dim3(s.U * a.split), kThreadsU, kSmemBytesU, st, mq,
+                           mk, mv, mko, mvo, a)) != cudaSuccess)
+      return e;
     launches = 1;
   } else {
     // the value update of each row block (the first leaves V0 + dV_0 in vpart)
@@ -1367,7 +1365,9 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
       a.rb = rb;
       a.row0 = rb * kRows;
       a.upd_mode = rb == 0 ? 1 : 2;
-      k_merge_update<<<s.U * a.split, kThreadsU, kSmemBytesU, st>>>(mq, mk, mv, mko, mvo, a);
+      if ((e = launch_kernel(true, 1, k_merge_update, dim3(s.U * a.split), kThreadsU, kSmemBytesU, st, mq,
+                           mk, mv, mko, mvo, a)) != cudaSuccess)
+      return e;
       launches += 1;
     }
   }

@@ -38,6 +38,7 @@ struct BudgetChunk {
 };
 __global__ void __launch_bounds__(1024) k_unit_table(const __grid_constant__ BudgetChunk c,
                                                      float beta, UnitRow* table) {
+  chain_wait();
   __shared__ int sh[32];
   const int i = threadIdx.x, b = i < c.count ? c.budget[i] : 0;
   int total;
@@ -160,12 +161,15 @@ extern "C" int grkv_compress_ragged(const grkv_params* p, const int32_t* budgets
       c.first = u0;
       c.off = (int64_t)r.off[u0];
       std::copy(budgets + u0, budgets + u0 + c.count, c.budget);
-      k_unit_table<<<1, 1024, 0, st>>>(c, p->beta, table);
+      const cudaError_t te =
+          launch_kernel(true, 1, k_unit_table, dim3(1), 1024, 0, st, c, p->beta, table);
+      if (te != cudaSuccess) return GRKV_ERR_CUDA;
       count_launches(1);
     }
     Shape rs = s;
     rs.units = table;
     rs.rows = rows;
+    rs.chained = true;
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = launch_select(rs, scores, idx, w, L, st);
     if (e == cudaSuccess)

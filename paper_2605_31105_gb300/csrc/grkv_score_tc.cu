@@ -295,6 +295,7 @@ __global__ void __launch_bounds__(score_threads(kPass, RB), 1)
                const __grid_constant__ CUtensorMap tmV, Args a) {
   using Lay = Layout<RB>;
   constexpr int kRing = Lay::kRing, kS = s_bufs(kPass);
+  if (kPass == 1) chain_wait();
   // One row block: each V is loaded one tile after its K, as it stays in the
   // ring through the tile's compute.  Two: its first use is half a tile after its K's.
   constexpr bool kLateV = RB == 1;
@@ -776,6 +777,7 @@ __global__ void __launch_bounds__(score_threads(kPass, RB), 1)
 // Deterministic mode: Y[u] = the unit's segment partials added in slot order.
 __global__ void k_y_sum_slots(const float4* __restrict__ part, float4* __restrict__ y, Sched sc,
                               int m, int maxc) {
+  chain_wait();
   const size_t per_unit = (size_t)m * kD / 4;
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < (size_t)sc.U * per_unit;
        i += (size_t)gridDim.x * blockDim.x) {
@@ -805,8 +807,7 @@ cudaError_t launch_pass(int G, const CUtensorMap& mq, const CUtensorMap& mk, con
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   count_launches(1);
-  kern<<<G, score_threads(kPass, RB), smem, st>>>(mq, mk, mv, a);
-  return cudaGetLastError();
+  return launch_kernel(kPass == 1, 1, kern, dim3(G), score_threads(kPass, RB), smem, st, mq, mk, mv, a);
 }
 
 // CTAs that can share one unit's tiles when U units are split evenly over
@@ -877,10 +878,9 @@ cudaError_t launch_score_tc(const Shape& s, const void* q, const void* k, const 
   if (e == cudaSuccess && a.ypart) {
     const size_t n4 = (size_t)s.U * s.m * kD / 4;
     const int blocks = (int)std::min<size_t>((n4 + 255) / 256, (size_t)G * 8);
-    k_y_sum_slots<<<blocks, 256, 0, st>>>((const float4*)a.ypart, (float4*)y, Sched{s.U, a.tpu, G},
-                                          s.m, a.maxc);
+    e = launch_kernel(true, 1, k_y_sum_slots, dim3(blocks), 256, 0, st, (const float4*)a.ypart,
+                      (float4*)y, Sched{s.U, a.tpu, G}, s.m, a.maxc);
     count_launches(1);
-    e = cudaGetLastError();
   }
   return e;
 }

@@ -28,6 +28,7 @@ namespace {
 __global__ void __launch_bounds__(1024) k_select(const float* __restrict__ scores, Shape s,
                                                  float* __restrict__ pooled,
                                                  int32_t* __restrict__ idx) {
+  chain_wait();
   __shared__ int hist[256];
   __shared__ int sh[48];
   const int u = blockIdx.x, tid = threadIdx.x, P = s.P, h = s.pool_k / 2;
@@ -185,6 +186,7 @@ __global__ void __launch_bounds__(kThr, 1) k_select_reg(const float* __restrict_
                                                         int32_t* __restrict__ idx) {
   extern __shared__ float sc[];
   __shared__ SelSmem sh;
+  chain_wait();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int u = blockIdx.x / kCs, rank = blockIdx.x % kCs;
   const int P = s.P, h = s.pool_k / 2;
@@ -514,19 +516,7 @@ cudaError_t launch_reg(const Shape& s, const float* scores, int32_t* idx, cudaSt
   const size_t bytes = reg_smem_bytes(kPer, kCs > 1 ? kMaxHalo : 0);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = kCs;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3((unsigned)s.U * kCs);
-  cfg.blockDim = dim3(kThr);
-  cfg.dynamicSmemBytes = bytes;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = kCs > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, scores, s, idx);
+  return launch_kernel(s.chained, kCs, kern, dim3((unsigned)s.U * kCs), kThr, bytes, st, scores, s, idx);
 }
 
 }  // namespace
@@ -547,8 +537,7 @@ cudaError_t launch_select_pooled(const Shape& s, const float* scores, int32_t* i
     if (per <= 16 * kCluster) return launch_reg<16, kCluster>(s, scores, idx, st);
     if (s.P <= kMaxClusterP) return launch_reg<32, kCluster>(s, scores, idx, st);
   }
-  k_select<<<s.U, 1024, 0, st>>>(scores, s, pooled, idx);
-  return cudaGetLastError();
+  return launch_kernel(s.chained, 1, k_select, dim3(s.U), 1024, 0, st, scores, s, pooled, idx);
 }
 
 cudaError_t launch_select(const Shape& s, const float* scores, int32_t* idx, char* ws,

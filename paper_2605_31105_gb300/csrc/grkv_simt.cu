@@ -170,6 +170,7 @@ __global__ void __launch_bounds__(kScT, 1)
                  int chunk, int nchunk, const float2* __restrict__ pstats,
                  float* __restrict__ row_stats, float* __restrict__ scores,
                  float* __restrict__ ypart) {
+  chain_wait();
   extern __shared__ __align__(16) float sm[];
   constexpr int MR = 16 * RT;
   float* qs = sm;                            // [MR][kSLD]
@@ -273,6 +274,7 @@ __global__ void __launch_bounds__(kScT, 1)
 // Y = sum of the chunks' shares, in chunk order; one float4 per thread.
 __global__ void __launch_bounds__(256) k_y_reduce(const float4* __restrict__ ypart, Shape s,
                                                   int nchunk, float4* __restrict__ y) {
+  chain_wait();
   const int u = blockIdx.y, md = s.m * (kD / 4), i = blockIdx.x * 256 + threadIdx.x;
   if (i >= md) return;
   float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -302,12 +304,14 @@ cudaError_t score_impl(const Shape& s, const T* q, const T* k, const T* v, float
   if (e != cudaSuccess) return e;
   const dim3 grid(L.nchunk, s.U);
   k_stats_chunk<T, RT><<<grid, kScT, smA, st>>>(q, k, s, L.chunk, L.nchunk, pstats);
-  k_prob_chunk<T, RT><<<grid, kScT, smB, st>>>(q, k, v, s, L.chunk, L.nchunk, pstats, row_stats,
-                                               scores, ypart);
-  k_y_reduce<<<dim3((s.m * (kD / 4) + 255) / 256, s.U), 256, 0, st>>>((const float4*)ypart, s,
-                                                                      L.nchunk, (float4*)y);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  e = launch_kernel(true, 1, k_prob_chunk<T, RT>, grid, kScT, smB, st, q, k, v, s, L.chunk, L.nchunk,
+                    (const float2*)pstats, row_stats, scores, ypart);
+  if (e != cudaSuccess) return e;
+  e = launch_kernel(true, 1, k_y_reduce, dim3((s.m * (kD / 4) + 255) / 256, s.U), 256, 0, st,
+                    (const float4*)ypart, s, L.nchunk, (float4*)y);
   count_launches(3);
-  return cudaGetLastError();
+  return e;
 }
 
 // The row tile follows m: 32 or 64 rows at a time waste less of it.

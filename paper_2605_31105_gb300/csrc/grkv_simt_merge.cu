@@ -178,6 +178,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_simt_logits(const T* __restrict__ q,
                                                      const T* __restrict__ k,
                                                      T* __restrict__ k_out, SArgs a) {
+  chain_wait();
   extern __shared__ __align__(16) float sm[];
   __shared__ int hist[256];
   __shared__ int sh[48];
@@ -229,6 +230,7 @@ __global__ void __launch_bounds__(256) k_simt_logits(const T* __restrict__ q,
 
 // X = row softmax over the retained keys; one warp per row of the unit.
 __global__ void __launch_bounds__(256) k_simt_softmax(SArgs a) {
+  chain_wait();
   const int lane = threadIdx.x & 31, B = a.s.B;
   const int u = blockIdx.x / a.tiles, r = blockIdx.x % a.tiles * 8 + (threadIdx.x >> 5);
   if (r >= a.s.m) return;
@@ -262,6 +264,7 @@ __host__ __device__ constexpr int regr_n_tiles(int m) {
 template <typename T, typename A>
 __global__ void __launch_bounds__(256) k_simt_regr(const T* __restrict__ v, SArgs a,
                                                    A* __restrict__ gram, A* __restrict__ rz) {
+  chain_wait();
   __shared__ float as[8][kRS + 1];
   __shared__ float bs[kRS][33];
   const Shape& s = a.s;
@@ -351,6 +354,7 @@ constexpr size_t kCholSmem = (size_t)(128 * kCLD + 4 * 32 * kBLD + 2 * 128) * si
 // its diagonal entry or below 2^-60, where pairs of floats leave too few
 // digits, sends the unit to fp64.
 __global__ void __launch_bounds__(kChT, 1) k_simt_chol(SArgs a, Df* __restrict__ gram) {
+  chain_wait();
   extern __shared__ __align__(16) float sm[];
   Df* N = (Df*)sm;                      // [128][kCLD]
   Df* inv = N + 128 * kCLD;             // [4][32][kBLD]
@@ -425,6 +429,7 @@ constexpr size_t kSubstSmem = (size_t)(10 * 32 * kBLD + 128 * 9 + 32 * 9) * size
 
 __global__ void __launch_bounds__(256) k_simt_subst(SArgs a, const Df* __restrict__ gram,
                                                     Df* __restrict__ rz) {
+  chain_wait();
   extern __shared__ __align__(16) float sm[];
   Df* Lb = (Df*)sm;                     // block (i, j), j <= i, at i (i + 1) / 2 + j
   Df* W = Lb + 10 * 32 * kBLD;          // [128][9]
@@ -496,6 +501,7 @@ template <typename T>
 __global__ void __launch_bounds__(512) k_simt_solve64(const T* __restrict__ v, SArgs a, int all,
                                                       Df* __restrict__ gram,
                                                       Df* __restrict__ rz) {
+  chain_wait();
   __shared__ int bad;
   const Shape& s = a.s;
   const int u = blockIdx.x, tid = threadIdx.x, m = s.m, B = s.B, nthr = blockDim.x;
@@ -583,6 +589,7 @@ template <typename T, typename A>
 __global__ void __launch_bounds__(256) k_simt_update(const T* __restrict__ v,
                                                      T* __restrict__ v_out, SArgs a,
                                                      const A* __restrict__ rz) {
+  chain_wait();
   __shared__ float xs[32][33];
   __shared__ A zs[32][32];
   const Shape& s = a.s;
@@ -638,16 +645,17 @@ cudaError_t merge_impl(const Shape& s, const T* q, const T* k, const T* v, const
   A* rz = (A*)(ws + L.rz);
   const unsigned U = (unsigned)s.U, nb = (unsigned)(s.B + 31) / 32, nr = (unsigned)(s.m + 31) / 32;
   a.tiles = (int)(1 + nb * nr);
-  k_simt_logits<T><<<U * a.tiles, 256, kLogitsSmem, st>>>(q, k, k_out, a);
+  cudaError_t e = launch_kernel(s.chained, 1, k_simt_logits<T>, dim3(U * a.tiles), 256, kLogitsSmem, st, q,
+                                k, k_out, a);
   count_launches(1);
-  cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && !s.lambda_inf) {
     a.tiles = (s.m + 7) / 8;
-    k_simt_softmax<<<U * a.tiles, 256, 0, st>>>(a);
+    e = launch_kernel(true, 1, k_simt_softmax, dim3(U * a.tiles), 256, 0, st, a);
+    if (e != cudaSuccess) return e;
     a.tiles = regr_r_tiles(s.m) + regr_n_tiles(s.m);
-    k_simt_regr<T, A><<<U * a.tiles, 256, 0, st>>>(v, a, gram, rz);
+    e = launch_kernel(true, 1, k_simt_regr<T, A>, dim3(U * a.tiles), 256, 0, st, v, a, gram, rz);
     count_launches(2);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (e != cudaSuccess) return e;
     if constexpr (std::is_same<A, Df>::value) {
       // the factor of m <= 128 fits shared memory as pairs; more rows take fp64
       const bool pairs = s.m <= 128;
@@ -658,13 +666,15 @@ cudaError_t merge_impl(const Shape& s, const T* q, const T* k, const T* v, const
           e = cudaFuncSetAttribute(k_simt_subst, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)kSubstSmem);
         if (e != cudaSuccess) return e;
-        k_simt_chol<<<U, kChT, kCholSmem, st>>>(a, gram);
-        k_simt_subst<<<U * (kD / 8), 256, kSubstSmem, st>>>(a, gram, rz);
+        e = launch_kernel(true, 1, k_simt_chol, dim3(U), kChT, kCholSmem, st, a, gram);
+        if (e == cudaSuccess)
+          e = launch_kernel(true, 1, k_simt_subst, dim3(U * (kD / 8)), 256, kSubstSmem, st, a,
+                            (const Df*)gram, rz);
+        if (e != cudaSuccess) return e;
         count_launches(2);
       }
-      k_simt_solve64<T><<<U, 512, 0, st>>>(v, a, pairs ? 0 : 1, gram, rz);
+      e = launch_kernel(true, 1, k_simt_solve64<T>, dim3(U), 512, 0, st, v, a, pairs ? 0 : 1, gram, rz);
       count_launches(1);
-      e = cudaGetLastError();
     } else {
       // gram's region holds 8 bytes per entry: the second half takes the factor
       // of the first 128 rows (m^2 >= 128^2 floats a unit where it is used)
@@ -675,9 +685,9 @@ cudaError_t merge_impl(const Shape& s, const T* q, const T* k, const T* v, const
   }
   if (e != cudaSuccess) return e;
   a.tiles = (int)nb * (kD / 32);
-  k_simt_update<T, A><<<U * a.tiles, 256, 0, st>>>(v, v_out, a, rz);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_kernel(true, 1, k_simt_update<T, A>, dim3(U * a.tiles), 256, 0, st, v, v_out, a,
+                       (const A*)rz);
 }
 
 }  // namespace

@@ -358,6 +358,7 @@ __device__ __forceinline__ void zero_tile(float (*x)[kTC]) {
 // m <= 128; kCols columns of R per CTA.
 template <int kCols>
 __global__ void __launch_bounds__(kThreads, 1) k_solve(SolveArgs a) {
+  chain_wait();
   extern __shared__ __align__(16) float sm[];
   SolveSmem& s = *(SolveSmem*)sm;
   constexpr int kSplit = kD / kCols, kTC = kCols / 16;
@@ -400,6 +401,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_solve(SolveArgs a) {
 // last also leaves L_A.
 constexpr int kCols2 = 64, kTC2 = kCols2 / 16;
 __global__ void __launch_bounds__(kThreads, 1) k_solve_first(SolveArgs a) {
+  chain_wait();
   extern __shared__ __align__(16) float sm[];
   SolveSmem& s = *(SolveSmem*)sm;
   const int u = blockIdx.x >> 2, which = blockIdx.x & 3;
@@ -442,6 +444,7 @@ static_assert(offsetof(SecondSmem, wb) % 16 == 0, "float4 rows");
 // m > 128, second row block and the backward pass of the first; two CTAs per
 // unit, 64 columns of R each.
 __global__ void __launch_bounds__(kThreads, 1) k_solve_second(SolveArgs a) {
+  chain_wait();
   extern __shared__ __align__(16) float sm[];
   SecondSmem& q = *(SecondSmem*)sm;
   SolveSmem& s = q.s;
@@ -537,6 +540,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_solve_second(SolveArgs a) {
 }
 
 __global__ void k_zero_rows(float4* __restrict__ p, size_t count) {
+  chain_wait();
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
        i += (size_t)gridDim.x * blockDim.x)
     p[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -546,9 +550,8 @@ template <typename K>
 cudaError_t run(K kern, unsigned grid, size_t smem, const SolveArgs& a, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<grid, kThreads, smem, st>>>(a);
   count_launches(1);
-  return cudaGetLastError();
+  return launch_kernel(true, 1, kern, dim3(grid), kThreads, smem, st, a);
 }
 
 }  // namespace
@@ -566,9 +569,9 @@ cudaError_t launch_solve(int U, int m, int ld, int sym, float lambda, int lambda
     return run(k_solve<128>, n, sizeof(SolveSmem), a, st);
   }
   if (lambda_inf) {
-    k_zero_rows<<<608, 256, 0, st>>>((float4*)rz, (size_t)U * ld * (kD / 4));
     count_launches(1);
-    return cudaGetLastError();
+    return launch_kernel(true, 1, k_zero_rows, dim3(608), 256, 0, st, (float4*)rz,
+                         (size_t)U * ld * (kD / 4));
   }
   cudaError_t e = run(k_solve_first, n * 4, sizeof(SolveSmem), a, st);
   if (e != cudaSuccess) return e;
