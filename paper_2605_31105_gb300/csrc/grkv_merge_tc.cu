@@ -184,6 +184,44 @@ struct Gatherer {
   }
 };
 
+// The same tile layout by 16-byte asynchronous copies, half a warp per 256-byte row: rows
+// r0 .. r0 + 32 kN - 1 of the tile at shared address `tile`, row r0 + 32 h + l from row j[h] of
+// lane l.  A gather4 tile takes 8 K cycles from issue to arrival beside another tile in flight
+// and the TMA stores, these copies about 3.5 K; the issuing warp has to see its copies land
+// before the tensor cores may read them, though.  256 units B = 2048: k_merge_gram 97 us with
+// gather4 and 88 with these; k_merge_update 102 us with gather4 for K0 and these for V0 (which only
+// threads read), 103 with these for both and 106 with gather4 for both.
+template <int kN>
+__device__ __forceinline__ void gather_async(uint32_t tile, int r0, const __nv_bfloat16* base,
+                                             const int* j, int lane) {
+  const int c = lane & 15;
+  const uint32_t dst = tile + (c >> 3) * (kTileBytes / 2);
+#pragma unroll
+  for (int i = 0; i < 16 * kN; ++i) {
+    const int r = 2 * i + (lane >> 4);
+    const int row = __shfl_sync(0xffffffffu, j[i / 16], r & 31);
+    cp_async16(dst + sw128_offset(r0 + r, c & 7), base + (size_t)row * kD + c * 8);
+  }
+}
+// Lane l's rows of gather_async: rows_u[first + 32 h + l], clamped to the last of `count`; an
+// entry outside [0, n) reads row 0.
+template <int kN>
+__device__ __forceinline__ void gather_index(const int32_t* rows_u, int first, int count, int n,
+                                             int lane, int* j) {
+#pragma unroll
+  for (int h = 0; h < kN; ++h) {
+    const int x = __ldg(rows_u + min(first + 32 * h + lane, count - 1));
+    j[h] = (unsigned)x < (unsigned)n ? x : 0;
+  }
+}
+// The warp's copies have landed and are visible to the tensor cores and TMA.
+__device__ __forceinline__ void gather_arrive(uint64_t* full, int lane) {
+  cp_async_wait_all();
+  fence_proxy_async_smem();
+  __syncwarp();
+  if (lane == 0) mbar_arrive(full);
+}
+
 // S = Q K0^T for one gathered tile into TMEM columns s_col (issued by one thread).
 __device__ __forceinline__ void issue_s(uint32_t s_tmem, uint32_t qa, uint32_t ka) {
   const uint32_t id_s = idesc_bf16(kRows, kTile, 0, 0);
@@ -351,15 +389,15 @@ __global__ void __launch_bounds__(256) k_merge_fixed(MArgs a) {
 // to registers and writes Xh and 2 (X - Xh) over them (TMEM A operands) and XGh =
 // Xh of the non-fixed positions to shared memory (the Gram's B operand).
 //
-// Bound by the gathers (5 K cycles per tile of K0 and V0 rows: TMA gather issue) where a
-// rank has many tiles, by latency where it has one.  The shares leave through
+// Bound by the gathers (4.4 K cycles per tile of K0 and V0 rows) where a rank has many
+// tiles, by latency where it has one.  The shares leave through
 // shared memory: stored from TMEM row by row, each instruction touched 32 lines
 // and the rows took 16 K cycles of 48 K.
 //
 // Measured, against one CTA per unit and block, two 128-thread groups on alternate
 // tiles, and a second launch for units that start over: 8 units B = 512 44 -> 15 us,
 // 64 units with budgets 200 .. 1536 88 -> 26 us, 32 units B = 1024 m = 256 103 -> 22 us,
-// 256 units B = 2048 129 -> 99 us (two waves).
+// 256 units B = 2048 129 -> 99 us (two waves), 88 with the asynchronous gathers.
 struct GBars {
   uint64_t ring_full[kRingG], ring_empty[kRingG];
   uint64_t q_full;
@@ -403,8 +441,7 @@ __device__ __forceinline__ void cluster_bar() {
 }
 
 __global__ void __launch_bounds__(kThreadsG, 1)
-    k_merge_gram(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                 const __grid_constant__ CUtensorMap tmV, MArgs a) {
+    k_merge_gram(const __grid_constant__ CUtensorMap tmQ, MArgs a) {
   chain_wait();
   extern __shared__ __align__(1024) uint8_t smraw[];
   uint8_t* sm = (uint8_t*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
@@ -419,7 +456,7 @@ __global__ void __launch_bounds__(kThreadsG, 1)
   const int ng = __ldg(a.ng + u);
   if (tid == 0) {
     for (int i = 0; i < kRingG; ++i) {
-      mbar_init(&bars->ring_full[i], 3);   // one expect_tx arrival per gathering warp
+      mbar_init(&bars->ring_full[i], 1);   // the gathering warp
       mbar_init(&bars->ring_empty[i], 1);
     }
     mbar_init(&bars->q_full, 1);
@@ -453,8 +490,7 @@ __global__ void __launch_bounds__(kThreadsG, 1)
   // slots / positions past vlim are invisible to this row (and so are those >= B)
   const int vlim = a.causal ? B - a.w + grow % a.w : B - 1;
   const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
-  Gatherer<kRingG, 3> gt{sm + kOffRing, bars->ring_full, bars->ring_empty};
-  uint32_t use = 0, job = 0;   // ring loads and S tiles so far (MMA warp, compute groups)
+  uint32_t use = 0, job = 0;   // ring loads (gathers, MMA warp) and S tiles (MMA warp, compute) so far
   bool single = a.rstats != nullptr, ok = true;
   float lam = INFINITY;
   if (single && computes && row_ok)
@@ -472,16 +508,23 @@ __global__ void __launch_bounds__(kThreadsG, 1)
   for (int ph = single ? 1 : 0, acc_use = 0;;) {
     float M = -INFINITY, L = 0.f;   // phase 0: row statistics; phase 1: largest logit, sum of X
     if (gathers) {
+      // the phase's loads in turn to the three warps, a whole tile each
       __syncwarp();
       const int32_t* rows_u = (ph ? a.src : a.idx) + ur.off;
-      int jn[4];
-      if (ta < tb) gt.rows(rows_u, B, a.n, u * a.n, ta, pw, lane, jn);
-      for (int t = ta; t < tb && ok; ++t) {
-        const int j[4] = {jn[0], jn[1], jn[2], jn[3]};
-        if (t + 1 < tb) gt.rows(rows_u, B, a.n, u * a.n, t + 1, pw, lane, jn);
-        ok = gt.load(&tmK, j, pw, lane, abort_flag);
-        if (ok && ph) ok = gt.load(&tmV, j, pw, lane, abort_flag);
+      const int per = ph + 1, loads = (tb - ta) * per;   // K0 of a tile, in phase 1 then its V0
+      int next[4];
+      if (pw < loads) gather_index<4>(rows_u, (ta + pw / per) * kTile, B, a.n, lane, next);
+      for (int i = pw; i < loads; i += 3) {
+        const int j[4] = {next[0], next[1], next[2], next[3]};
+        if (i + 3 < loads) gather_index<4>(rows_u, (ta + (i + 3) / per) * kTile, B, a.n, lane, next);
+        const uint32_t n = use + i, slot = n % kRingG;
+        if (n >= kRingG) ok = ok && mbar_wait_warp(&bars->ring_empty[slot], (n / kRingG - 1) & 1, abort_flag);
+        if (!ok) break;
+        gather_async<4>(smem_u32(sm + kOffRing + slot * kTileBytes), 0,
+                        (ph && (i & 1) ? a.v : a.k) + (size_t)u * a.n * kD, j, lane);
+        gather_arrive(&bars->ring_full[slot], lane);
       }
+      use += loads;
     } else if (warp == 1) {
       constexpr uint32_t id_s = idesc_bf16(kRows, kTile, 0, 0);   // S = Q K0^T
       constexpr uint32_t id_r = idesc_bf16(kRows, kD, 0, 1);      // R~ += Xh V0 (V0 MN-major)
@@ -671,7 +714,6 @@ __global__ void __launch_bounds__(kThreadsG, 1)
     cluster_bar();   // no rank leaves while a peer reads its shares
     break;
   }
-  if (gathers) gt.drain(abort_flag);
   if (warp == 1) {
     // every MMA issued completes before TMEM is released
     mma_commit_elect(&bars->drain);
@@ -882,7 +924,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // ======================================================== k_merge_update
 // Slot order, a unit's tiles over `split` CTAs, 736 threads.  Roles: warp 0 the Q load and
 // the K_out tile stores, warp 22 the V_out tile stores; warp 1 MMA issue;
-// warps 2, 3, 16, 17 the K0 gathers and 18-21 the V0 gathers (two-slot rings
+// warps 2, 3, 16, 17 the K0 gathers (TMA) and 18-21 the V0 gathers (cp.async; two-slot rings
 // each, on all four SM sub-partitions); warps 4-7 and 8-11
 // two compute groups taking alternate tiles (one thread per token = TMEM lane
 // of S^T): X_G^T from S^T, zero for fixed slots, written back over S^T as
@@ -919,8 +961,8 @@ __device__ __forceinline__ void copy_rows(__nv_bfloat16* dst, const uint8_t* til
 
 __global__ void __launch_bounds__(kThreadsU, 1)
     k_merge_update(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmKo,
-                   const __grid_constant__ CUtensorMap tmVo, MArgs a) {
+                   const __grid_constant__ CUtensorMap tmKo, const __grid_constant__ CUtensorMap tmVo,
+                   MArgs a) {
   chain_wait();
   extern __shared__ __align__(1024) uint8_t smraw[];
   uint8_t* sm = (uint8_t*)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
@@ -928,7 +970,8 @@ __global__ void __launch_bounds__(kThreadsU, 1)
   float* lam_s = (float*)(sm + kOffLamU);
   uint8_t* zh = sm + kOffZU;
   uint8_t* zl = zh + kTileBytes;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform for the compiler
   // the CTA's tiles T0 .. T0 + T - 1 of the unit (`split` CTAs per unit)
   const int u = blockIdx.x / a.split, part = blockIdx.x - u * a.split;
   const UnitRow ur = unit_row(a.units, u, a.B, a.n_fix);
@@ -944,7 +987,7 @@ __global__ void __launch_bounds__(kThreadsU, 1)
   if (tid == 0) {
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bars->k_full[i], 4);    // one expect_tx arrival per gathering warp
-      mbar_init(&bars->v_full[i], 4);
+      mbar_init(&bars->v_full[i], 128);  // every gathering thread, once its copies have landed
       mbar_init(&bars->k_empty[i], 2);   // the S^T MMA and the K_out store
       mbar_init(&bars->v_empty[i], 1);   // the V_out store
       mbar_init(&bars->s_full[i], 1);
@@ -1047,73 +1090,72 @@ __global__ void __launch_bounds__(kThreadsU, 1)
         mbar_wait_warp(&bars->vo_full[t_part & 1], (t_part >> 1) & 1, abort_flag))
       copy_rows(a.v_out + (ur.off + S0 + (size_t)t_part * kTile) * kD,
                 sm + kOffVU + (t_part & 1) * kTileBytes, B - S0 - t_part * kTile, lane);
-  } else if (warp == 2 || warp == 3 || (warp >= 16 && warp < 22)) {
-    // K0 gathers: warps 2, 3, 16, 17; V0 gathers: warps 18 - 21 (own rings, so
-    // that a K tile never waits for a V slot)
-    const bool is_v = warp >= 18;
-    const int pw = warp < 4 ? warp - 2 : (is_v ? warp - 18 : warp - 14), row0 = u * a.n;
-    // mode 2 builds V_out from vpart: no V0 tiles
-    const int TG = is_v && a.upd_mode == 2 ? 0 : T;
-    Gatherer<2, 4> g{sm + (is_v ? kOffVU : kOffKU), is_v ? bars->v_full : bars->k_full,
-                     is_v ? bars->v_empty : bars->k_empty};
-    const CUtensorMap* map = is_v ? &tmV : &tmK;
+  } else if (warp == 2 || warp == 3 || warp == 16 || warp == 17) {
+    // K0 gathers
+    const int pw = warp < 4 ? warp - 2 : warp - 14, row0 = u * a.n;
+    Gatherer<2, 4> g{sm + kOffKU, bars->k_full, bars->k_empty};
     int jn[4];
-    if (TG > 0) g.rows(idx_u, B, a.n, row0, T0, pw, lane, jn);
+    if (T > 0) g.rows(idx_u, B, a.n, row0, T0, pw, lane, jn);
     bool ok = true;
-    for (int t = 0; t < TG && ok; ++t) {
+    for (int t = 0; t < T && ok; ++t) {
       const int j[4] = {jn[0], jn[1], jn[2], jn[3]};
-      if (t + 1 < TG) g.rows(idx_u, B, a.n, row0, T0 + t + 1, pw, lane, jn);
-      ok = g.load(map, j, pw, lane, abort_flag);
+      if (t + 1 < T) g.rows(idx_u, B, a.n, row0, T0 + t + 1, pw, lane, jn);
+      ok = g.load(&tmK, j, pw, lane, abort_flag);
     }
     g.drain(abort_flag);
-  } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t id_s = idesc_bf16(kTile, kRows, 0, 0);   // S^T = K0 Q^T
-      const uint32_t id_d = idesc_bf16(kTile, kD, 0, 1);      // dV = X_G^T Z (Z MN-major)
-      const uint32_t qa = smem_u32(sm + kOffQ);
-      const uint32_t bh = smem_u32(zh), bl = smem_u32(zl);
-      bool ok = mbar_wait(&bars->q_full, 0, abort_flag, kBudget);
-      auto issue_d = [&](int t) -> bool {
-        const uint32_t d = tmem + kColD + (t & 1) * kD, x = tmem + kColS + (t & 1) * kTile;
-        bool w = mbar_wait(&bars->x_full[t & 1], (t >> 1) & 1, abort_flag, kBudget);
-        if (w && t >= 2) w = mbar_wait(&bars->d_empty[t & 1], ((t >> 1) - 1) & 1, abort_flag, kBudget);
-        if (!w) return false;
-        tc_fence_after();
-#pragma unroll
-        for (int kk = 0; kk < kRows / 16; ++kk)
-          mma_bf16_ts(d, x + xt_col(kk, 0), sw128_desc(bh + kk * 2048, kTileBytes / 2, 1024), id_d,
-                      kk > 0);
-#pragma unroll
-        for (int kk = 0; kk < kRows / 16; ++kk)
-          mma_bf16_ts(d, x + xt_col(kk, 0), sw128_desc(bl + kk * 2048, kTileBytes / 2, 1024), id_d, 1);
-#pragma unroll
-        for (int kk = 0; kk < kRows / 16; ++kk)
-          mma_bf16_ts(d, x + xt_col(kk, 1), sw128_desc(bh + kk * 2048, kTileBytes / 2, 1024), id_d, 1);
-        mma_commit(&bars->d_full[t & 1]);
-        return true;
-      };
-      for (int t = 0; t < T && ok; ++t) {
-        const int sl = t & 1;
-        ok = mbar_wait(&bars->k_full[sl], (t >> 1) & 1, abort_flag, kBudget);
-        if (!ok) break;
-        tc_fence_after();
-        // S^T into buffer sl: its previous contents (X_G^T of tile t - 2) were
-        // read by the dV MMAs issued before this one
-        const uint32_t ka = smem_u32(sm + kOffKU + sl * kTileBytes);
-#pragma unroll
-        for (int kk = 0; kk < kD / 16; ++kk) {
-          const uint32_t off = (kk >> 2) * (kTileBytes / 2) + (kk & 3) * 32;
-          mma_bf16(tmem + kColS + sl * kTile, sw128_desc(ka + off, 16, 1024),
-                   sw128_desc(qa + off, 16, 1024), id_s, kk > 0);
-        }
-        mma_commit(&bars->k_empty[sl]);
-        mma_commit(&bars->s_full[sl]);
-        if (t >= 1) ok = issue_d(t - 1);
-      }
-      if (ok && T > 0) ok = issue_d(T - 1);
-      mma_commit(&bars->drain);
-      mbar_wait(&bars->drain, 0, abort_flag, kBudget);
+  } else if (warp >= 18 && warp < 22) {
+    // V0 gathers: a quarter of every tile each (own ring, so that a K tile never waits
+    // for a V slot); only threads read a V0 tile, so the copies themselves arrive
+    const int r0 = 32 * (warp - 18);
+    const __nv_bfloat16* v0 = a.v + (size_t)u * a.n * kD;
+    // mode 2 builds V_out from vpart: no V0 tiles
+    const int TG = a.upd_mode == 2 ? 0 : T;
+    int next[1];
+    if (TG > 0) gather_index<1>(idx_u, T0 * kTile + r0, B, a.n, lane, next);
+    for (int t = 0; t < TG; ++t) {
+      const int j[1] = {next[0]}, sl = t & 1;
+      if (t + 1 < TG) gather_index<1>(idx_u, (T0 + t + 1) * kTile + r0, B, a.n, lane, next);
+      if (t >= 2 && !mbar_wait_warp(&bars->v_empty[sl], ((t >> 1) - 1) & 1, abort_flag)) break;
+      gather_async<1>(smem_u32(sm + kOffVU + sl * kTileBytes), r0, v0, j, lane);
+      cp_async_arrive(&bars->v_full[sl]);
     }
+    cp_async_wait_all();
+  } else if (warp == 1) {
+    // the whole warp walks the tiles, an elected lane issues (as in the scoring kernel)
+    constexpr uint32_t id_s = idesc_bf16(kTile, kRows, 0, 0);   // S^T = K0 Q^T
+    constexpr uint32_t id_d = idesc_bf16(kTile, kD, 0, 1);      // dV = X_G^T Z (Z MN-major)
+    const uint64_t q_desc = sw128_desc(smem_u32(sm + kOffQ), 16, 1024);
+    const uint64_t k_desc = sw128_desc(smem_u32(sm + kOffKU), 16, 1024);
+    const uint64_t zh_desc = sw128_desc(smem_u32(zh), kTileBytes / 2, 1024);
+    const uint64_t zl_desc = sw128_desc(smem_u32(zl), kTileBytes / 2, 1024);
+    bool ok = mbar_wait_warp(&bars->q_full, 0, abort_flag);
+    auto issue_d = [&](int t) -> bool {
+      const uint32_t d = tmem + kColD + (t & 1) * kD, x = tmem + kColS + (t & 1) * kTile;
+      if (!mbar_wait_warp(&bars->x_full[t & 1], (t >> 1) & 1, abort_flag)) return false;
+      if (t >= 2 && !mbar_wait_warp(&bars->d_empty[t & 1], ((t >> 1) - 1) & 1, abort_flag)) return false;
+      tc_fence_after();
+      mma8_ts<id_d, false>(d, x, zh_desc, false);
+      mma8_ts<id_d, false>(d, x, zl_desc, true);
+      mma8_ts<id_d, false>(d, x + 16, zh_desc, true);
+      mma_commit_elect(&bars->d_full[t & 1]);
+      return true;
+    };
+    for (int t = 0; t < T && ok; ++t) {
+      const int sl = t & 1;
+      ok = mbar_wait_warp(&bars->k_full[sl], (t >> 1) & 1, abort_flag);
+      if (!ok) break;
+      tc_fence_after();
+      // S^T into buffer sl: its previous contents (X_G^T of tile t - 2) were
+      // read by the dV MMAs issued before this one
+      mma8_ss<id_s>(tmem + kColS + sl * kTile, k_desc + sl * (kTileBytes >> 4), q_desc);
+      mma_commit_elect(&bars->k_empty[sl]);
+      mma_commit_elect(&bars->s_full[sl]);
+      if (t >= 1) ok = issue_d(t - 1);
+    }
+    if (ok && T > 0) ok = issue_d(T - 1);
+    mma_commit_elect(&bars->drain);
+    volatile int no_abort = 0;
+    mbar_wait(&bars->drain, 0, &no_abort, kBudget);
   } else if (warp >= 4 && warp < 12) {
     // compute groups: group cg takes the tiles t with t % 2 == cg
     const int cg = (warp - 4) >> 2, q = warp & 3, tok = q * 32 + lane;
@@ -1257,13 +1299,12 @@ MergeWs merge_ws(const Shape& s) {
 
 // As many ranks as leave every cluster room on the SMs at once: 8 units of B = 512
 // take 15 us with four ranks, one tile each.
-cudaError_t launch_gram(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
-                        MArgs a, cudaStream_t st) {
+cudaError_t launch_gram(const CUtensorMap& mq, MArgs a, cudaStream_t st) {
   const int tiles = (a.B + kTile - 1) / kTile, blocks = a.U * a.nrb;
   a.ranks = 1;
   while (a.ranks < 8 && 2 * a.ranks <= tiles && blocks * 2 * a.ranks <= kClusterSms) a.ranks *= 2;
   return launch_kernel(true, a.ranks, k_merge_gram, dim3(blocks * a.ranks), kThreadsG, kSmemBytes, st,
-                       mq, mk, mv, a);
+                       mq, a);
 }
 
 size_t merge_tc_ws_bytes(const Shape& s) { return merge_ws(s).total; }
@@ -1276,10 +1317,9 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
                             const float* scores, const float* y, const float* row_stats,
                             const int32_t* idx, void* k_out, void* v_out, char* ws,
                             const WsLayout& L, cudaStream_t st) {
-  CUtensorMap mq, mk, mv, mko, mvo;
+  CUtensorMap mq, mk, mko, mvo;
   if (!encode_bf16_3d(&mq, q, kD, s.m, s.U, 64, kRows) ||
       !encode_bf16_2d_rows(&mk, k, kD, (uint64_t)s.U * s.n) ||
-      !encode_bf16_2d_rows(&mv, v, kD, (uint64_t)s.U * s.n) ||
       !encode_bf16_3d(&mko, k_out, kD, s.units ? s.rows : s.B, s.units ? 1 : s.U, 64, kTile) ||
       !encode_bf16_3d(&mvo, v_out, kD, s.units ? s.rows : s.B, s.units ? 1 : s.U, 64, kTile))
     return cudaErrorInvalidValue;
@@ -1334,7 +1374,7 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
   if ((e = launch_kernel(s.chained, 1, k_merge_fixed, dim3(s.U), 256, s.B * 4, st, a)) != cudaSuccess)
     return e;
   // the retained statistics, R and the diagonal Gram block of every row block
-  if ((e = launch_gram(mq, mk, mv, a, st)) != cudaSuccess) return e;
+  if ((e = launch_gram(mq, a, st)) != cudaSuccess) return e;
   int launches = 2;
   if (W.nrb > 1) {
     if ((e = launch_kernel(true, 1, k_merge_cross, dim3(s.U), kThreads, kSmemBytesC, st, mq, mk, a)) !=
@@ -1355,7 +1395,7 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
     a.row0 = 0;
     a.upd_mode = 0;
     if ((e = launch_kernel(true, 1, k_merge_update, dim3(s.U * a.split), kThreadsU, kSmemBytesU, st, mq,
-                           mk, mv, mko, mvo, a)) != cudaSuccess)
+                           mk, mko, mvo, a)) != cudaSuccess)
       return e;
     launches = 1;
   } else {
@@ -1366,7 +1406,7 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
       a.row0 = rb * kRows;
       a.upd_mode = rb == 0 ? 1 : 2;
       if ((e = launch_kernel(true, 1, k_merge_update, dim3(s.U * a.split), kThreadsU, kSmemBytesU, st, mq,
-                           mk, mv, mko, mvo, a)) != cudaSuccess)
+                           mk, mko, mvo, a)) != cudaSuccess)
       return e;
       launches += 1;
     }
