@@ -88,15 +88,15 @@ SCORE_SRC = os.path.join("paper_2605_31105_gb300", "csrc", "grkv_score_tc.cu")
 # the ncu capture in profiles/score_tc_c2_llama_32k.md, keyed by the SHA-256 of the
 # kernel source it was taken on.
 SCORE_TRAFFIC = {
-    "c2_llama_32k_bf16": ("0ea59ba48bb5a0be128f6060b1dd07717b01f47bfca8e89e80517f105e7d52bc",
-                          6532132864),
+    "c2_llama_32k_bf16": ("a99f3a36b4b67c9c0fe41fa9c256432bdf02ec59c39be001fd499e5086dba2dc",
+                          6543142912),
 }
 
 
 SCORE_KERNEL = {
     "default": "grkv_score stage (k_score_tc: window scoring + target, two launches)",
     "one_read": "grkv_score stage (k_score_pipe: window scoring + target, one read of K)",
-    "portable": "grkv_score stage (CUDA-core kernels: k_stats_chunk, k_stats_reduce, k_prob_chunk, k_y_reduce)",
+    "portable": "grkv_score stage (CUDA-core kernels: k_stats_chunk, k_prob_chunk, k_y_reduce)",
 }
 
 

@@ -1,7 +1,7 @@
 // GRKV value step on the tensor cores (bf16, d = 128, m <= 256, B <= 32768).
 //
 // Algorithm 1's value step in dual form (Sec. 3.4, App. D.1) with the fixed
-// tokens of App. D.3, one unit per CTA:
+// tokens of App. D.3:
 //   k_merge_fixed   the fixed set (retained sinks, the window, and the n_fix
 //                   retained prefix tokens with the largest scores), a flag per
 //                   slot, and a stable partition of the B retained slots into
@@ -9,15 +9,15 @@
 //                   ones, each in slot order.  The window stays last in both
 //                   orders, so slot or position p is visible to window row r
 //                   exactly when p <= B - w + r % w.
-//   k_merge_gram    pass 1 over the slots: row max / sum of l = s Q K0^T (K0
-//                   gathered with TMA gather4); pass 2 over the positions:
+//   k_merge_gram    a cluster of CTAs per unit: phase 0 over the slots: row max /
+//                   sum of l = s Q K0^T; phase 1 over the positions:
 //                   X = softmax, R~ += Xh V0 and the Gram G += Xh XGh^T +
 //                   (2 Xl) XGh^T on tcgen05 (Xh, Xl the bf16 high / low parts
 //                   of X; XGh is Xh with the fixed columns zeroed, which removes
 //                   them from both terms; N = (G + G^T) / 2 restores the cross
 //                   terms).  Writes R = Y - R~, G and the row normalisers to the
-//                   workspace.  With the full-cache row statistics only pass 2
-//                   runs.
+//                   workspace.  With the full-cache row statistics only phase 1
+//                   runs, unless they lie far above the retained ones.
 //   launch_solve    N = sym(G) + lambda I, Z = N^-1 R in fp32 (grkv_solve.cu).
 //   k_merge_update  over the slots: S^T = K0 Q^T (one TMEM lane per token),
 //                   X_G^T (zero for fixed slots) as bf16 high / low parts back
