@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(kChT, 1) k_simt_chol(SArgs a, Df* __restrict__
   extern __shared__ __align__(16) float sm[];
   Df* N = (Df*)sm;                      // [128][kCLD]
   Df* inv = N + 128 * kCLD;             // [4][32][kBLD]
-  Df* col = inv + 4 * 32 * kBLD;        // [128] the current column of L
+  Df* col = inv + 4 * 32 * kBLD;        // [128] the current column of L below the diagonal
   Df* dinv = col + 128;                 // [128] 1 / L_jj
   const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int m = a.s.m, mp = (m + 31) / 32 * 32;
@@ -376,9 +376,11 @@ __global__ void __launch_bounds__(kChT, 1) k_simt_chol(SArgs a, Df* __restrict__
         if (tid == 0) a.state[u] = kNeeds64;
         return;
       }
-      const Df root = df_sqrt(d), rinv = df_rcp(root);
-      if (tid < mp - j) {
-        const Df l = tid == 0 ? root : df_mul(N[(j + tid) * kCLD + j], rinv);
+      // the pivot stays as it is: other warps may not have read it yet, and L_jj is only
+      // used through its reciprocal
+      const Df rinv = df_rcp(df_sqrt(d));
+      if (tid > 0 && tid < mp - j) {
+        const Df l = df_mul(N[(j + tid) * kCLD + j], rinv);
         N[(j + tid) * kCLD + j] = l;
         col[j + tid] = l;
       }
