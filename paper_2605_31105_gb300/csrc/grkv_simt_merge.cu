@@ -438,7 +438,8 @@ __global__ void __launch_bounds__(256) k_simt_subst(SArgs a, const Df* __restric
   Df* tmp = W + 128 * 9;                // [32][9]
   const int u = blockIdx.x / (kD / 8), tid = threadIdx.x, r = tid >> 3, c = tid & 7;
   const int m = a.s.m, nb = (m + 31) / 32;
-  if (a.state[u] != kSolved) return;
+  // another CTA of the unit may give it to fp64 meanwhile: one answer for the block
+  if (__syncthreads_or(a.state[u] != kSolved)) return;
   const Df* G = gram + (size_t)u * m * m;
   Df* Z = rz + (size_t)u * m * kD + blockIdx.x % (kD / 8) * 8;
   for (int i = tid >> 5; i < nb * 32; i += 8)

@@ -105,6 +105,25 @@ extern "C" int run_chol(int m, int descending, double* gram, int* state) {
   for (size_t i = 0; i < n.size(); ++i) gram[i] = (double)n[i].hi + n[i].lo;
   return rc;
 }
+// Every block of one unit; turn `flip` of the first block finds the unit given to fp64 by another.
+static int g_flip;
+extern "C" int run_subst(int m, int descending, const double* factor, double* rz, int* state,
+                         int flip) {
+  std::vector<Df> n((size_t)m * m), r((size_t)m * kD);
+  for (size_t i = 0; i < n.size(); ++i) n[i] = {(float)factor[i], (float)(factor[i] - (float)factor[i])};
+  for (size_t i = 0; i < r.size(); ++i) r[i] = {(float)rz[i], (float)(rz[i] - (float)rz[i])};
+  g_args = {{m}, state};
+  g_gram = n.data();
+  g_rz = r.data();
+  g_flip = flip;
+  int rc = 0;
+  for (int b = 0; b < kD / 8; ++b)
+    rc |= run_block(256, b, descending, [] { k_simt_subst(g_args, g_gram, g_rz); },
+                    b == 0 && flip >= 0 ? [](int turn) { if (turn == g_flip) *g_args.state = kNeeds64; }
+                                        : (void (*)(int))nullptr);
+  for (size_t i = 0; i < r.size(); ++i) rz[i] = (double)r[i].hi + r[i].lo;
+  return rc;
+}
 """
 
 
@@ -136,3 +155,14 @@ def chol(lib, n, descending):
                       ctypes.byref(state))
     assert rc == 0, "threads of the block leave while others wait at a barrier"
     return a, state.value
+
+
+def subst(lib, factor, r, descending, flip=-1):
+    """Z of the residuals r [m][128] given k_simt_chol's factor, and the unit's state.  flip: the
+    turn (a thread's run up to its next barrier) before which another block gives the unit to fp64."""
+    f = np.array(factor, dtype=np.float64, order="C")
+    z, state = np.array(r, dtype=np.float64, order="C"), ctypes.c_int(0)
+    rc = lib.run_subst(len(f), int(descending), f.ctypes.data_as(ctypes.c_void_p),
+                       z.ctypes.data_as(ctypes.c_void_p), ctypes.byref(state), flip)
+    assert rc == 0, "threads of the block leave while others wait at a barrier"
+    return z, state.value

@@ -37,3 +37,25 @@ def test_factor_in_any_thread_order(lib, m):
     low = np.tril(np.ones((m, m), bool))
     # 2^-46 per operation, a few hundred of them in a chain, condition number about 1e2
     assert np.abs(up - want)[low].max() <= 2.0 ** -36 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("m", [1, 32, 33, 128])
+def test_substitution_in_any_thread_order(lib, m):
+    n, r = _system(m, m), np.random.default_rng(1).standard_normal((m, 128))
+    f, _ = H.chol(lib, n, False)
+    (up, s0), (down, s1) = H.subst(lib, f, r, False), H.subst(lib, f, r, True)
+    assert s0 == s1 == 0
+    np.testing.assert_array_equal(up, down)
+    want = np.linalg.solve(n, r)
+    assert np.abs(up - want).max() <= 2.0 ** -34 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("flip", [0, 1, 100, 255])
+def test_a_block_agrees_on_leaving_a_unit_to_fp64(lib, flip):
+    """Another block of the unit finds a value outside fp32's range while this one starts."""
+    n, r = _system(40, 7), np.random.default_rng(2).standard_normal((40, 128))
+    f, _ = H.chol(lib, n, False)
+    z, state = H.subst(lib, f, r, False, flip)
+    assert state == 1
+    if flip == 0:
+        assert np.abs(z - r).max() <= 2.0 ** -46 * np.abs(r).max()   # nothing was solved
