@@ -496,16 +496,20 @@ __global__ void __launch_bounds__(256) k_simt_subst(SArgs a, const Df* __restric
   }
 }
 
-// Units left to fp64 (and every unit with m > 128), one CTA each: R and N
-// formed again in fp64 when the pairs lost digits, right-looking Cholesky in
-// global memory, substitution with one column per thread.  Z goes back as
-// pairs.  A non-positive pivot is GRKV_ERR_NUMERIC and leaves V0 in place.
+// Units left to fp64 (and every unit with m > 128), one CTA each: right-looking
+// Cholesky in global memory, substitution with one column per thread.  With m > 128 it starts
+// from the R and N formed in pairs, under k_simt_chol's rule: a pivot too small for pairs, or
+// a residual outside fp32's range, starts the unit over.  Units that pairs cannot hold have R
+// and N formed again in fp64.  Z goes back as pairs.  A non-positive pivot is then
+// GRKV_ERR_NUMERIC and leaves V0 in place.
 template <typename T>
 __global__ void __launch_bounds__(512) k_simt_solve64(const T* __restrict__ v, SArgs a, int all,
                                                       Df* __restrict__ gram,
                                                       Df* __restrict__ rz) {
   chain_wait();
-  __shared__ int bad;
+  __shared__ double diag[kMaxM];
+  enum { kGood, kLost, kNotPositive };
+  __shared__ int pivot;
   const Shape& s = a.s;
   const int u = blockIdx.x, tid = threadIdx.x, m = s.m, B = s.B, nthr = blockDim.x;
   if (!all && a.state[u] != kNeeds64) return;
@@ -516,55 +520,69 @@ __global__ void __launch_bounds__(512) k_simt_solve64(const T* __restrict__ v, S
   Df* Rd = rz + (size_t)u * m * kD;
   double* N = (double*)Gd;
   double* R = (double*)Rd;
-  if (all) {
-    for (int p = tid; p < m * m; p += nthr) {
-      const Df g = Gd[p];
-      N[p] = (double)g.hi + (double)g.lo;
+  for (bool pairs = all;; pairs = false) {
+    if (pairs) {
+      for (int p = tid; p < m * m; p += nthr) {
+        const Df g = Gd[p];
+        N[p] = (double)g.hi + (double)g.lo;
+      }
+      bool out = false;
+      for (int p = tid; p < m * kD; p += nthr) {
+        const Df g = Rd[p];
+        R[p] = (double)g.hi + (double)g.lo;
+        out |= !isfinite(R[p]);
+      }
+      if (__syncthreads_or(out)) continue;
+    } else {
+      for (int p = tid / 32; p < m * m; p += nthr / 32) {   // a warp per entry on or below the diagonal
+        const int r1 = p / m, r2 = p % m;
+        if (r2 > r1) continue;
+        double g = 0.0;
+        for (int i = tid % 32; i < B; i += 32)
+          if (!F[i]) g += (double)X[(size_t)r1 * B + i] * (double)X[(size_t)r2 * B + i];
+        for (int o = 16; o; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+        if (tid % 32 == 0) N[p] = r1 == r2 ? g + (double)s.lambda : g;
+      }
+      for (int p = tid; p < m * kD; p += nthr) {
+        const int r = p / kD, c = p % kD;
+        double g = 0.0;
+        for (int i = 0; i < B; ++i)
+          g += (double)X[(size_t)r * B + i] * (double)ldv(vu, (size_t)rpos(a, u, i) * kD + c);
+        R[p] = (double)a.y[(size_t)u * m * kD + p] - g;
+      }
+      __syncthreads();
     }
-    for (int p = tid; p < m * kD; p += nthr) {
-      const Df g = Rd[p];
-      R[p] = (double)g.hi + (double)g.lo;
-    }
-  } else {
-    for (int p = tid; p < m * m; p += nthr) {
-      const int r1 = p / m, r2 = p % m;
-      double g = r1 == r2 ? (double)s.lambda : 0.0;
-      for (int i = 0; i < B; ++i)
-        if (!F[i]) g += (double)X[(size_t)r1 * B + i] * (double)X[(size_t)r2 * B + i];
-      N[p] = g;
-    }
-    for (int p = tid; p < m * kD; p += nthr) {
-      const int r = p / kD, c = p % kD;
-      double g = 0.0;
-      for (int i = 0; i < B; ++i)
-        g += (double)X[(size_t)r * B + i] * (double)ldv(vu, (size_t)rpos(a, u, i) * kD + c);
-      R[p] = (double)a.y[(size_t)u * m * kD + p] - g;
-    }
-  }
-  __syncthreads();
-  for (int c = 0; c < m; ++c) {
-    if (tid == 0) {
-      const double d = N[(size_t)c * m + c];
-      bad = !(d > 0.0);
-      if (d > 0.0) N[(size_t)c * m + c] = sqrt(d);
-    }
+    if (tid < m) diag[tid] = N[(size_t)tid * m + tid];
     __syncthreads();
-    if (bad) {
+    int now = kGood;
+    for (int c = 0; c < m; ++c) {
+      if (tid == 0) {
+        const double d = N[(size_t)c * m + c];
+        pivot = pairs && !(d > 0x1p-60 && d > 0x1p-20 * diag[c]) ? kLost
+                : !(d > 0.0)                                     ? kNotPositive
+                                                                 : kGood;
+        if (pivot == kGood) N[(size_t)c * m + c] = sqrt(d);
+      }
+      __syncthreads();
+      if ((now = pivot) != kGood) break;
+      const double piv = N[(size_t)c * m + c];
+      for (int i = c + 1 + tid; i < m; i += nthr) N[(size_t)i * m + c] /= piv;
+      __syncthreads();
+      const int rest = m - c - 1;
+      for (int p = tid; p < rest * rest; p += nthr) {
+        const int i = c + 1 + p / rest, j = c + 1 + p % rest;
+        if (j <= i) N[(size_t)i * m + j] -= N[(size_t)i * m + c] * N[(size_t)j * m + c];
+      }
+      __syncthreads();
+    }
+    if (now == kGood) break;
+    if (now == kNotPositive) {
       if (tid == 0) {
         a.state[u] = kSingular;
         set_status(a.status, GRKV_ERR_NUMERIC);
       }
       return;
     }
-    const double piv = N[(size_t)c * m + c];
-    for (int i = c + 1 + tid; i < m; i += nthr) N[(size_t)i * m + c] /= piv;
-    __syncthreads();
-    const int rest = m - c - 1;
-    for (int p = tid; p < rest * rest; p += nthr) {
-      const int i = c + 1 + p / rest, j = c + 1 + p % rest;
-      if (j <= i) N[(size_t)i * m + j] -= N[(size_t)i * m + c] * N[(size_t)j * m + c];
-    }
-    __syncthreads();
   }
   if (tid < kD) {
     for (int i = 0; i < m; ++i) {

@@ -53,23 +53,44 @@ def test_tile_edges(grkv_lib, g, w, n, B, dtype):
         G.assert_values(vo[i], ref["v_out"], dtype)
 
 
-def test_ill_conditioned_unit_is_solved_in_fp64(grkv_lib):
+def _merge_inputs(c, op):
+    ora = [O.compress_unit(c.q[i], c.k[i], c.v[i], op) for i in range(c.U)]
+    return (np.stack([o["scores32"] for o in ora]),
+            np.stack([o["y"].astype(np.float32) for o in ora]), np.stack([o["idx"] for o in ora]))
+
+
+@pytest.mark.parametrize("w,n,B", [(33, 600, 90), (140, 900, 260)], ids=["m33", "m140"])
+def test_ill_conditioned_unit_is_solved_in_fp64(grkv_lib, w, n, B):
     """Two equal window rows and lambda = 1e-9: the second row's Cholesky pivot is about
     2 lambda, far below 2^-20 of its diagonal, so the unit leaves the pair arithmetic.  The equal rows
     have equal residuals, so the merged values stay well determined."""
-    wl = _case(1, 33, 600, 90, "f32")
+    wl = _case(1, w, n, B, "f32")
     c = G.Case(wl)
     c.q[0, 0, 7] = c.q[0, 0, 3]
     c.dq = G.to_device(c.q, wl.dtype)
     # without the causal rule the two rows see the same keys
     op = G.oracle_params(wl, lambda_v=1e-9, causal=False)
     p = G.lib_params(wl, c.U, lambda_v=1e-9, causal=False)
-    ora = [O.compress_unit(c.q[i], c.k[i], c.v[i], op) for i in range(c.U)]
-    s32 = np.stack([o["scores32"] for o in ora])
-    y32 = np.stack([o["y"].astype(np.float32) for o in ora])
+    s32, y32, idx = _merge_inputs(c, op)
     y32[0, 7] = y32[0, 3]
-    idx = np.stack([o["idx"] for o in ora])
     _, vo = G.run_merge(c, p, s32, y32, idx)
     for i in range(c.U):
         ref = O.merge_unit(c.q[i], c.k[i], c.v[i], s32[i], y32[i], idx[i], op)
         G.assert_values(vo[i], ref["v_out"], "f32")
+
+
+@pytest.mark.parametrize("w,n,B", [(40, 700, 150), (140, 900, 260)], ids=["m40", "m140"])
+def test_near_singular_unit_has_fp64_sums(grkv_lib, w, n, B):
+    """Half of the window rows differ from the other half by one rounding of one element, and
+    lambda = 2^-51: the second half's pivots are below the rounding of sums in pairs of floats (which
+    made one non-positive) and above that of fp64 sums."""
+    wl = _case(1, w, n, B, "f32")
+    c, h = G.Case(wl), w // 2
+    c.q[:, 0, h:] = c.q[:, 0, :h]
+    c.q[:, 0, h:, 5] = np.nextafter(c.q[:, 0, :h, 5], np.float32(9))
+    c.dq = G.to_device(c.q, wl.dtype)
+    p = G.lib_params(wl, c.U, lambda_v=2.0 ** -51, causal=False)
+    s32, y32, idx = _merge_inputs(c, G.oracle_params(wl, causal=False))
+    y32[:, h:] = y32[:, :h]
+    _, vo = G.run_merge(c, p, s32, y32, idx)   # the status is GRKV_OK
+    assert np.isfinite(vo).all()
