@@ -6,7 +6,7 @@
 // SM and clock against 128 in fp32, so the products run as pairs of floats
 // (Df): each product is exact (two_prod), sums keep their rounding errors
 // (two_sum), 10 to 12 fp32 instructions per multiply-add, about 2^-46 relative.  A
-// unit that needs more (a pivot far below its diagonal, a value outside
+// unit that needs more (a pivot far below its diagonal, residuals or a Z near the ends of
 // fp32's range) is solved again in fp64 (k_simt_solve64).
 //
 // One CTA per unit and fp64 took 19.3 ms for 8 units of m = 128, B = 512 and
@@ -109,9 +109,14 @@ __device__ __forceinline__ void stv(__nv_bfloat16* p, size_t i, float x) {
   p[i] = __float2bfloat16_rn(x);
 }
 
-// State of a unit's solve (workspace): Z is valid, left to fp64, or the dual
-// system has no Cholesky factor (V_out = V0).
-enum { kSolved = 0, kNeeds64 = 1, kSingular = 2 };
+// State of a unit's solve (workspace): Z is valid, left to fp64, the dual system has no
+// Cholesky factor (V_out = V0), or Z is valid and in fp64.
+enum { kSolved = 0, kNeeds64 = 1, kSingular = 2, kSolved64 = 3 };
+
+// The range of residuals and of Z that pairs of floats hold: products of values below kSmall
+// have rounding errors below fp32's smallest, and sums of 256 values of kLarge stay far below
+// its largest.
+constexpr float kSmall = 0x1p-100f, kLarge = 0x1p100f;
 
 struct SArgs {
   Shape s;
@@ -427,7 +432,8 @@ __global__ void __launch_bounds__(kChT, 1) k_simt_chol(SArgs a, Df* __restrict__
 
 // Z = L^-T L^-1 R by 32-row blocks, 8 columns per CTA; thread (row, column).
 // The factor's blocks are all staged first.
-constexpr size_t kSubstSmem = (size_t)(10 * 32 * kBLD + 128 * 9 + 32 * 9) * sizeof(Df);
+constexpr size_t kSubstSmem =
+    (size_t)(10 * 32 * kBLD + 128 * 9 + 32 * 9) * sizeof(Df) + 8 * sizeof(uint32_t);
 
 __global__ void __launch_bounds__(256) k_simt_subst(SArgs a, const Df* __restrict__ gram,
                                                     Df* __restrict__ rz) {
@@ -436,8 +442,10 @@ __global__ void __launch_bounds__(256) k_simt_subst(SArgs a, const Df* __restric
   Df* Lb = (Df*)sm;                     // block (i, j), j <= i, at i (i + 1) / 2 + j
   Df* W = Lb + 10 * 32 * kBLD;          // [128][9]
   Df* tmp = W + 128 * 9;                // [32][9]
+  uint32_t* seen = (uint32_t*)(tmp + 32 * 9);   // [8] of a column's residuals: 1 nonzero, 2 not small
   const int u = blockIdx.x / (kD / 8), tid = threadIdx.x, r = tid >> 3, c = tid & 7;
   const int m = a.s.m, nb = (m + 31) / 32;
+  if (tid < 8) seen[tid] = 0;
   // another CTA of the unit may give it to fp64 meanwhile: one answer for the block
   if (__syncthreads_or(a.state[u] != kSolved)) return;
   const Df* G = gram + (size_t)u * m * m;
@@ -449,12 +457,16 @@ __global__ void __launch_bounds__(256) k_simt_subst(SArgs a, const Df* __restric
       Lb[((bi * (bi + 1) / 2 + bj) * 32 + i % 32) * kBLD + j % 32] =
           (i < m && j < m) ? G[(size_t)i * m + j] : pad;
     }
+  uint32_t size = 0;
   for (int b = 0; b < nb; ++b) {
     const int i = b * 32 + r;
-    W[i * 9 + c] = i < m ? Z[(size_t)i * kD + c] : Df{0.f, 0.f};
+    const Df x = i < m ? Z[(size_t)i * kD + c] : Df{0.f, 0.f};
+    W[i * 9 + c] = x;
+    size |= (x.hi != 0.f ? 1u : 0u) | (fabsf(x.hi) >= kSmall ? 2u : 0u);
   }
+  atomicOr(&seen[c], size);
   __syncthreads();
-  bool finite = true;
+  bool fits = seen[c] != 1u;
   auto solve_block = [&](int b, Df acc, bool back) {
     tmp[r * 9 + c] = df_norm(acc);
     __syncthreads();
@@ -464,7 +476,7 @@ __global__ void __launch_bounds__(256) k_simt_subst(SArgs a, const Df* __restric
     for (int e = 0; e < 32; ++e) df_mac(z, back ? I[e * kBLD + r] : I[r * kBLD + e], tmp[e * 9 + c]);
     z = df_norm(z);
     W[(b * 32 + r) * 9 + c] = z;
-    if (back) finite = finite && isfinite(z.hi);
+    if (back) fits = fits && fabsf(z.hi) < kLarge;   // false for NaN
     __syncthreads();
   };
   for (int b = 0; b < nb; ++b) {   // L W = R
@@ -485,8 +497,8 @@ __global__ void __launch_bounds__(256) k_simt_subst(SArgs a, const Df* __restric
     }
     solve_block(b, acc, true);
   }
-  // outside fp32's range: R is needed again, so Z is only written when it holds
-  if (__syncthreads_or(!finite)) {
+  // outside the range of pairs: R is needed again, so Z is only written when it holds
+  if (__syncthreads_or(!fits)) {
     if (tid == 0) a.state[u] = kNeeds64;
     return;
   }
@@ -498,16 +510,17 @@ __global__ void __launch_bounds__(256) k_simt_subst(SArgs a, const Df* __restric
 
 // Units left to fp64 (and every unit with m > 128), one CTA each: right-looking
 // Cholesky in global memory, substitution with one column per thread.  With m > 128 it starts
-// from the R and N formed in pairs, under k_simt_chol's rule: a pivot too small for pairs, or
-// a residual outside fp32's range, starts the unit over.  Units that pairs cannot hold have R
-// and N formed again in fp64.  Z goes back as pairs.  A non-positive pivot is then
-// GRKV_ERR_NUMERIC and leaves V0 in place.
+// from the R and N formed in pairs, under the rules of k_simt_chol and k_simt_subst: a pivot or
+// a residual that pairs cannot hold starts the unit over.  Such units have R and N formed again
+// in fp64.  Z goes back as pairs, or stays in fp64 where a column is outside their range.  A
+// non-positive pivot is then GRKV_ERR_NUMERIC and leaves V0 in place.
 template <typename T>
 __global__ void __launch_bounds__(512) k_simt_solve64(const T* __restrict__ v, SArgs a, int all,
                                                       Df* __restrict__ gram,
                                                       Df* __restrict__ rz) {
   chain_wait();
   __shared__ double diag[kMaxM];
+  __shared__ uint8_t seen[512];
   enum { kGood, kLost, kNotPositive };
   __shared__ int pivot;
   const Shape& s = a.s;
@@ -526,13 +539,20 @@ __global__ void __launch_bounds__(512) k_simt_solve64(const T* __restrict__ v, S
         const Df g = Gd[p];
         N[p] = (double)g.hi + (double)g.lo;
       }
-      bool out = false;
+      // thread (phase, column): kD divides the block's threads
+      bool finite = true, nonzero = false, fits = false;
       for (int p = tid; p < m * kD; p += nthr) {
         const Df g = Rd[p];
         R[p] = (double)g.hi + (double)g.lo;
-        out |= !isfinite(R[p]);
+        finite = finite && isfinite(R[p]);
+        nonzero |= g.hi != 0.f;
+        fits |= fabsf(g.hi) >= kSmall;
       }
-      if (__syncthreads_or(out)) continue;
+      seen[tid] = (nonzero ? 1 : 0) | (fits ? 2 : 0);
+      __syncthreads();
+      int size = 0;
+      for (int h = tid % kD; h < nthr; h += kD) size |= seen[h];
+      if (__syncthreads_or(!finite || size == 1)) continue;
     } else {
       for (int p = tid / 32; p < m * m; p += nthr / 32) {   // a warp per entry on or below the diagonal
         const int r1 = p / m, r2 = p % m;
@@ -584,7 +604,9 @@ __global__ void __launch_bounds__(512) k_simt_solve64(const T* __restrict__ v, S
       return;
     }
   }
+  bool wide = false;   // the thread's column of Z does not fit pairs
   if (tid < kD) {
+    double largest = 0.0;
     for (int i = 0; i < m; ++i) {
       double z = R[(size_t)i * kD + tid];
       for (int c = 0; c < i; ++c) z -= N[(size_t)i * m + c] * R[(size_t)c * kD + tid];
@@ -593,19 +615,37 @@ __global__ void __launch_bounds__(512) k_simt_solve64(const T* __restrict__ v, S
     for (int i = m - 1; i >= 0; --i) {
       double z = R[(size_t)i * kD + tid];
       for (int c = i + 1; c < m; ++c) z -= N[(size_t)c * m + i] * R[(size_t)c * kD + tid];
-      R[(size_t)i * kD + tid] = z / N[(size_t)i * m + i];
+      z /= N[(size_t)i * m + i];
+      R[(size_t)i * kD + tid] = z;
+      largest = fmax(largest, fabs(z));
+      wide |= !(fabs(z) < (double)kLarge);   // NaN too
     }
-    for (int i = 0; i < m; ++i) {
-      const double z = R[(size_t)i * kD + tid];
-      const float hi = (float)z;
-      Rd[(size_t)i * kD + tid] = {hi, (float)(z - (double)hi)};
-    }
+    wide |= largest > 0.0 && largest < (double)kSmall;
   }
-  if (tid == 0) a.state[u] = kSolved;
+  wide = __syncthreads_or(wide);
+  if (tid == 0) a.state[u] = wide ? kSolved64 : kSolved;
+  if (wide || tid >= kD) return;
+  for (int i = 0; i < m; ++i) {
+    const double z = R[(size_t)i * kD + tid];
+    const float hi = (float)z;
+    Rd[(size_t)i * kD + tid] = {hi, (float)(z - (double)hi)};
+  }
+}
+
+// One output in fp64: a column x [m] of X, a column z [m] of Z, in fp64 if wide.
+__device__ __noinline__ float update64(const float* x, int B, const Df* z, int m, bool wide,
+                                       float v0) {
+  double g = 0.0;
+  for (int r = 0; r < m; ++r) {
+    const Df p = z[(size_t)r * kD];
+    const double zr = wide ? ((const double*)z)[(size_t)r * kD] : (double)p.hi + (double)p.lo;
+    g += (double)x[(size_t)r * B] * zr;
+  }
+  return (float)((double)v0 + g);
 }
 
 // V_out[G] = V0[G] + X_G^T Z, V_out[F] = V0[F]: 32 slots x 32 columns per CTA,
-// four outputs per thread.
+// four outputs per thread.  Outputs that pairs cannot hold are formed in fp64.
 template <typename T, typename A>
 __global__ void __launch_bounds__(256) k_simt_update(const T* __restrict__ v,
                                                      T* __restrict__ v_out, SArgs a,
@@ -624,7 +664,8 @@ __global__ void __launch_bounds__(256) k_simt_update(const T* __restrict__ v,
 #pragma unroll
   for (int i = 0; i < 4; ++i) zero(acc[i]);
   const bool keep = s.lambda_inf || a.state[u] == kSingular;   // V_out = V0
-  for (int r0 = 0; r0 < m && !keep; r0 += 32) {
+  const bool wide = !s.lambda_inf && a.state[u] == kSolved64;
+  for (int r0 = 0; r0 < m && !keep && !wide; r0 += 32) {
     __syncthreads();
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -649,10 +690,14 @@ __global__ void __launch_bounds__(256) k_simt_update(const T* __restrict__ v,
     if (slot >= B) break;
     const size_t o = ((size_t)u * B + slot) * kD + c0 + lane;
     const T v0 = vu[(size_t)rpos(a, u, slot) * kD + c0 + lane];
-    if (keep || a.flags[(size_t)u * B + slot])
+    if (keep || a.flags[(size_t)u * B + slot]) {
       v_out[o] = v0;
-    else
-      stv(v_out, o, value(plus(acc[i], ldv(&v0, 0))));
+      continue;
+    }
+    float x = value(plus(acc[i], ldv(&v0, 0)));
+    if constexpr (std::is_same<A, Df>::value)
+      if (wide || !isfinite(x)) x = update64(X + slot, B, Z + c0 + lane, m, wide, ldv(&v0, 0));
+    stv(v_out, o, x);
   }
 }
 

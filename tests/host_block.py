@@ -37,6 +37,7 @@ static float __fadd_rn(float a, float b) { return a + b; }
 static float __fsub_rn(float a, float b) { return a - b; }
 static float __fmul_rn(float a, float b) { return a * b; }
 static float __fmaf_rn(float a, float b, float c) { return fmaf(a, b, c); }
+static uint32_t atomicOr(uint32_t* p, uint32_t v) { const uint32_t old = *p; *p |= v; return old; }
 static void chain_wait() {}
 
 struct Fiber { ucontext_t ctx; std::vector<char> stack; bool done; int pred; };
@@ -89,7 +90,6 @@ static int run_block(int threads, unsigned block, bool descending, void (*kernel
 constexpr int kD = 128;
 struct Shape { int m; };
 struct SArgs { Shape s; int* state; };
-enum { kSolved = 0, kNeeds64 = 1, kSingular = 2 };
 alignas(16) float sm[1 << 16];
 """
 
@@ -138,6 +138,7 @@ def load(tmp):
     with open(SRC) as f:
         text = f.read()
     code = (HARNESS + _slice(text, "struct alignas(8) Df {", "// Accumulator policies")
+            + _slice(text, "// State of a unit's solve", "struct SArgs {")
             + _slice(text, "constexpr int kChT", "// Units left to fp64") + ENTRY)
     code = re.sub(r"#pragma unroll.*", "", code)
     src, lib = os.path.join(tmp, "block.cpp"), os.path.join(tmp, "block.so")

@@ -94,3 +94,24 @@ def test_near_singular_unit_has_fp64_sums(grkv_lib, w, n, B):
     y32[:, h:] = y32[:, :h]
     _, vo = G.run_merge(c, p, s32, y32, idx)   # the status is GRKV_OK
     assert np.isfinite(vo).all()
+
+
+@pytest.mark.parametrize("w,n,B", [(40, 700, 150), (140, 900, 260)], ids=["m40", "m140"])
+@pytest.mark.parametrize("exp", [-134, 125])
+def test_values_at_the_ends_of_fp32(grkv_lib, w, n, B, exp):
+    """Values whose products' rounding errors are below fp32's range (subnormal values), and
+    values whose Z = N^-1 R is above it: both ends were within an fp64 regression's range."""
+    wl = _case(1, w, n, B, "f32")
+    c = G.Case(wl)
+    c.v = np.ldexp(c.v / np.abs(c.v).max(), exp).astype(np.float32)
+    c.dv = G.to_device(c.v, wl.dtype)
+    op = G.oracle_params(wl)
+    s32, y32, idx = _merge_inputs(c, op)
+    _, vo = G.run_merge(c, G.lib_params(wl, c.U), s32, y32, idx)
+    for i in range(c.U):
+        ref = O.merge_unit(c.q[i], c.k[i], c.v[i], s32[i], y32[i], idx[i], op)["v_out"]
+        # the last rounding (half a unit, 2^-150 or 2^-24 relative), and X's fp32 error, a few
+        # 1e-6, times |X_G^T N^-1| <= 1 / (2 sqrt(lambda)) = 5 times |R|'s scale
+        lim = 2.0 ** -149 + 2.0 ** -23 * np.abs(ref) + 2e-5 * np.abs(c.v[i]).max()
+        err = np.abs(vo[i].astype(np.float64) - ref)
+        assert (err <= lim).all(), f"{err.max():.3e} against {lim.max():.3e}"

@@ -59,3 +59,13 @@ def test_a_block_agrees_on_leaving_a_unit_to_fp64(lib, flip):
     assert state == 1
     if flip == 0:
         assert np.abs(z - r).max() <= 2.0 ** -46 * np.abs(r).max()   # nothing was solved
+
+
+@pytest.mark.parametrize("exp,state", [(-99, 0), (-101, 1), (98, 1)])
+def test_a_column_outside_the_range_of_pairs(lib, exp, state):
+    """One small (or, after N^-1, large) column gives the unit to fp64; a zero column does not."""
+    n, r = _system(40, 7), np.random.default_rng(2).standard_normal((40, 128))
+    r[:, 3] = 0.0
+    r[:, 77] = np.ldexp(np.sign(r[:, 77]), exp)
+    f, _ = H.chol(lib, n, False)
+    assert H.subst(lib, f, r, False)[1] == state
