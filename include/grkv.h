@@ -91,7 +91,9 @@ extern "C" {
                                     instead of with float atomics (costs a workspace of
                                     U x slots x m x d floats and one more kernel; selects
                                     the two-launch scoring even with GRKV_ONE_READ_SCORE).
-                                    Every other step is reproducible in either mode */
+                                    Every other step is reproducible in either mode.  A
+                                    unit's last bits may differ between calls with other
+                                    numbers of units: few units are split further */
 
 #define GRKV_CHECKS        0x10u /* device-side argument checks, written to the status word:
                                     a non-finite q, k or v element -> GRKV_ERR_INVALID_ARG;
@@ -196,7 +198,8 @@ int grkv_compress(const grkv_params* p, const void* q, const void* k, const void
  * Outputs are packed: unit u's budgets[u] entries of idx and rows of k_out /
  * v_out start at row off_u = budgets[0] + ... + budgets[u-1] (idx [sum B_u]
  * int32, k_out / v_out [sum B_u][d]); each unit's results are those of
- * grkv_compress with B = budgets[u].  The scoring step, and on the
+ * grkv_compress on the same units with B = budgets[u], under GRKV_DETERMINISTIC
+ * bit for bit (up to rounding with the key step).  The scoring step, and on the
  * tensor-core value step the selection and the merge, run once over all
  * units; the portable value step and the key step run once per run of
  * consecutive units with equal budgets.  ws must hold

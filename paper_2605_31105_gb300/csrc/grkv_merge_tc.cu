@@ -370,8 +370,8 @@ __global__ void __launch_bounds__(256) k_merge_fixed(MArgs a) {
 }
 
 // ======================================================== k_merge_gram
-// A cluster of a.ranks CTAs per unit and row block, each on a contiguous share of
-// the unit's tiles; the shares of R~ and of the Gram meet in distributed shared
+// A cluster of a.ranks CTAs (a power of two) per unit and row block, each on a contiguous
+// share of the unit's tiles; the shares of R~ and of the Gram meet in distributed shared
 // memory, where rank r adds rows [128 r / ranks, 128 (r + 1) / ranks) of all shares
 // in rank order and writes them.
 //
@@ -452,7 +452,12 @@ __global__ void __launch_bounds__(kThreadsG, 1)
   const int u = ub / a.nrb, row0 = (ub % a.nrb) * kRows;   // window rows row0 .. row0 + 127
   const UnitRow ur = unit_row(a.units, u, a.B, a.n_fix);
   const int B = ur.B, T = (B + kTile - 1) / kTile;
-  const int ta = T * rank / C, tb = T * (rank + 1) / C;    // this rank's tiles
+  // A unit is split as launch_gram splits a call at its own budget, so that its sums, and
+  // with them its results' last bits, do not follow the largest budget of the call.
+  int split = C;
+  while (split > T) split /= 2;
+  const int ta = rank < split ? T * rank / split : T;      // this rank's tiles
+  const int tb = rank < split ? T * (rank + 1) / split : T;
   const int ng = __ldg(a.ng + u);
   if (tid == 0) {
     for (int i = 0; i < kRingG; ++i) {
@@ -1298,7 +1303,8 @@ MergeWs merge_ws(const Shape& s) {
 }
 
 // As many ranks as leave every cluster room on the SMs at once: 8 units of B = 512
-// take 15 us with four ranks, one tile each.
+// take 15 us with four ranks, one tile each.  With budgets per unit B is the largest; the
+// kernel leaves ranks of units with fewer tiles idle.
 cudaError_t launch_gram(const CUtensorMap& mq, MArgs a, cudaStream_t st) {
   const int tiles = (a.B + kTile - 1) / kTile, blocks = a.U * a.nrb;
   a.ranks = 1;

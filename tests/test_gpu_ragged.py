@@ -63,10 +63,12 @@ def test_equal_budgets_are_grkv_compress(grkv_lib):
 
 @pytest.mark.parametrize("wl,pattern", [
     (gi.workload(1).replace(units=6, n=1500, budget=0), [32, 33, 127, 128, 129, 640]),
+    # three tiles of 128 slots beside one and nine: the Gram's ranks follow a unit's own budget
+    (gi.workload(1).replace(units=6, n=1500, budget=0), [300, 1100, 384, 100, 257, 640]),
     (gi.Workload("m256", 3, 4, 1200, 128, 64, 0, 7, 1e-1, "bf16", "spans", 321), [64, 200, 256]),
     # more units than one chunk of the budget table holds
     (gi.Workload("many", 965, 1, 150, 128, 8, 0, 5, 1e-2, "bf16", "lowrank", 55), [9, 60, 8, 130]),
-], ids=["tile_edges", "m256", "two_chunks"])
+], ids=["tile_edges", "three_tiles", "m256", "two_chunks"])
 def test_mixed_budgets_are_grkv_compress_unit_by_unit(grkv_lib, wl, pattern):
     """Every unit's rows equal grkv_compress's at that unit's budget, bit for bit, and the
     packed rows of a unit end where the next unit's begin."""
