@@ -251,9 +251,11 @@ int grkv_transfer_check(const grkv_params* p, int32_t held, const void* q_win,
  * nothing: the pooled scores go to a 16 MiB array in the library's device
  * image, which every GPU that loads the library holds until the process exits.
  * Prefixes of n - window <= 32768 positions are selected in shared memory and
- * use no scratch, at any unit count.  Longer prefixes use the array, limited
- * to units * (n - window) <= 4,194,304 floats; larger sizes return
- * GRKV_ERR_WORKSPACE_TOO_SMALL.  The first call on a device looks up the
+ * use no scratch, at any unit count.  Longer prefixes may use the array (past
+ * 262144 positions, with pooling wider than 129, or on a partition of the GPU
+ * that holds no cluster of 8 CTAs), limited to units * (n - window) <=
+ * 4,194,304 floats; larger sizes return GRKV_ERR_WORKSPACE_TOO_SMALL whether
+ * or not the array would be used.  The first call on a device looks up the
  * array's device address (cudaGetSymbolAddress) with that device current;
  * make that first call before any stream capture.  All calls share the array
  * and it keeps the last call's contents; every element a call reads is first

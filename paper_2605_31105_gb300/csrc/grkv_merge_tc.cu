@@ -1309,6 +1309,7 @@ cudaError_t launch_gram(const CUtensorMap& mq, MArgs a, cudaStream_t st) {
   const int tiles = (a.B + kTile - 1) / kTile, blocks = a.U * a.nrb;
   a.ranks = 1;
   while (a.ranks < 8 && 2 * a.ranks <= tiles && blocks * 2 * a.ranks <= kClusterSms) a.ranks *= 2;
+  while (a.ranks > 1 && !cluster_fits(a.ranks, k_merge_gram, kThreadsG, kSmemBytes)) a.ranks /= 2;
   return launch_kernel(true, a.ranks, k_merge_gram, dim3(blocks * a.ranks), kThreadsG, kSmemBytes, st,
                        mq, a);
 }

@@ -13,8 +13,8 @@
 // positions per thread, four full histogram passes and two scans it took 33 us
 // for n - w = 8160 (255 threads at work) and 317 us for 131,008 (one CTA
 // re-reading a pooled copy from global memory).
-// Longer prefixes, and pooling wider than 129, take k_select (a pooled copy in
-// the workspace).
+// Longer prefixes, pooling wider than 129, and devices that hold no cluster of 8 take
+// k_select (a pooled copy in the workspace).
 #include <algorithm>
 #include <cmath>
 
@@ -516,6 +516,7 @@ cudaError_t launch_reg(const Shape& s, const float* scores, int32_t* idx, cudaSt
   const size_t bytes = reg_smem_bytes(kPer, kCs > 1 ? kMaxHalo : 0);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   if (e != cudaSuccess) return e;
+  if (kCs > 1 && !cluster_fits(kCs, kern, kThr, bytes)) return cudaErrorInvalidClusterSize;
   return launch_kernel(s.chained, kCs, kern, dim3((unsigned)s.U * kCs), kThr, bytes, st, scores, s, idx);
 }
 
@@ -532,11 +533,16 @@ cudaError_t launch_select_pooled(const Shape& s, const float* scores, int32_t* i
   if (per <= 8) return launch_reg<8, 1>(s, scores, idx, st);
   if (per <= 16) return launch_reg<16, 1>(s, scores, idx, st);
   if (per <= 32) return launch_reg<32, 1>(s, scores, idx, st);
+  cudaError_t e = cudaErrorInvalidClusterSize;   // until a cluster takes it
   if (s.pool_k / 2 <= kMaxHalo) {
-    if (per <= 8 * kCluster) return launch_reg<8, kCluster>(s, scores, idx, st);
-    if (per <= 16 * kCluster) return launch_reg<16, kCluster>(s, scores, idx, st);
-    if (s.P <= kMaxClusterP) return launch_reg<32, kCluster>(s, scores, idx, st);
+    if (per <= 8 * kCluster)
+      e = launch_reg<8, kCluster>(s, scores, idx, st);
+    else if (per <= 16 * kCluster)
+      e = launch_reg<16, kCluster>(s, scores, idx, st);
+    else if (s.P <= kMaxClusterP)
+      e = launch_reg<32, kCluster>(s, scores, idx, st);
   }
+  if (e != cudaErrorInvalidClusterSize) return e;
   return launch_kernel(s.chained, 1, k_select, dim3(s.U), 1024, 0, st, scores, s, pooled, idx);
 }
 
