@@ -137,8 +137,6 @@ void count_launches(int n) { g_launches.fetch_add((uint64_t)n, std::memory_order
 WsLayout plan_workspace(const Shape& s) {
   WsLayout L{};
   const size_t U = (size_t)s.U, m = (size_t)s.m, d = (size_t)kD;
-  L.chunk = score_simt_chunk(s);
-  L.nchunk = (s.n + L.chunk - 1) / L.chunk;
   size_t off = 0;
   auto take = [&](size_t bytes) {
     const size_t at = off;
@@ -153,6 +151,8 @@ WsLayout plan_workspace(const Shape& s) {
     L.lam_tc = take(U * 128 * sizeof(float));
     if (s.deterministic) L.ypart_tc = take(U * (size_t)maxc * m * d * sizeof(float));
   } else {
+    L.chunk = score_simt_chunk(s);
+    L.nchunk = (s.n + L.chunk - 1) / L.chunk;
     L.pstats = take(U * L.nchunk * m * 8);
     L.ypart = take(U * L.nchunk * m * d * 4);
   }

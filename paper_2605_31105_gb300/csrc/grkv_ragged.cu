@@ -51,10 +51,10 @@ struct RaggedPlan {
   bool once;                  // selection and merge in one launch each
   size_t table;               // UnitRow [U] (once)
   Shape all;                  // every unit, the largest budget (scoring only)
+  WsLayout layout;            // the scoring workspace (status word first)
   std::vector<int> begin;     // first unit of each run
   std::vector<int> budget;    // its budget
   std::vector<size_t> off;    // packed row offset of each unit (U + 1 entries)
-  size_t main_total;          // the scoring workspace (status word first)
   size_t run_ws;              // offset of the per-run workspace
   size_t run_total;           // its size (the largest run's)
   size_t idx_scratch;         // 16-byte aligned idx of the current run
@@ -75,7 +75,7 @@ int plan_ragged(const grkv_params* p, const int32_t* budgets, RaggedPlan* r) {
   r->begin.clear();
   r->budget.clear();
   r->off.assign(1, 0);
-  r->main_total = plan_workspace(r->all).total;
+  r->layout = plan_workspace(r->all);
   // packed rows index the output tensor maps; a chunk's scan is 32-bit
   size_t run_total = 0, idx_max = 0, rows = 0;
   for (int u = 0; u < p->units; ++u) rows += (size_t)budgets[u];
@@ -88,7 +88,7 @@ int plan_ragged(const grkv_params* p, const int32_t* budgets, RaggedPlan* r) {
     }
   }
   if (r->once) {
-    r->table = align256(r->main_total);
+    r->table = align256(r->layout.total);
     r->total = align256(r->table + (size_t)p->units * sizeof(UnitRow));
     return GRKV_OK;
   }
@@ -102,7 +102,7 @@ int plan_ragged(const grkv_params* p, const int32_t* budgets, RaggedPlan* r) {
     run_total = std::max(run_total, plan_workspace(s).total);
     idx_max = std::max(idx_max, (size_t)s.U * s.B);
   }
-  r->run_ws = align256(r->main_total);
+  r->run_ws = align256(r->layout.total);
   r->run_total = run_total;
   r->idx_scratch = align256(r->run_ws + run_total);
   r->total = align256(r->idx_scratch + idx_max * sizeof(int32_t));
@@ -146,7 +146,7 @@ extern "C" int grkv_compress_ragged(const grkv_params* p, const int32_t* budgets
     return rc;
   cudaStream_t st = (cudaStream_t)stream;
   char* w = (char*)ws;
-  const WsLayout L = plan_workspace(s);
+  const WsLayout& L = r.layout;
   if (cudaMemsetAsync(w + L.status, 0, 4, st) != cudaSuccess) return GRKV_ERR_CUDA;
   if (s.U == 0) return GRKV_OK;
   float* scores = (float*)(w + L.scores);

@@ -338,19 +338,23 @@ cudaError_t launch_score_simt(const Shape& s, const void* q, const void* k, cons
 // Keys per CTA of the portable scoring passes: whole tiles of 64, so that the
 // U x chunks CTAs (one per SM at a time) finish soonest, a CTA costing its
 // tiles plus about two tiles of set-up.
+// One chunk count is tried per chunk size: the smallest that gives it.
 int score_simt_chunk(const Shape& s) {
-  const long long tiles = (s.n + kKeys - 1) / kKeys, sms = 152, U = std::max(s.U, 1);
-  long long best = 1, cost = -1;
-  for (long long chunks = 1; chunks <= std::min(tiles, 608ll); ++chunks) {
-    const long long per = (tiles + chunks - 1) / chunks;
-    const long long ctas = U * ((tiles + per - 1) / per);
-    const long long c = (ctas + sms - 1) / sms * (per + 2);
+  const int tiles = (s.n + kKeys - 1) / kKeys, sms = 152;
+  const long long U = std::max(s.U, 1);
+  long long cost = -1;
+  int best = 1;
+  for (int chunks = 1; chunks <= std::min(tiles, 608);) {
+    const int per = (tiles + chunks - 1) / chunks, used = (tiles + per - 1) / per;
+    const long long c = (U * used + sms - 1) / sms * (per + 2);
     if (cost < 0 || c < cost) {
       cost = c;
       best = per;
     }
+    if (per == 1) break;
+    chunks = (tiles + per - 2) / (per - 1);   // the first with smaller chunks
   }
-  return (int)best * kKeys;
+  return best * kKeys;
 }
 
 }  // namespace grkv

@@ -95,6 +95,30 @@ def test_workspace_size_and_validation(lib):
     assert b.grkv_workspace_size(b.params(8, 4, 8192, 32, 512, lambda_v=float("inf"))) > 0
 
 
+def _portable_scoring_chunks(units, n):
+    """Chunks of 64-key tiles per unit: the fewest rounds of 152 CTAs, a CTA costing its tiles plus two."""
+    tiles, best = (n + 63) // 64, None
+    for chunks in range(1, min(tiles, 608) + 1):
+        per = -(-tiles // chunks)
+        cost = -(-units * -(-tiles // per) // 152) * (per + 2)
+        if best is None or cost < best[0]:
+            best = (cost, per)
+    return -(-n // (64 * best[1]))
+
+
+@pytest.mark.parametrize("units", [1, 3, 8, 151, 256])
+def test_portable_workspace_follows_the_chunk_search(lib, units):
+    for n in (40, 64, 65, 1000, 5003, 8192, 38913, 131072):
+        g, w, B = 2, 20, 40
+        m, P, total = g * w, n - w, 0
+        c = _portable_scoring_chunks(units, n)
+        for nbytes in (256, units * c * m * 8, units * c * m * 512, units * P * 4, units * m * B * 4,
+                       units * B, units * m * m * 8, units * m * 128 * 8, units * 4, units * P * 4,
+                       units * m * 512, units * m * 8):
+            total += -(-nbytes // 256) * 256
+        assert b.grkv_workspace_size(b.params(units, g, n, w, B, dtype="f32")) == total
+
+
 def test_host_checks_before_any_launch(lib):
     p = b.params(2, 4, 1024, 32, 128)
     need = b.grkv_workspace_size(p)
