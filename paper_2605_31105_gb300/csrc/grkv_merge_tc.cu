@@ -110,6 +110,12 @@ __device__ __forceinline__ uint32_t xt_col(int kk, int lo) {
   return (kk >> 1) * 32 + lo * 16 + (kk & 1) * 8;
 }
 
+// The wait for copies or MMAs in flight at the end of a CTA: bounded, whether or not another
+// wait has given up.
+__device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity) {
+  volatile int no_abort = 0;
+  mbar_wait(bar, parity, &no_abort, kBudget);
+}
 // mbar_wait for all lanes of a warp with one answer, so that warp-collective
 // instructions after a wait are reached by all lanes or by none.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort) {
@@ -178,9 +184,8 @@ struct Gatherer {
     return true;
   }
   // every issued gather lands before the CTA can exit
-  __device__ __forceinline__ void drain(volatile int* abort_flag) {
-    for (uint32_t i = use > R ? use - R : 0; i < use; ++i)
-      mbar_wait(&full[i % R], (i / R) & 1, abort_flag, kBudget);
+  __device__ __forceinline__ void drain() {
+    for (uint32_t i = use > R ? use - R : 0; i < use; ++i) mbar_drain(&full[i % R], (i / R) & 1);
   }
 };
 
@@ -719,11 +724,11 @@ __global__ void __launch_bounds__(kThreadsG, 1)
     cluster_bar();   // no rank leaves while a peer reads its shares
     break;
   }
+  if (warp == 0 && lane == 0) mbar_drain(&bars->q_full, 0);
   if (warp == 1) {
     // every MMA issued completes before TMEM is released
     mma_commit_elect(&bars->drain);
-    volatile int no_abort = 0;
-    mbar_wait(&bars->drain, 0, &no_abort, kBudget);
+    mbar_drain(&bars->drain, 0);
   }
   if (!ok && lane == 0) set_status(a.status, GRKV_ERR_TIMEOUT);
   tc_fence_before();
@@ -816,7 +821,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (t + 1 < TG) gt.rows(src_u, B, a.n, u * a.n, t + 1, pw, lane, jn);
       ok = gt.load(&tmK, j, pw, lane, abort_flag);
     }
-    gt.drain(abort_flag);
+    gt.drain();
+    if (warp == 0 && lane == 0) mbar_drain(&bars->q_full, 0);
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t id_g = idesc_bf16(kRows, kRows, 0, 0);   // G01 += A XG1^T
@@ -857,7 +863,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       mma_commit(&bars->acc_done);
       mma_commit(&bars->drain);
-      mbar_wait(&bars->drain, 0, abort_flag, kBudget);
+      mbar_drain(&bars->drain, 0);
     }
   } else {
     const int grp = (warp - 4) >> 2, q = warp & 3, row = q * 32 + lane;
@@ -1062,6 +1068,7 @@ __global__ void __launch_bounds__(kThreadsU, 1)
         mbar_arrive(&bars->k_empty[sl]);
       }
       bulk_wait_all();
+      mbar_drain(&bars->q_full, 0);
       if (!ok) set_status(a.status, GRKV_ERR_TIMEOUT);
     }
     __syncwarp();
@@ -1107,7 +1114,7 @@ __global__ void __launch_bounds__(kThreadsU, 1)
       if (t + 1 < T) g.rows(idx_u, B, a.n, row0, T0 + t + 1, pw, lane, jn);
       ok = g.load(&tmK, j, pw, lane, abort_flag);
     }
-    g.drain(abort_flag);
+    g.drain();
   } else if (warp >= 18 && warp < 22) {
     // V0 gathers: a quarter of every tile each (own ring, so that a K tile never waits
     // for a V slot); only threads read a V0 tile, so the copies themselves arrive
@@ -1159,8 +1166,7 @@ __global__ void __launch_bounds__(kThreadsU, 1)
     }
     if (ok && T > 0) ok = issue_d(T - 1);
     mma_commit_elect(&bars->drain);
-    volatile int no_abort = 0;
-    mbar_wait(&bars->drain, 0, &no_abort, kBudget);
+    mbar_drain(&bars->drain, 0);
   } else if (warp >= 4 && warp < 12) {
     // compute groups: group cg takes the tiles t with t % 2 == cg
     const int cg = (warp - 4) >> 2, q = warp & 3, tok = q * 32 + lane;
