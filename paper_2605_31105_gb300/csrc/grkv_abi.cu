@@ -102,7 +102,6 @@ int make_shape(const grkv_params* p, Shape* s) {
   s->B = p->budget;
   s->m = p->group * p->window;
   s->P = p->n - p->window;
-  s->kk = p->budget - p->window;
   s->pool_k = p->pool_kernel;
   s->pool_type = p->pool_type;
   s->n_sink = p->n_sink;

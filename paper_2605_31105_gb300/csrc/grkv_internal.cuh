@@ -30,7 +30,6 @@ struct UnitRow {
 struct Shape {
   int U, g, n, d, w, B, m;
   int P;          // prefix length n - w (scored, pooled, selectable)
-  int kk;         // prefix tokens kept: B - w
   int pool_k, pool_type, n_sink, n_fix, causal, dtype;
   float lambda, scale;
   int lambda_inf; // lambda_v == +inf: values stay V0

@@ -71,8 +71,7 @@ constexpr uint32_t kColD = 256;
 
 struct MArgs {
   int U, n, w, m, P, B, causal, n_sink, n_fix;
-  float sl2, lambda;
-  int lambda_inf;
+  float sl2;
   const int32_t* idx;        // [U][B]
   const float* scores;       // [U][P]
   const float* y;            // [U][m][128]
@@ -88,10 +87,10 @@ struct MArgs {
   int32_t* ng;               // [U]            number of non-fixed slots
   uint8_t* fixed;            // [U][B]         1 for a fixed slot
   int ranks;                 // k_merge_gram: CTAs per unit and row block
-  // Row blocks (m > 128): an update launch takes the 128 window rows row0 .. row0+127
-  // of block rb (of nrb); the per-unit arrays hold ldr rows (128 or 256):
+  // Row blocks (nrb of them): an update launch takes the 128 window rows row0 .. row0+127;
+  // the per-unit arrays hold ldr rows (128 or 256):
   // rz [U][ldr][128], gram [U][ldr][ldr], lam [U][ldr].
-  int row0, rb, nrb, ldr;
+  int row0, nrb, ldr;
   int upd_mode;              // update: 0 V_out = V0 + dV; 1 vpart = V0 + dV; 2 V_out = vpart + dV
   float* vpart;              // [U][B][128] fp32, between the update's two row blocks
   int* status;
@@ -1347,8 +1346,6 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
   a.n_sink = s.n_sink;
   a.n_fix = s.n_fix;
   a.sl2 = (float)((double)s.scale * 1.4426950408889634);
-  a.lambda = s.lambda;
-  a.lambda_inf = s.lambda_inf;
   a.idx = idx;
   a.scores = scores;
   a.y = y;
@@ -1404,7 +1401,6 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
                         a.status, st)) != cudaSuccess)
     return e;
   if (W.nrb == 1) {
-    a.rb = 0;
     a.row0 = 0;
     a.upd_mode = 0;
     if ((e = launch_kernel(true, 1, k_merge_update, dim3(s.U * a.split), kThreadsU, kSmemBytesU, st, mq,
@@ -1415,7 +1411,6 @@ cudaError_t launch_merge_tc(const Shape& s, const void* q, const void* k, const 
     // the value update of each row block (the first leaves V0 + dV_0 in vpart)
     launches = 0;
     for (int rb = 0; rb < 2; ++rb) {
-      a.rb = rb;
       a.row0 = rb * kRows;
       a.upd_mode = rb == 0 ? 1 : 2;
       if ((e = launch_kernel(true, 1, k_merge_update, dim3(s.U * a.split), kThreadsU, kSmemBytesU, st, mq,

@@ -64,20 +64,10 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 }
 
 // ---------------------------------------------------------------- cp.async
-// 16-byte global -> shared copy that bypasses L1; completes with the
-// executing thread's commit groups.
+// 16-byte global -> shared copy that bypasses L1.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() {
-  asm volatile("cp.async.commit_group;" ::: "memory");
-}
-// Waits until at most N of this thread's commit groups are still pending.
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 // Arrives once on `bar` (counted in its expected arrivals) when this thread's copies so
 // far have landed.
 __device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
