@@ -89,8 +89,8 @@ SCORE_SRC = os.path.join("paper_2605_31105_gb300", "csrc", "grkv_score_tc.cu")
 # the ncu capture in profiles/score_tc_c2_llama_32k.md, keyed by the SHA-256 of the
 # kernel source it was taken on.
 SCORE_TRAFFIC = {
-    "c2_llama_32k_bf16": ("a99f3a36b4b67c9c0fe41fa9c256432bdf02ec59c39be001fd499e5086dba2dc",
-                          6543142912),
+    "c2_llama_32k_bf16": ("18b49fe4ab48399db5d99a87d125dfb61fd49fed945ed11a0becca0646f150b0",
+                          6538969088),
 }
 
 

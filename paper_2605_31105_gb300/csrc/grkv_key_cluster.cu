@@ -17,10 +17,10 @@
 // owners; p . Ap; ||r||^2; p's slices and rho1 to everyone.  Every rank adds in rank
 // order, so all hold the same scalars and take the same branches.
 //
-// Bound by latency: three dependent products and five exchanges an iteration,
-// about 3 K cycles of tensor-core time in 11 K.  The split through global memory
-// that this replaces staged every operand in each iteration and met at two
-// global barriers: 95 us an iteration for B = 512.
+// Bound by latency: three dependent products and five exchanges an iteration, 37 K cycles
+// (17.7 us; 8 units of m = 128, B = 512), the tensor pipe busy in 13% of them.  The split
+// through global memory that this replaces staged every operand in each iteration and met
+// at two global barriers: 95 us an iteration.
 #include <cmath>
 #include <type_traits>
 

@@ -111,9 +111,12 @@ __device__ __forceinline__ uint32_t xt_col(int kk, int lo) {
 
 // The wait for copies or MMAs in flight at the end of a CTA: bounded, whether or not another
 // wait has given up.
-__device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity) {
+__device__ __noinline__ void mbar_drain_wait(uint64_t* bar, uint32_t parity) {
   volatile int no_abort = 0;
   mbar_wait(bar, parity, &no_abort, kBudget);
+}
+__device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity) {
+  if (!mbar_try_wait(bar, parity)) mbar_drain_wait(bar, parity);
 }
 // mbar_wait for all lanes of a warp with one answer, so that warp-collective
 // instructions after a wait are reached by all lanes or by none.
@@ -458,10 +461,8 @@ __global__ void __launch_bounds__(kThreadsG, 1)
   const int B = ur.B, T = (B + kTile - 1) / kTile;
   // A unit is split as launch_gram splits a call at its own budget, so that its sums, and
   // with them its results' last bits, do not follow the largest budget of the call.
-  int split = C;
-  while (split > T) split /= 2;
-  const int ta = rank < split ? T * rank / split : T;      // this rank's tiles
-  const int tb = rank < split ? T * (rank + 1) / split : T;
+  const int lg = min(31 - __clz(C), 31 - __clz(T));        // 2^lg ranks hold tiles
+  const int ta = min(T, (T * rank) >> lg), tb = min(T, (T * (rank + 1)) >> lg);   // this rank's
   const int ng = __ldg(a.ng + u);
   if (tid == 0) {
     for (int i = 0; i < kRingG; ++i) {
@@ -941,7 +942,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // packed bf16 (rows 32c .. 32c+31 of chunk c: high parts to columns 32c ..
 // 32c+15, low parts to 32c+16 .. 32c+31, each chunk read before it is
 // overwritten); warps 12-15 the epilogue (thread = token): V_out = V0 + dV in
-// the V0 tile, which warp 0 then stores.  A fixed slot has X = 0 and so
+// the V0 tile, which warp 22 then stores.  A fixed slot has X = 0 and so
 // dV = 0: its row is left as V0.
 struct UBars {
   uint64_t k_full[2], k_empty[2], v_full[2], v_empty[2];

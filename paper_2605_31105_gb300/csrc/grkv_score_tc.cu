@@ -624,8 +624,9 @@ __global__ void __launch_bounds__(score_threads(kPass, RB), 1)
           lam[0] = lam_s[lb * kRows + row];
           mbar_arrive_warp(&bars->lam_empty[lb], lane);
         } else {
-          // Each group combines a quarter of the unit's slots.  A segment's jobs pass
-          // through s_done of every warp, so no warp still reads the last shares.
+          // Each group combines a quarter of the unit's slots.  No warp still reads the last
+          // segment's shares: this warp has waited for that segment's y_full, which follows Y MMAs
+          // that waited for p_full of every warp, and a warp arrives there after it has read them.
           const int ns = sc.nslots(it.u), c0 = sc.first_cta(it.u);
           const bool dense = sc.tiles() >= sc.G;   // every CTA holds tiles
           float2 st[RB];

@@ -16,9 +16,11 @@ namespace {
 // Both passes form S = Q K^T in tiles of MR window rows x 64 keys: 256 threads
 // as 16 x 16, thread (ty, tx) rows ty MR/16 .. and keys tx, tx + 16, ...  The
 // operands stay [row][t] in shared memory with rows of 132 floats, read four t
-// at a time: with MR = 128, 12 16-byte loads feed 128 FMAs and the tile is
-// bound by the FMAs (one load per FMA, one output per thread and 64-key
-// chunks cut into 512 CTAs took 355 + 603 us for 8 units of n = 8192, m = 128).
+// at a time: with MR = 128, 12 16-byte loads feed 128 FMAs.  Bound by a tile's phases
+// (load, products, exponentials, P) between block barriers, with two warps per scheduler to
+// cover them: 8 units of n = 8192, m = 128 take 88 + 156 us, the FMA pipe busy in 38% and 41%
+// of the cycles (one load per FMA, one output per thread and 64-key chunks cut into 512 CTAs
+// took 355 + 603).
 constexpr int kKeys = 64;        // keys per tile
 constexpr int kSLD = kD + 4;     // row stride of staged operands
 constexpr int kScT = 256;

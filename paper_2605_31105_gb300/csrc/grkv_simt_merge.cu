@@ -357,7 +357,8 @@ constexpr size_t kCholSmem = (size_t)(128 * kCLD + 4 * 32 * kBLD + 2 * 128) * si
 // diagonal blocks are inverted, one warp each.  Writes L's blocks below the
 // diagonal and the inverted diagonal blocks over N.  A pivot below 2^-20 of
 // its diagonal entry or below 2^-60, where pairs of floats leave too few
-// digits, sends the unit to fp64.
+// digits, sends the unit to fp64.  Bound by the chain of columns, two block barriers, a root and
+// a division each: 8 units of m = 128 take 114 us, one of m = 32 29 us.
 __global__ void __launch_bounds__(kChT, 1) k_simt_chol(SArgs a, Df* __restrict__ gram) {
   chain_wait();
   extern __shared__ __align__(16) float sm[];
