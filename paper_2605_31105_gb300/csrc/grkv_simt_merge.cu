@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(kChT, 1) k_simt_chol(SArgs a, Df* __restrict__
 // Z = L^-T L^-1 R by 32-row blocks, 8 columns per CTA; thread (row, column).
 // The factor's blocks are all staged first.
 constexpr size_t kSubstSmem =
-    (size_t)(10 * 32 * kBLD + 128 * 9 + 32 * 9) * sizeof(Df) + 8 * sizeof(uint32_t);
+    (size_t)(10 * 32 * kBLD + 128 * 9 + 32 * 9) * sizeof(Df) + 256;
 
 __global__ void __launch_bounds__(256) k_simt_subst(SArgs a, const Df* __restrict__ gram,
                                                     Df* __restrict__ rz) {
@@ -443,12 +443,10 @@ __global__ void __launch_bounds__(256) k_simt_subst(SArgs a, const Df* __restric
   Df* Lb = (Df*)sm;                     // block (i, j), j <= i, at i (i + 1) / 2 + j
   Df* W = Lb + 10 * 32 * kBLD;          // [128][9]
   Df* tmp = W + 128 * 9;                // [32][9]
-  uint32_t* seen = (uint32_t*)(tmp + 32 * 9);   // [8] of a column's residuals: 1 nonzero, 2 not small
+  uint8_t* seen = (uint8_t*)(tmp + 32 * 9);   // [32][8] of a thread's residuals: 1 nonzero, 2 not small
   const int u = blockIdx.x / (kD / 8), tid = threadIdx.x, r = tid >> 3, c = tid & 7;
   const int m = a.s.m, nb = (m + 31) / 32;
-  if (tid < 8) seen[tid] = 0;
-  // another CTA of the unit may give it to fp64 meanwhile: one answer for the block
-  if (__syncthreads_or(a.state[u] != kSolved)) return;
+  const int state = a.state[u];
   const Df* G = gram + (size_t)u * m * m;
   Df* Z = rz + (size_t)u * m * kD + blockIdx.x % (kD / 8) * 8;
   for (int i = tid >> 5; i < nb * 32; i += 8)
@@ -458,16 +456,21 @@ __global__ void __launch_bounds__(256) k_simt_subst(SArgs a, const Df* __restric
       Lb[((bi * (bi + 1) / 2 + bj) * 32 + i % 32) * kBLD + j % 32] =
           (i < m && j < m) ? G[(size_t)i * m + j] : pad;
     }
-  uint32_t size = 0;
+  int size = 0;
   for (int b = 0; b < nb; ++b) {
     const int i = b * 32 + r;
     const Df x = i < m ? Z[(size_t)i * kD + c] : Df{0.f, 0.f};
     W[i * 9 + c] = x;
-    size |= (x.hi != 0.f ? 1u : 0u) | (fabsf(x.hi) >= kSmall ? 2u : 0u);
+    size |= (x.hi != 0.f ? 1 : 0) | (fabsf(x.hi) >= kSmall ? 2 : 0);
   }
-  atomicOr(&seen[c], size);
-  __syncthreads();
-  bool fits = seen[c] != 1u;
+  seen[tid] = (uint8_t)size;
+  // another CTA of the unit may have given it to fp64 between two reads: one answer for the block
+  if (__syncthreads_or(state != kSolved)) return;
+  bool fits = true;
+  if (tid < 8) {
+    for (int e = tid; e < 256; e += 8) size |= seen[e];
+    fits = size != 1;
+  }
   auto solve_block = [&](int b, Df acc, bool back) {
     tmp[r * 9 + c] = df_norm(acc);
     __syncthreads();

@@ -37,7 +37,6 @@ static float __fadd_rn(float a, float b) { return a + b; }
 static float __fsub_rn(float a, float b) { return a - b; }
 static float __fmul_rn(float a, float b) { return a * b; }
 static float __fmaf_rn(float a, float b, float c) { return fmaf(a, b, c); }
-static uint32_t atomicOr(uint32_t* p, uint32_t v) { const uint32_t old = *p; *p |= v; return old; }
 static void chain_wait() {}
 
 struct Fiber { ucontext_t ctx; std::vector<char> stack; bool done; int pred; };
