@@ -19,7 +19,6 @@ import json
 import math
 import multiprocessing as mp
 import os
-import select
 import statistics
 import subprocess
 import sys
@@ -241,9 +240,7 @@ class ClockSampler:
                 ["nvidia-smi", "-i", self.gpu_id, f"--query-gpu={self.FIELDS}",
                  "--format=csv,noheader,nounits", "-lms", "20"],
                 stdout=subprocess.PIPE, stderr=subprocess.DEVNULL, text=True)
-            # The sampler's start holds up launches of this process; its first line ends it.
-            if select.select([self.proc.stdout], [], [], 5.0)[0]:
-                self.proc.stdout.readline()
+            time.sleep(0.5)
         except Exception:
             self.proc = None
 
