@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(256) k_merge_fixed(MArgs a) {
 // Measured, against one CTA per unit and block, two 128-thread groups on alternate
 // tiles, and a second launch for units that start over: 8 units B = 512 44 -> 15 us,
 // 64 units with budgets 200 .. 1536 88 -> 26 us, 32 units B = 1024 m = 256 103 -> 22 us,
-// 256 units B = 2048 129 -> 99 us (two waves), 88 with the asynchronous gathers.
+// 256 units B = 2048 129 -> 99 us (two waves), 84 with the asynchronous gathers.
 struct GBars {
   uint64_t ring_full[kRingG], ring_empty[kRingG];
   uint64_t q_full;
