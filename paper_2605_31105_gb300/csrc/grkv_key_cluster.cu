@@ -230,6 +230,32 @@ __global__ void __launch_bounds__(kThr, 1) k_key_cluster(KeyClusterArgs a) {
         }
     mma_commit(&x.mma);
   };
+  // The once-per-unit products, as exact as fp32 multiply-add chains: parts of combined order
+  // <= 3, the leading one alone in the first accumulator (low = 0), the others in the second.
+  // With one accumulator for the six parts of order <= 2 the update's error after one iteration
+  // (fp32 inputs, of |K* - K0|) is 1.4 to 3.0e-5, with two 0.2 to 0.5e-5, in plain fp32 0.7 to
+  // 1.4e-5: the residual Y - X V* is a small difference.  2 us more a call for 8 units.
+  auto products2 = [&](int pa_n, int pb_n, auto issue) {
+    uint32_t acc = 0;
+    for (int pa = 0; pa < pa_n; ++pa)
+      for (int pb = 0; pb < pb_n; ++pb) {
+        if (pa + pb > 3) continue;
+        const int low = pa + pb > 0;
+        issue(pa, pb, low, low ? acc : 0u);
+        acc |= low;
+      }
+    mma_commit(&x.mma);
+  };
+  // the sum of two accumulators' 32 columns
+  auto load2 = [&](uint32_t col, uint32_t col_low, float* v) {
+    float l[32];
+    tmem_ld32f(lane_tm + col_low, l);
+    tmem_ld32f(lane_tm + col, v);
+    tmem_wait32(l);
+    tmem_wait32(v);
+#pragma unroll
+    for (int e = 0; e < 32; ++e) v[e] += l[e];
+  };
   auto split_store_tmem = [&](const float* v, uint32_t col, uint32_t part_cols) {   // 32 values
     uint32_t w[3][16];
 #pragma unroll
@@ -275,14 +301,20 @@ __global__ void __launch_bounds__(kThr, 1) k_key_cluster(KeyClusterArgs a) {
     if (tid == 0) mbar_expect_tx(bar, kC * 128 * 4);
   };
   auto sum2 = [](float p, float r) { return p + r; };
-  // the rows' partial product (64 columns of kColO per thread) to the slices' owners
-  auto send_out = [&]() {
+  // the rows' partial product (64 columns of kColO per thread; two: its second accumulator
+  // in kColP) to the slices' owners
+  auto send_out = [&](auto two) {
     const uint32_t at = smem_u32(dbuf), b = smem_u32(&x.ex_out);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       float v[32];
-      tmem_ld32f(lane_tm + kColO + 64 * half + 32 * h, v);
-      tmem_wait32(v);
+      const uint32_t c = 64 * half + 32 * h;
+      if constexpr (decltype(two)::value) {
+        load2(kColO + c, kColP + c, v);
+      } else {
+        tmem_ld32f(lane_tm + kColO + c, v);
+        tmem_wait32(v);
+      }
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         const int col4 = 16 * half + 8 * h + e, owner = col4 / (kW / 4), ch = col4 % (kW / 4);
@@ -313,28 +345,32 @@ __global__ void __launch_bounds__(kThr, 1) k_key_cluster(KeyClusterArgs a) {
 
   // ---- S = Q K0^T and Q Q^T
   if (tid == 0) {
-    products(kParts, kParts, [&](int pa, int pb, uint32_t acc) {
+    products2(kParts, kParts, [&](int pa, int pb, int low, uint32_t acc) {
 #pragma unroll
       for (int kk = 0; kk < 8; ++kk)
-        mma_bf16(tm + kColT, sw128_desc(gqa + pa * kQPart + (kk >> 2) * (kQPart / 2) + (kk & 3) * 32, 16, 1024),
+        mma_bf16(tm + kColT + 64 * low, sw128_desc(gqa + pa * kQPart + (kk >> 2) * (kQPart / 2) + (kk & 3) * 32, 16, 1024),
                  sw128_desc(vta + pb * kVPart + (kk >> 2) * (kVPart / 2) + (kk & 3) * 32, 16, 1024),
                  idesc_bf16(128, nn, 0, 0), acc | (kk > 0));
     });
   }
   live = __syncthreads_and(mma_done()) && live;
   if (tid == 0) {
-    products(kParts, kParts, [&](int pa, int pb, uint32_t acc) {
+    products2(kParts, kParts, [&](int pa, int pb, int low, uint32_t acc) {
 #pragma unroll
       for (int kk = 0; kk < 8; ++kk)
-        mma_bf16(tm + kColP, sw128_desc(gqa + pa * kQPart + (kk >> 2) * (kQPart / 2) + (kk & 3) * 32, 16, 1024),
+        mma_bf16(tm + kColP + 128 * low, sw128_desc(gqa + pa * kQPart + (kk >> 2) * (kQPart / 2) + (kk & 3) * 32, 16, 1024),
                  sw128_desc(gqa + pb * kQPart + (kk >> 2) * (kQPart / 2) + (kk & 3) * 32, 16, 1024),
                  idesc_bf16(128, 128, 0, 0), acc | (kk > 0));
     });
   }
   float X[32];
   uint32_t vis = 0, fixed = 0;   // bit e: column 32 half + e
-  tmem_ld32f(lane_tm + kColT + 32 * half, X);
-  tmem_wait32(X);
+  if constexpr (kParts > 1) {
+    load2(kColT + 32 * half, kColT + 64 + 32 * half, X);
+  } else {
+    tmem_ld32f(lane_tm + kColT + 32 * half, X);
+    tmem_wait32(X);
+  }
   {
     const int lim = a.causal ? a.n - a.w + row % a.w : a.n - 1;
     const int32_t* idx = a.idx + (size_t)u * B + c0;
@@ -372,8 +408,13 @@ __global__ void __launch_bounds__(kThr, 1) k_key_cluster(KeyClusterArgs a) {
 #pragma unroll 1
   for (int h = 0; h < 2; ++h) {
     float v[32];
-    tmem_ld32f(lane_tm + kColP + 64 * half + 32 * h, v);
-    tmem_wait32(v);
+    const uint32_t c = 64 * half + 32 * h;
+    if constexpr (kParts > 1) {
+      load2(kColP + c, kColP + 128 + c, v);
+    } else {
+      tmem_ld32f(lane_tm + kColP + c, v);
+      tmem_wait32(v);
+    }
     const float s2 = a.scale * a.scale;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -396,15 +437,21 @@ __global__ void __launch_bounds__(kThr, 1) k_key_cluster(KeyClusterArgs a) {
   for (int e = 0; e < 32; ++e) X[e] *= inv;
 
   // ---- products of the CG
-  auto out_product = [&]() {   // (parts at kColX) V*
-    if (tid == 0)
-      products(3, kParts, [&](int pa, int pb, uint32_t acc) {
-        for (int kk = 0; kk < nn / 16; ++kk)
-          mma_bf16_ts(tm + kColO, tm + kColX + pa * 32 + kk * 8,
-                      sw128_desc(vta + pb * kVPart + kk * 2048, kVPart / 2, 1024),
-                      idesc_bf16(128, 128, 0, 1), acc | (kk > 0));
-      });
+  auto issue_out = [&](uint32_t col, int pa, int pb, uint32_t acc) {   // (parts at kColX) V*
+    for (int kk = 0; kk < nn / 16; ++kk)
+      mma_bf16_ts(tm + col, tm + kColX + pa * 32 + kk * 8,
+                  sw128_desc(vta + pb * kVPart + kk * 2048, kVPart / 2, 1024),
+                  idesc_bf16(128, 128, 0, 1), acc | (kk > 0));
   };
+  auto out_product = [&]() {
+    if (tid == 0)
+      products(3, kParts, [&](int pa, int pb, uint32_t acc) { issue_out(kColO, pa, pb, acc); });
+  };
+  if (kParts > 1) {   // Q Q^T's second accumulator has been read by all: X's parts overlap it
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+  }
   split_store_tmem(X, kColX + 16 * half, 32);
   tmem_st_wait();
   fence_proxy_async_smem();
@@ -413,10 +460,15 @@ __global__ void __launch_bounds__(kThr, 1) k_key_cluster(KeyClusterArgs a) {
   for (int e = 0; e < kH; ++e) xv[e] = r[e] = p[e] = al[e] = 0.f;
   float rs = 0.f, stop = 0.f;
   if (ready(ok)) {
-    out_product();
+    if (tid == 0)
+      products2(3, kParts, [&](int pa, int pb, int low, uint32_t acc) {
+        issue_out(low ? kColP : kColO, pa, pb, acc);
+      });
     ok = mma_done();
-    send_out();
+    send_out(std::true_type());
+    tc_fence_before();
     live = __syncthreads_and(wait(&x.ex_out, ph_out) && ok) && live;
+    tc_fence_after();   // the second accumulator's columns take p next
     recv_out(xv);
     const float* y = a.y + ((size_t)u * m + min(row, m - 1)) * kD + rank * kW + half * kH;
 #pragma unroll
@@ -540,7 +592,7 @@ __global__ void __launch_bounds__(kThr, 1) k_key_cluster(KeyClusterArgs a) {
     if (!ready(ok)) break;
     out_product();
     ok = mma_done();
-    send_out();
+    send_out(std::false_type());
     live = __syncthreads_and(wait(&x.ex_out, ph_out) && ok) && live;
     float ap[kH], pap = 0.f;
     recv_out(ap);
@@ -574,17 +626,16 @@ __global__ void __launch_bounds__(kThr, 1) k_key_cluster(KeyClusterArgs a) {
     stage_ds();
     if (ready(ok)) {
       if (tid == 0)
-        products(kParts, 3, [&](int pa, int pb, uint32_t acc) {
+        products2(kParts, 3, [&](int pa, int pb, int low, uint32_t acc) {
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)
-            mma_bf16(tm + kColT, sw128_desc(gqa + pa * kQPart + kk * 2048, kQPart / 2, 1024),
+            mma_bf16(tm + kColT + 64 * low, sw128_desc(gqa + pa * kQPart + kk * 2048, kQPart / 2, 1024),
                      sw128_desc(dta + pb * kSPart + kk * 2048, kSPart, 1024),
                      idesc_bf16(128, nn, 1, 1), acc | (kk > 0));
         });
       live = __syncthreads_and(mma_done()) && live;
       float dk[32];
-      tmem_ld32f(lane_tm + kColT + 32 * half, dk);
-      tmem_wait32(dk);
+      load2(kColT + 32 * half, kColT + 64 + 32 * half, dk);
       const int d = row;
       if (live)
 #pragma unroll
